@@ -54,7 +54,8 @@ extern "C" {
 #define RICI_MAX_RESOLUTION 128
 
 /* Generation modes (rici_generate_ex). */
-#define RICI_GEN_DEFAULT 0   /* FP32 arithmetic; predicates inside the error band redone in FP64 */
+#define RICI_GEN_DEFAULT 0   /* FP32 arithmetic; predicates inside the error band redone with pairs
+                                of floats, and in FP64 where those do not decide */
 #define RICI_GEN_FP64 1      /* every (triangle, layer) evaluated in FP64 (slow reference mode) */
 
 /* Search modes (crss_search). */
@@ -118,7 +119,7 @@ RICI_API int rici_generate(const float *vertices, const float *normals, int64_t 
  * counters (NULL or device int64[4]) receives, added to its contents:
  *   [0] (origin, triangle) pairs fully processed after culling,
  *   [1] (origin, triangle, layer) items processed,
- *   [2] items re-evaluated in FP64 because a predicate fell inside the FP32 error band,
+ *   [2] items re-evaluated (float pairs, FP64) because a predicate fell inside the FP32 error band,
  *   [3] candidate (origin, triangle) pairs tested one by one by the spatial cull (those in
  *       32-triangle chunks whose bounding spheres passed). */
 RICI_API int rici_generate_ex(const float *vertices, const float *normals, int64_t num_vertices,

@@ -22,11 +22,12 @@
 // The clutter measure and spin images (bottom of this file) bin triangles into a hashed uniform
 // grid instead and scan the grid cells around each oriented point.
 //
-// Exactness: the FP32 path carries a forward error bound for every predicate (vertex side
-// of a layer, |E|^2 against alpha^2, the signs of E0.D and E1.D, alpha^2 |D|^2 against
-// (E0 x D)^2).  A (triangle, layer) whose predicate lies inside its bound is recomputed in
-// FP64 with the definition's operation order (explicit _rn intrinsics, no contraction), so
-// every count equals the FP64 definition bit for bit.
+// Exactness: the FP32 path carries a forward error bound for every predicate (vertex side of a
+// layer, |E| against alpha, the signs of E0.D and E1.D, the distance of the chord's closest point).
+// A (triangle, layer) whose predicate lies inside its bound is evaluated again with pairs of floats
+// (48 bits, their own bounds), and where those do not decide either in FP64 with the definition's
+// operation order (explicit _rn intrinsics, no contraction), so every count equals the FP64
+// definition bit for bit.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -40,13 +41,15 @@ constexpr float kU = 5.9604644775390625e-08f;  // 2^-24: unit roundoff of FP32
 constexpr float kSafety = 2.0f;                // multiplies every derived error bound
 constexpr uint32_t kSkip = 0xFFFFFFFEu;
 constexpr float kCellClamp = 1048576.0f;  // |cell coordinate| limit (2^20)
-constexpr int kSlot = 21;  // words per staged triangle (odd stride: conflict-free lookups)
+constexpr int kSlot = 20;  // words per staged triangle (a multiple of 4 whose first 8 multiples
+                           // lie in 8 different groups of 4 banks: conflict-free 16-byte loads)
 constexpr int kScanItems = kGenScanItems;
 constexpr int kGenMaxCellsPerReach = 4;      // generation: up to (2 x 4 + 1)^3 cells per point
 constexpr int kClutterMaxCellsPerReach = 3;  // clutter measure and spin images: up to 7^3
-// shared words per warp: candidate queue, FP64 queue (triangle records, then their layers as
-// bytes), staged triangles
-constexpr int kPerWarp = 64 + 64 + 16 + 32 * kSlot;
+constexpr int kBandQ = 128;  // band queue of a warp: 31 left over + 3 layers of each of 32 triangles
+// shared words per warp: candidate queue, band queue (triangle records, then their layers as
+// bytes), place in the walk over groups, staged triangles; a multiple of 4
+constexpr int kPerWarp = 64 + kBandQ + kBandQ / 4 + 4 + 32 * kSlot;
 
 __host__ __device__ constexpr uint32_t bucket_count(int64_t nt) { return generate_bucket_count(nt); }
 
@@ -447,43 +450,49 @@ struct KArgs {
   int *status;
 };
 
+struct Pair;
 struct Shared {
-  int *diff;     // [N][N] difference image
+  int *diff;     // [N][N + 1] difference image (the last column takes interval ends at N; the odd
+                 // stride spreads equal columns of consecutive layers over the banks)
   double *a2d;   // alpha_c^2 (FP64 definition)
   double *bd;    // beta_r (FP64 definition)
-  float *a2f;    // alpha_c^2 rounded to FP32
-  float *bf;     // beta_r rounded to FP32
   double *fr;    // S (3 doubles), Nax, Nay, Nbx, Nbz
-  int *buckets;  // neighbour buckets ((2 nhalf + 1)^3 cells + the big list), then the first
-                 // candidate of each
-  int *bdup;     // 1: skip this entry (out of reach or repeated bucket), then the end of its
-                 // candidate range (= its first candidate for a skipped entry)
+  Pair *fp;      // the frame for layer_pairs (6 pairs)
+  float4 *ff;    // gax, gay, gbx, gbz; fax, fay, N / R; S and the sphere test's margin; the axis: read
+                 // where they are used, so that they hold no registers in between
   int *wq;       // this warp's candidate queue [64]
-  int *wst;      // this warp's item-owner marks for the current 32 items [32] (aliases the first
-                 // half of wq, which is free once a batch's triangles are staged)
-  int *bq_rec;   // this warp's FP64 queue: triangle record [64]
-  unsigned char *bq_r;  // this warp's FP64 queue: layer [64]
+  int *bq_rec;   // this warp's band queue: triangle record [kBandQ]
+  unsigned char *bq_r;  // this warp's band queue: layer [kBandQ]
+  int *walk;     // this warp's place in the walk over groups: next window, window and mask left in it
   float *slots;  // this warp's staged triangles [32][kSlot]
 };
 
-// slot layout (words)
+// A staged triangle, in units of R / N (one column, one layer), heights Z counted in layers (layer
+// r at Z = r), vertices sorted by height: 0 lowest, 1 middle, 2 highest.  Layers between 0 and 1
+// cross the edges 0-2 and 0-1, layers between 1 and 2 cross 0-2 and 1-2, so both crossed edges
+// start at vertex 0 for the former and at vertex 2 for the latter, and the crossing points are
+// E = (x, y) + (r - Z) (slope) with the slopes dx/dZ, dy/dZ of the two edges.
 enum {
-  SX = 0, SY = 3, SZ = 6, SGID = 9, SDE = 12,
-  SINV = 15,   // 1 / (z_j - z_i) of edge k (opposite vertex k, i < j local indices)
-  SMETA = 18,  // first layer (bits 0-7), side-band layer of each vertex (bits 8-15, 16-23,
-               // 24-31; kNoBand for none; kAllBand in bits 8-15: every layer goes to FP64)
-  SREC = 19
+  S_V0 = 0,     // x0, y0, Z0, column margin of the lower segment (see item margins below)
+  S_V2 = 4,     // x2, y2, Z2, column margin of the upper segment
+  S_LONG = 8,   // slope of edge 0-2, slope of edge 0-1
+  S_UP = 12,    // slope of edge 1-2, first item (int), layers (int: first layer of the lower
+                // segment, its layer count << 8, (first upper layer - that count) << 16)
+  S_REC = 16    // triangle record (int)
 };
-constexpr unsigned kNoBand = 0xFF, kAllBand = 0xFE;
 
-// Estimate of the number of columns c with alpha_c^2 <= x (alpha_c = R (2c+1) / 2N, so the count
-// is floor(N sqrt(x) / R + 1/2)), in [0, N].  Off by one at most, and only within a few ulps of a
-// column boundary: every caller then checks the margins to both neighbouring columns, a check that
-// fails (sends the item to FP64) whenever the estimate is not the exact count.
-__device__ __forceinline__ int count_estimate_f(float x, int N, float scale) {
-  const float s = x > 0.0f ? x * rsqrtf(x) * scale : 0.0f;
-  const float fc = floorf((s + 1.0f) * 0.5f);
-  return (fc >= (float)N) ? N : ((fc > 0.0f) ? (int)fc : 0);
+// Adding kRound to a float of magnitude below 2^22 rounds it to an integer, held in the low bits.
+constexpr float kRound = 12582912.0f;  // 1.5 * 2^23
+
+__device__ __forceinline__ float rsqrt_fast(float x) {  // relative error below 2^-22.9
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_fast(float x) {  // at most 1 ulp off
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 __device__ __forceinline__ int lower_count_d(double x, const double *a2d, int N) {
@@ -569,7 +578,7 @@ __device__ __forceinline__ void project64(float px, float py, float pz, const do
 // Returns false when the triangle does not cross the layer; otherwise the single-crossing
 // columns are [lo, hi) and the double-crossing columns [dlo, lo).
 // (Plain pointer arguments: no structure has to live in local memory.)
-__device__ __forceinline__ bool layer_fp64(const float4 *__restrict__ recs, int64_t rs,
+__device__ __noinline__ bool layer_fp64(const float4 *__restrict__ recs, int64_t rs,
                                         const double *fr, const double *bd, const double *a2d,
                                         int N, int rec, int r, int &lo, int &hi, int &dlo) {
   float4 r1 = recs[rs + rec], r2 = recs[2 * rs + rec], r3 = recs[3 * rs + rec];
@@ -622,105 +631,234 @@ __device__ __forceinline__ bool layer_fp64(const float4 *__restrict__ recs, int6
   return true;
 }
 
-// FP32 evaluation with forward error bounds against the FP64 definition.
-// Returns 0: no crossing, 1: intervals valid, 2: a predicate lies inside its error band
-// (the caller re-evaluates the item in FP64).
-__device__ __forceinline__ int layer_fp32(const float *__restrict__ bf, const float *__restrict__ a2f,
-                                          int N, const float *sl, int r, float scale, int &lo,
-                                          int &hi, int &dlo) {
-  const float beta = bf[r];
-  float tz0 = sl[SZ], tz1 = sl[SZ + 1], tz2 = sl[SZ + 2];
-  int s0 = tz0 >= beta, s1 = tz1 >= beta, s2 = tz2 >= beta;
-  if (s0 == s1 && s1 == s2) return 0;
-  int lone = (s0 != s1 && s0 != s2) ? 0 : ((s1 != s0 && s1 != s2) ? 1 : 2);
-  int oa = lone == 0 ? 1 : 0;
-  int ob = lone == 2 ? 1 : 2;
-  // slice the two crossed edges (lone, oa) and (lone, ob) in local vertex order: E lies within
-  // the per-edge bound of the FP64 point whatever the orientation, so the FP32 path only has to
-  // keep the roles of E0 and E1 (chosen by global vertex indices as in the definition)
-  const int g_l = __float_as_int(sl[SGID + lone]), g_a = __float_as_int(sl[SGID + oa]),
-            g_b = __float_as_int(sl[SGID + ob]);
-  const int ia = min(lone, oa), ja = max(lone, oa);  // edge opposite ob
-  const int ib = min(lone, ob), jb = max(lone, ob);  // edge opposite oa
-  const float la = __fmul_rn(__fsub_rn(beta, sl[SZ + ia]), sl[SINV + ob]);
-  const float lb = __fmul_rn(__fsub_rn(beta, sl[SZ + ib]), sl[SINV + oa]);
-  float Eax = __fmaf_rn(la, __fsub_rn(sl[SX + ja], sl[SX + ia]), sl[SX + ia]);
-  float Eay = __fmaf_rn(la, __fsub_rn(sl[SY + ja], sl[SY + ia]), sl[SY + ia]);
-  float Ebx = __fmaf_rn(lb, __fsub_rn(sl[SX + jb], sl[SX + ib]), sl[SX + ib]);
-  float Eby = __fmaf_rn(lb, __fsub_rn(sl[SY + jb], sl[SY + ib]), sl[SY + ib]);
-  // E0 is the crossed edge with the smaller (lower, higher) global index key
-  const int gua = min(g_l, g_a), gva = max(g_l, g_a);
-  const int gub = min(g_l, g_b), gvb = max(g_l, g_b);
-  bool swap = gub < gua || (gub == gua && gvb < gva);
-  float E0x = swap ? Ebx : Eax, E0y = swap ? Eby : Eay;
-  float E1x = swap ? Eax : Ebx, E1y = swap ? Eay : Eby;
-  // |E32 - E64| per component; edge (lone, oa) is opposite ob and vice versa
-  const float dE = fmaxf(sl[SDE + ob], sl[SDE + oa]);
-  if (!(dE < 1e30f)) return 2;
-  float e0 = __fmaf_rn(E0x, E0x, __fmul_rn(E0y, E0y));
-  float e1 = __fmaf_rn(E1x, E1x, __fmul_rn(E1y, E1y));
-  const float A0 = fabsf(E0x) + fabsf(E0y) + 2.0f * dE;  // bounds |E0x*| + |E0y*|
-  const float A1 = fabsf(E1x) + fabsf(E1y) + 2.0f * dE;
-  const float de0 = kSafety * (2.0f * A0 * dE + 3.01f * kU * e0) + 1e-37f;
-  const float de1 = kSafety * (2.0f * A1 * dE + 3.01f * kU * e1) + 1e-37f;
-  int c0 = count_estimate_f(e0, N, scale), c1 = count_estimate_f(e1, N, scale);
-  // the two columns around each transition must be decided with certainty (this also rejects a
-  // wrong estimate: one of the two differences is then <= 0)
-  if (c0 > 0 && e0 - a2f[c0 - 1] <= de0 + kU * a2f[c0 - 1]) return 2;
-  if (c0 < N && a2f[c0] - e0 <= de0 + kU * a2f[c0]) return 2;
-  if (c1 > 0 && e1 - a2f[c1 - 1] <= de1 + kU * a2f[c1 - 1]) return 2;
-  if (c1 < N && a2f[c1] - e1 <= de1 + kU * a2f[c1]) return 2;
+// Column count of a distance w from the axis (in columns, at most N + 1/4): alpha_c = c + 1/2, so
+// the columns with alpha_c <= w are [0, round(w)).  f is the distance to that integer: the count
+// is certain for an error of w below 1/2 - |f|.
+__device__ __forceinline__ int column_count(float w, float &f) {
+  const float m = __fadd_rn(w, kRound);
+  f = __fsub_rn(w, __fsub_rn(m, kRound));
+  return __float_as_int(m) - __float_as_int(kRound);
+}
+
+// Double crossings of one segment E0, E1 (in columns): the columns [dlo, lo) below lo, the count of
+// the nearer end, whose circles cross the segment twice because its closest point C to the axis
+// is strictly inside it (E0.D < 0 < E1.D) and nearer than they are.  v0, v1: |E0| and |E1|, w the
+// smaller, cut off at wmax = N + 1/4.  hd = 1/2 - delta with delta >= 2 x sqrt(2) dE (dE the error
+// of a point's component) + the rounding of a distance.  Returns false when the test lies inside
+// its error bound.
+__device__ __forceinline__ bool double_columns(float E0x, float E0y, float E1x, float E1y, float v0,
+                                               float v1, float w, float hd, float wmax, int lo,
+                                               int &dlo) {
+  dlo = lo;
+  // the products E.D are known to vm 2 sqrt(2) dE + L sqrt(2) dE + 4 dE^2 + 3 u vm L, vm the larger
+  // distance, L = |Dx| + |Dy|; tau is over twice that
+  const float Dx = __fsub_rn(E1x, E0x), Dy = __fsub_rn(E1y, E0y);
+  const float d0 = __fmaf_rn(E0x, Dx, __fmul_rn(E0y, Dy));
+  const float d1 = __fmaf_rn(E1x, Dx, __fmul_rn(E1y, Dy));
+  const float delta = 0.5f - hd;
+  const float vm = fmaxf(v0, v1), L = fabsf(Dx) + fabsf(Dy);
+  const float tau = __fmaf_rn(2.0f * delta, vm + L + 1.0f, 8.0f * kU * vm * L);
+  if (lo == 0 || d0 > tau || d1 < -tau) return true;
+  // C is inside, or may be.  Nothing happens if no column lies between the nearer end and C: C is at
+  // least sqrt(w^2 - (l/2)^2) away, l the segment's length, so the column boundary lo - 1/2 below
+  // w is out of reach when (w - delta)^2 - (lo - 1/2)^2 >= (l/2 + delta)^2, for which the test
+  // below is sufficient.
+  const float l2 = __fmaf_rn(Dx, Dx, __fmul_rn(Dy, Dy));
+  const float fd = w - ((float)lo - 0.5f);
+  if ((fd - delta) * w * 0.999f > 0.27f * l2 + 20.0f * delta * delta) return true;
+  // distance of C: both ends moved by at most sqrt(2) dE, plus the rounding of the cross product,
+  // the length and the root (l2 > 1e-30: the product is then no NaN that the minimum would hide)
+  const float cr = __fmaf_rn(E0x, Dy, -__fmul_rn(E0y, Dx));
+  float f;
+  const int ch = column_count(fminf(fabsf(cr) * rsqrt_fast(l2), wmax), f);
+  dlo = min(ch, lo);
+  return d0 < -tau && d1 > tau && l2 > 1e-30f && l2 < 1e30f && fabsf(f) < hd - 16.0f * kU * vm;
+}
+
+// FP32 evaluation of one (triangle, layer) from its two crossing points (in columns, frame origin on
+// the axis) with forward error bounds against the FP64 definition; hd as above.  Returns false when
+// a predicate lies inside its bound (or hd is not a positive number); otherwise the
+// single-crossing columns are [lo, hi) and the double-crossing columns [dlo, lo), each plus
+// kRoundBits.  E0 and E1 may be exchanged.
+constexpr int kRoundBits = 0x4B400000;  // the bits of kRound
+__device__ __forceinline__ bool layer_fp32(float E0x, float E0y, float E1x, float E1y, float hd,
+                                           float wmax, int &lo, int &hi, int &dlo) {
+  // e is kept off zero for the reciprocal root (columns start at 1/2)
+  const float e0 = __fmaf_rn(E0x, E0x, __fmaf_rn(E0y, E0y, 1e-30f));
+  const float e1 = __fmaf_rn(E1x, E1x, __fmaf_rn(E1y, E1y, 1e-30f));
+  const float v0 = __fmul_rn(e0, rsqrt_fast(e0)), v1 = __fmul_rn(e1, rsqrt_fast(e1));
+  const float w0 = fminf(v0, wmax), w1 = fminf(v1, wmax);
+  float f0, f1;
+  const int c0 = column_count(w0, f0) + kRoundBits, c1 = column_count(w1, f1) + kRoundBits;
   lo = min(c0, c1);
   hi = max(c0, c1);
   dlo = lo;
-  if (lo > 0) {
-    float Dx = __fsub_rn(E1x, E0x), Dy = __fsub_rn(E1y, E0y);
-    const float dD = 2.0f * dE + kU * (fabsf(Dx) + fabsf(Dy));
-    const float B = fabsf(Dx) + fabsf(Dy) + 2.0f * dD;  // bounds |Dx*| + |Dy*|
-    // is the line's closest point C strictly inside the segment (E0.D < 0 < E1.D)?
-    float d0 = __fmaf_rn(E0x, Dx, __fmul_rn(E0y, Dy));
-    float d1 = __fmaf_rn(E1x, Dx, __fmul_rn(E1y, Dy));
-    const float dd0 = kSafety * (A0 * dD + B * dE + 2.0f * kU * A0 * B) + 1e-37f;
-    const float dd1 = kSafety * (A1 * dD + B * dE + 2.0f * kU * A1 * B) + 1e-37f;
-    if (fabsf(d0) <= dd0 || fabsf(d1) <= dd1) return 2;
-    if (d0 < 0.0f && d1 > 0.0f) {
-      // alpha_c^2 |D|^2 > (E0 x D)^2  <=>  alpha_c^2 > h^2, h = |C| the segment's distance to
-      // the axis.  C is inside the segment for the FP32 and the FP64 endpoints, and moving
-      // each endpoint by at most dE per component moves h by at most sqrt(2) dE, so h^2 is
-      // known to 2 h dh + dh^2 plus the rounding of the cross product, |D|^2 and the quotient.
-      float cr = __fmaf_rn(E0x, Dy, -__fmul_rn(E0y, Dx));
-      float dd = __fmaf_rn(Dx, Dx, __fmul_rn(Dy, Dy));
-      if (!(dd >= 1e-30f && dd <= 1e30f)) return 2;  // keep the fast quotient in its range
-      // fast quotient (at most 2 ulp = 4 kU relative from the rounded operands) and fast root
-      // (used in the bound only, raised by 1e-6 relative to cover its own error)
-      float h2 = __fdividef(__fmul_rn(cr, cr), dd);
-      const float h = h2 > 0.0f ? h2 * rsqrtf(h2) * 1.000001f : 0.0f;
-      const float dh = 1.5f * (dE + kU * B);
-      const float rb = B * rsqrtf(dd);  // (|Dx| + |Dy| + 2 dD) / |D|
-      const float dq = kSafety * (2.0f * h * dh + 2.0f * dh * dh + 4.0f * kU * h * A0 * rb +
-                                  2.0f * kU * h2 * (1.0f + rb * rb) + 4.0f * kU * h2) + 1e-37f;
-      if (!(dq < 1e30f)) return 2;
-      const int cs = count_estimate_f(h2, N, scale);  // first column with alpha^2 > h^2
-      if (cs >= lo) {
-        if (h2 - a2f[lo - 1] <= dq + kU * a2f[lo - 1]) return 2;
-      } else {
-        if (cs > 0 && h2 - a2f[cs - 1] <= dq + kU * a2f[cs - 1]) return 2;
-        if (a2f[cs] - h2 <= dq + kU * a2f[cs]) return 2;
-        dlo = cs;
-      }
-    }
+  bool ok = fmaxf(fabsf(f0), fabsf(f1)) < hd;
+  // Most segments have their closest point to the axis at an end, which E0.D > 0 or E1.D < 0 tells:
+  // E0.E1 - |E0|^2 > 0 or E0.E1 - |E1|^2 > 0.  With both ends within vm < 4 N, |D| <= 2 vm and dE as
+  // above these are known to vm 2 sqrt(2) dE + 2 vm sqrt(2) dE + 4 dE^2 + 5 u vm^2 <= 2 delta vm +
+  // delta^2 + 20 u N vm; delta >= 12 u N and vm >= 1/2 (where lo > 0) make that below 5 delta vm.
+  const float vm = fmaxf(v0, v1);
+  const float out = __fmaf_rn(E0x, E1x, __fmul_rn(E0y, E1y)) - fminf(e0, e1);
+  const bool ends = out > vm * __fmaf_rn(-10.0f, hd, 5.0f) && vm < 4.0f * wmax - 1.0f;
+  if (!ends && lo > kRoundBits) {
+    ok = double_columns(E0x, E0y, E1x, E1y, v0, v1, fminf(w0, w1), hd, wmax, lo - kRoundBits, dlo) &&
+         ok;
+    dlo += kRoundBits;
   }
-  return 1;
+  return ok;
 }
 
-__device__ __forceinline__ void add_intervals(int *row, int N, int lo, int hi, int dlo) {
+// ---- pairs of floats: h + l with |l| <= u |h|.  Each operation's error is below kUU times the sum
+// of its operands' (a product's: its own) magnitudes.
+struct Pair {
+  float h, l;
+};
+constexpr float kUU = 5.6843418860808015e-14f;  // 2^-44 = 16 u^2
+
+__device__ __forceinline__ Pair pair_norm(float s, float e) {  // |s| >= |e|
+  const float h = __fadd_rn(s, e);
+  return Pair{h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ Pair two_sum(float a, float b) {  // exact (Knuth)
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return Pair{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ Pair operator-(Pair a) { return Pair{-a.h, -a.l}; }
+__device__ __forceinline__ Pair operator+(Pair a, Pair b) {
+  const Pair s = two_sum(a.h, b.h);
+  return pair_norm(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ Pair operator-(Pair a, Pair b) { return a + (-b); }
+__device__ __forceinline__ Pair operator*(Pair a, Pair b) {
+  const float p = __fmul_rn(a.h, b.h);
+  const float e = __fmaf_rn(a.h, b.h, -p);  // exact
+  return pair_norm(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, e)));
+}
+__device__ __forceinline__ Pair operator/(Pair n, Pair d) {
+  const float rc = rcp_fast(d.h), q = __fmul_rn(n.h, rc);
+  const float r = __fadd_rn(__fmaf_rn(-q, d.h, n.h), __fmaf_rn(-q, d.l, n.l));
+  return pair_norm(q, __fmul_rn(r, rc));
+}
+__device__ __forceinline__ Pair to_pair(double x) {
+  const float h = __double2float_rn(x);
+  return Pair{h, __double2float_rn(x - (double)h)};
+}
+
+// Evaluation of one (triangle, layer) with pairs of floats, by the steps of the FP32 path with kUU
+// in the place of u.  fp: Nax, Nay, then Nax, Nay, Nbx, Nbz scaled by perd = N / R, as pairs.
+// Returns 0: no crossing, 1: intervals valid, 2: a predicate lies inside its error bound.
+// Band items that would take about 110 FP64 operations at 1/64 of the FP32 rate take about 600 FP32
+// operations here, and about one in 10^4 of them is left to FP64.
+__device__ __forceinline__ int layer_pairs(const float4 *__restrict__ recs, int64_t rs,
+                                           const float *S, const Pair *fp, float perd, int N,
+                                           int rec, int r, int &lo, int &hi, int &dlo) {
+  const float4 r1 = recs[rs + rec], r2 = recs[2 * rs + rec], r3 = recs[3 * rs + rec];
+  const float P[9] = {r1.x, r1.y, r1.z, r1.w, r2.x, r2.y, r2.z, r2.w, r3.x};
+  Pair X[3], Y[3], H[3];  // H: height above the layer
+  float M = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const Pair dx = two_sum(P[3 * k], -S[0]), dy = two_sum(P[3 * k + 1], -S[1]),
+               dz = two_sum(P[3 * k + 2], -S[2]);
+    const Pair qx = fp[0] * dx + fp[1] * dy;
+    X[k] = fp[5] * qx - fp[4] * dz;
+    Y[k] = fp[2] * dy - fp[3] * dx;
+    H[k] = (fp[4] * qx + fp[5] * dz) + Pair{0.5f * (float)(N - 1) - (float)r, 0.0f};
+    M = fmaxf(M, fabsf(dx.h) + fabsf(dy.h) + fabsf(dz.h));
+  }
+  const float dT = 10.1f * kUU * M * perd + 2.0f * kUU * (float)N + 1e-37f;
+  const float dside = kSafety * (dT + kUU * (float)N);
+  if (!(fminf(fminf(fabsf(H[0].h), fabsf(H[1].h)), fabsf(H[2].h)) > dside)) return 2;
+  const bool s0 = H[0].h > 0.0f, s1 = H[1].h > 0.0f, s2 = H[2].h > 0.0f;
+  if (s0 == s1 && s1 == s2) return 0;
+  // the vertex alone on its side to place 0
+  const bool m1 = s1 != s0 && s1 != s2, m2 = s2 != s0 && s2 != s1;
+  auto to_front = [](bool b, Pair &p, Pair &q) {
+    const Pair t = p;
+    p.h = b ? q.h : p.h;
+    p.l = b ? q.l : p.l;
+    q.h = b ? t.h : q.h;
+    q.l = b ? t.l : q.l;
+  };
+  to_front(m1, X[0], X[1]);
+  to_front(m1, Y[0], Y[1]);
+  to_front(m1, H[0], H[1]);
+  to_front(m2, X[0], X[2]);
+  to_front(m2, Y[0], Y[2]);
+  to_front(m2, H[0], H[2]);
+  float mag = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) mag = fmaxf(mag, fmaxf(fabsf(X[k].h), fabsf(Y[k].h)));
+  Pair Ex[2], Ey[2];
+  float v[2], w[2], dE = 0.0f, magE = 0.0f;
+  int c[2];
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const Pair den = H[k + 1] - H[0], dx = X[k + 1] - X[0], dy = Y[k + 1] - Y[0];
+    const float ad = fabsf(den.h), ext = fmaxf(fabsf(dx.h), fabsf(dy.h));
+    ok = ok && ad > 40.0f * dT;
+    const Pair lam = -H[0] / den;
+    Ex[k] = X[0] + lam * dx;
+    Ey[k] = Y[0] + lam * dy;
+    const float el = 3.3f * dT * rcp_fast(ad) + 7.0f * kUU;
+    const float de = 1.1f * (3.0f * dT + 4.0f * kUU * (ext + mag) + (ext + 2.0f * dT) * el);
+    dE = fmaxf(dE, de);
+    const Pair e = Ex[k] * Ex[k] + Ey[k] * Ey[k];
+    const float A = fabsf(Ex[k].h) + fabsf(Ey[k].h) + 2.0f * de;
+    const float dd = kSafety * (2.0f * A * de + 8.0f * kUU * e.h) + 1e-37f;
+    const float eh = fmaxf(e.h, 1e-30f);
+    v[k] = __fmul_rn(eh, rsqrt_fast(eh));
+    w[k] = fminf(v[k], (float)N + 0.25f);
+    float f;
+    c[k] = column_count(w[k], f);
+    // alpha^2 of the columns on either side of the count (exact): a wrong count fails one of the two
+    const float b0 = (float)c[k] - 0.5f, b1 = (float)c[k] + 0.5f;
+    ok = ok && (c[k] == 0 || __fadd_rn(__fsub_rn(e.h, __fmul_rn(b0, b0)), e.l) > dd) &&
+         (c[k] >= N || __fsub_rn(__fsub_rn(__fmul_rn(b1, b1), e.h), e.l) > dd);
+    magE = fmaxf(magE, fmaxf(fabsf(Ex[k].h), fabsf(Ey[k].h)));
+  }
+  if (!ok) return 2;
+  lo = min(c[0], c[1]);
+  hi = max(c[0], c[1]);
+  // the double crossings decide on coarser predicates, for which the points' leading parts do
+  const float hd = 0.5f - (kSafety * 1.4143f * (dE + kU * magE) + 12.0f * kU * (float)(N + 1));
+  return double_columns(Ex[0].h, Ey[0].h, Ex[1].h, Ey[1].h, v[0], v[1], fminf(w[0], w[1]), hd,
+                        (float)N + 0.25f, lo, dlo)
+             ? 1
+             : 2;
+}
+
+// One (triangle, layer) that FP32 could not decide, or every one of the reference mode: pairs of
+// floats, then the FP64 definition.  Bits 0-7: 1 when the triangle crosses the layer; then lo, hi,
+// dlo (at most 128).  Called, not inlined: few warps are in here at a time, and the batch code
+// stays small.
+__device__ __noinline__ unsigned band_item(const float4 *__restrict__ recs, int64_t rs,
+                                           const double *fr, const Pair *fp, const double *bd,
+                                           const double *a2d, float perd, int N, bool fp64_only,
+                                           int rec, int r) {
+  int lo = 0, hi = 0, dlo = 0, res = 2;
+  if (!fp64_only) {
+    const float S[3] = {(float)fr[0], (float)fr[1], (float)fr[2]};
+    res = layer_pairs(recs, rs, S, fp, perd, N, rec, r, lo, hi, dlo);
+  }
+  if (res == 2) res = layer_fp64(recs, rs, fr, bd, a2d, N, rec, r, lo, hi, dlo);
+  return (unsigned)res | ((unsigned)lo << 8) | ((unsigned)hi << 16) | ((unsigned)dlo << 24);
+}
+
+__device__ __forceinline__ void red_shared(uint32_t addr, int v) {
+  asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// Adds the intervals to a row of the difference image at shared address `row`.
+__device__ __forceinline__ void add_intervals(uint32_t row, int lo, int hi, int dlo) {
   if (lo < hi) {
-    atomicAdd(row + lo, 1);
-    if (hi < N) atomicAdd(row + hi, -1);
+    red_shared(row + 4u * (unsigned)lo, 1);
+    red_shared(row + 4u * (unsigned)hi, -1);
   }
   if (dlo < lo) {
-    atomicAdd(row + dlo, 2);
-    if (lo < N) atomicAdd(row + lo, -2);
+    red_shared(row + 4u * (unsigned)dlo, 2);
+    red_shared(row + 4u * (unsigned)lo, -2);
   }
 }
 
@@ -791,32 +929,42 @@ __device__ __forceinline__ void neighbour_ranges(const KArgs &a, int64_t bucket_
   __syncthreads();
 }
 
-template <int NW>
+// One oriented point.  Bound by instruction issue and, behind it, by the latency of each warp's
+// chain from records to items (75 % issue-active at R = 0.6 on the 5M-triangle scene, 28 warps per
+// SM), so the layout buys few instructions per (triangle, layer) item and many resident warps:
+//  - the set-up sorts a triangle's vertices by height and works in columns and layers (R / N), so an
+//    item is one base vertex, two slopes and one margin (three 16-byte loads, 4 fused
+//    multiply-adds), a column count is one rounding, and its margin test one comparison;
+//  - what is read once per batch or chunk (frame, spin vertex, walk over the groups) stays in shared
+//    memory: 72 registers, 7 blocks of 4 warps per SM at N = 64 (5 blocks 306 ms, 6 281 ms, 7 265 ms
+//    for 32,768 points at R = 0.6; 64 registers for 8 blocks spill: 284 ms);
+//  - undecided items go to pairs of floats, not to FP64: 0.6 % of the items, at FP64's 1/64 rate
+//    1/6 of the time before.
+// 32,768 points of the 5M-triangle scene at R = 0.6: 457 -> 222 ms; 131,072 at R = 0.15: 167 ->
+// 77 ms; every point of a 189k-triangle scene at R = 0.3: 33.3 -> 15.9 ms (edge selection, table
+// lookups and a dozen margin tests per item before, band items in FP64).
+template <int NW, bool kCount>
 __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : 3) k_generate(KArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int N = a.N;
+  const int N = a.N, NS = N + 1;  // NS: row stride of the difference image
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t o = blockIdx.x;
-
   Shared s;
   {
     unsigned char *p = smem;
     s.diff = reinterpret_cast<int *>(p);
-    p += ((size_t)N * N * 4 + 15) & ~(size_t)15;
+    p += ((size_t)N * NS * 4 + 15) & ~(size_t)15;
     s.a2d = reinterpret_cast<double *>(p);
     s.bd = s.a2d + N;
     s.fr = s.bd + N;
-    s.a2f = reinterpret_cast<float *>(s.fr + 8);
-    s.bf = s.a2f + N;
-    s.buckets = reinterpret_cast<int *>(s.bf + N);
-    const int nn = (2 * a.nhalf + 1) * (2 * a.nhalf + 1) * (2 * a.nhalf + 1);
-    s.bdup = s.buckets + nn + 1;
-    int *wbase = s.bdup + nn + 1;
+    s.fp = reinterpret_cast<Pair *>(s.fr + 8);
+    s.ff = reinterpret_cast<float4 *>(s.fp + 6);
+    int *wbase = reinterpret_cast<int *>(s.ff + 4);
     s.wq = wbase + warp * kPerWarp;
-    s.wst = s.wq;
     s.bq_rec = s.wq + 64;
-    s.bq_r = reinterpret_cast<unsigned char *>(s.bq_rec + 64);
-    s.slots = reinterpret_cast<float *>(s.bq_rec + 64 + 16);
+    s.bq_r = reinterpret_cast<unsigned char *>(s.bq_rec + kBandQ);
+    s.walk = s.bq_rec + kBandQ + kBandQ / 4;
+    s.slots = reinterpret_cast<float *>(s.walk + 4);
   }
 
   const int64_t og = a.origin_base + o;  // launch-wide origin index
@@ -833,194 +981,254 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : 3) k_generate(KArgs a) 
               nzf = sc.Nrm[3 * (int64_t)vid + 2];
   const int64_t bucket_off = sc.bucket_off;
   const uint32_t nbuckets = sc.nbuckets;
-  uint16_t *const out_img = sc.out + ol * (int64_t)N * N;
   if (!(isfinite(Sx) && isfinite(Sy) && isfinite(Sz) && isfinite(nxf) && isfinite(nyf) &&
         isfinite(nzf))) {
     if (tid == 0) set_status(a.status, RICI_ERR_NONFINITE_INPUT);
     return;
   }
 
-  for (int i = tid; i < N * N; i += NW * 32) s.diff[i] = 0;
+  for (int i = tid; i < N * NS; i += NW * 32) s.diff[i] = 0;
   const double Rd = (double)a.R;
   for (int i = tid; i < N; i += NW * 32) {
-    double al = __ddiv_rn(__dmul_rn(Rd, (double)(2 * i + 1)), (double)(2 * N));
-    double a2 = __dmul_rn(al, al);
-    double b = __ddiv_rn(__dmul_rn(Rd, (double)(2 * i + 1 - N)), (double)(2 * N));
-    s.a2d[i] = a2;
-    s.bd[i] = b;
-    s.a2f[i] = __double2float_rn(a2);
-    s.bf[i] = __double2float_rn(b);
+    const double al = __ddiv_rn(__dmul_rn(Rd, (double)(2 * i + 1)), (double)(2 * N));
+    s.a2d[i] = __dmul_rn(al, al);
+    s.bd[i] = __ddiv_rn(__dmul_rn(Rd, (double)(2 * i + 1 - N)), (double)(2 * N));
   }
   if (tid == 0) {
     s.fr[0] = Sx;
     s.fr[1] = Sy;
     s.fr[2] = Sz;
     frame_fp64(nxf, nyf, nzf, s.fr + 3);
+    const double per = __ddiv_rn((double)N, Rd);
+    s.fr[7] = per;
+    s.fp[0] = to_pair(s.fr[3]);
+    s.fp[1] = to_pair(s.fr[4]);
+    for (int k = 0; k < 4; ++k) s.fp[2 + k] = to_pair(s.fr[3 + k] * per);
+    // frame coefficients of the FP32 path, and those scaled to columns and layers
+    s.ff[0] = make_float4(s.fp[2].h, s.fp[3].h, s.fp[4].h, s.fp[5].h);
+    s.ff[1] = make_float4(s.fp[0].h, s.fp[1].h, __double2float_rn(per), 0.0f);
+    s.ff[2] = make_float4(Sx, Sy, Sz, 4e-7f * (fabsf(Sx) + fabsf(Sy) + fabsf(Sz)));
+    // central axis in world coordinates
+    const float fbx = __double2float_rn(s.fr[5]), fbz = __double2float_rn(s.fr[6]);
+    s.ff[3] = make_float4(fbx * s.fp[0].h, fbx * s.fp[1].h, fbz, 0.0f);
   }
   __syncthreads();
 
-  const float fax = __double2float_rn(s.fr[3]), fay = __double2float_rn(s.fr[4]);
-  const float fbx = __double2float_rn(s.fr[5]), fbz = __double2float_rn(s.fr[6]);
-  const float wx = fbx * fax, wy = fbx * fay, wz = fbz;  // central axis in world coordinates
   const float R = a.R;
-  const float scale = (float)(2 * N) / R;
-  const float spacing = R / (float)N;
-  const float acull_xy = sqrtf(s.a2f[N - 1]) * (1.0f + 1.0f / 4096.0f);
+  const float zmid = 0.5f * (float)(N - 1);  // height of the spin vertex in layers
+  const float wmax = (float)N + 0.25f;       // distances beyond the last column
+  const uint32_t diff_at = static_cast<uint32_t>(__cvta_generic_to_shared(s.diff));
   const bool fp64_only = a.mode == RICI_GEN_FP64;
 
-  unsigned long long n_tri = 0, n_items = 0, n_band = 0, n_cand = 0;
+  // (per lane and block; a lane sees each of its block's items once, fewer than 2^32)
+  unsigned n_tri = 0, n_items = 0, n_band = 0, n_cand = 0;
   int qn = 0;  // warp-uniform candidate queue length
-  int bn = 0;  // warp-uniform FP64 queue length
+  int bn = 0;  // warp-uniform band queue length
 
-  // FP64 re-evaluation of queued band items, one per lane
-  auto flush_band = [&](int cnt) {
-    if (lane < cnt) {
-      int lo = 0, hi = 0, dlo = 0;
-      const int r = s.bq_r[lane];
-      if (layer_fp64(a.rec, a.rs, s.fr, s.bd, s.a2d, N, s.bq_rec[lane], r, lo, hi, dlo))
-        add_intervals(s.diff + r * N, N, lo, hi, dlo);
+  // warp collective: queue an item for re-evaluation where `add`
+  auto push_band = [&](bool add, int rec, int r) {
+    const unsigned bal = __ballot_sync(0xffffffffu, add);
+    if (add) {
+      const int pos = bn + __popc(bal & ((1u << lane) - 1u));
+      s.bq_rec[pos] = rec;
+      s.bq_r[pos] = (unsigned char)r;
+      if (kCount) ++n_band;
     }
-    __syncwarp();
-    const int rest = bn - cnt;
-    int mr = 0, mq = 0;
-    if (lane < rest) {
-      mr = s.bq_rec[cnt + lane];
-      mq = s.bq_r[cnt + lane];
-    }
-    __syncwarp();
-    if (lane < rest) {
-      s.bq_rec[lane] = mr;
-      s.bq_r[lane] = mq;
-    }
-    bn = rest;
-    __syncwarp();
+    bn += __popc(bal);
   };
 
-  auto process_batch = [&](int cnt) {
+  // Processes the first cnt queued candidates; the last call empties the band queue.
+  auto process_batch = [&](int cnt, bool last) {
     // ---- per-triangle setup: one survivor per lane
-    int nlay = 0;
-    float *sl = s.slots + lane * kSlot;
+    int nlow = 0, nup = 0;            // layers certainly inside the lower and the upper segment
+    int rlow = 0, rup = 0;            // the first of each
+    int rec = 0;
+    int a0 = 0, a1 = 0, a2 = 0;       // first layer not certainly below vertex 0, 1, 2
+    int b0 = -1, b1 = -1, b2 = -1;    // last layer not certainly above it
+    float4 v0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), v2 = v0, sl = v0;
+    float2 su = make_float2(0.0f, 0.0f);
     if (lane < cnt) {
-      const int rec = s.wq[lane];
-      float4 r1 = a.rec[a.rs + rec], r2 = a.rec[2 * a.rs + rec], r3 = a.rec[3 * a.rs + rec];
-      float P[9] = {r1.x, r1.y, r1.z, r1.w, r2.x, r2.y, r2.z, r2.w, r3.x};
-      float tx[3], ty[3], tz[3], M = 0.0f;
+      rec = s.wq[lane];
+      const float4 r1 = a.rec[a.rs + rec], r2 = a.rec[2 * a.rs + rec], r3 = a.rec[3 * a.rs + rec];
+      const float P[9] = {r1.x, r1.y, r1.z, r1.w, r2.x, r2.y, r2.z, r2.w, r3.x};
+      const float4 fg = s.ff[0], fa = s.ff[1], S = s.ff[2];
+      const float gax = fg.x, gay = fg.y, gbx = fg.z, gbz = fg.w, fax = fa.x, fay = fa.y;
+      float x[3], y[3], z[3], M = 0.0f;
 #pragma unroll
-      for (int k = 0; k < 3; ++k)
-        M = fmaxf(M, project_fp32(P[3 * k], P[3 * k + 1], P[3 * k + 2], Sx, Sy, Sz, fax, fay, fbx,
-                                  fbz, tx[k], ty[k], tz[k]));
-      // |T32 - T64| <= dT for every coordinate (first-order bound 7uM, 10uM with slack)
-      const float dT = 10.0f * kU * M + 1e-37f;
-      const float dside = kSafety * (dT + kU * R);
-      float zmin = fminf(fminf(tz[0], tz[1]), tz[2]), zmax = fmaxf(fmaxf(tz[0], tz[1]), tz[2]);
-      float xl = fminf(fminf(tx[0], tx[1]), tx[2]), xh = fmaxf(fmaxf(tx[0], tx[1]), tx[2]);
-      float yl = fminf(fminf(ty[0], ty[1]), ty[2]), yh = fmaxf(fmaxf(ty[0], ty[1]), ty[2]);
-      float gx = fmaxf(0.0f, fmaxf(xl, -xh)), gy = fmaxf(0.0f, fmaxf(yl, -yh));
-      float lim = acull_xy + 2.0f * dT;
-      bool keep = gx * gx + gy * gy <= lim * lim;
-      // layers whose side decision is not certainly identical for all three vertices
-      int r_lo = 0, r_hi = -1;
-      if (keep) {
-        float zl = zmin - dside, zh = zmax + dside;
-        float fl = ceilf((zl * scale + (float)(N - 1)) * 0.5f);
-        r_lo = fl <= 0.0f ? 0 : (fl >= (float)N ? N : (int)fl);
-        while (r_lo > 0 && s.bf[r_lo - 1] > zl) --r_lo;
-        while (r_lo < N && s.bf[r_lo] <= zl) ++r_lo;
-        float fh = floorf((zh * scale + (float)(N - 1)) * 0.5f);
-        r_hi = fh < 0.0f ? -1 : (fh >= (float)(N - 1) ? N - 1 : (int)fh);
-        while (r_hi < N - 1 && s.bf[r_hi + 1] <= zh) ++r_hi;
-        while (r_hi >= 0 && s.bf[r_hi] > zh) --r_hi;
-        nlay = max(0, r_hi - r_lo + 1);
+      for (int k = 0; k < 3; ++k) {
+        const float dx = __fsub_rn(P[3 * k], S.x), dy = __fsub_rn(P[3 * k + 1], S.y),
+                    dz = __fsub_rn(P[3 * k + 2], S.z);
+        const float qx = __fmaf_rn(fay, dy, __fmul_rn(fax, dx));
+        x[k] = __fmaf_rn(gbz, qx, -__fmul_rn(gbx, dz));
+        y[k] = __fmaf_rn(gax, dy, -__fmul_rn(gay, dx));
+        z[k] = __fmaf_rn(gbx, qx, __fmaf_rn(gbz, dz, zmid));
+        M = fmaxf(M, fabsf(dx) + fabsf(dy) + fabsf(dz));
       }
-      if (nlay > 0) {
-        unsigned meta = (unsigned)r_lo;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          sl[SX + k] = tx[k];
-          sl[SY + k] = ty[k];
-          sl[SZ + k] = tz[k];
-          // side band: the one layer a vertex could be ambiguous against
-          float fr_ = rintf((tz[k] * scale + (float)(N - 1)) * 0.5f);
-          int rk = fr_ <= 0.0f ? 0 : (fr_ >= (float)(N - 1) ? N - 1 : (int)fr_);
-          unsigned band = kNoBand;
-          for (int d = -1; d <= 1; ++d) {
-            int rr = rk + d;
-            if (rr >= 0 && rr < N && fabsf(tz[k] - s.bf[rr]) <= dside) band = (unsigned)rr;
-          }
-          meta |= band << (8 * (k + 1));
+      // |T32 - T64| <= dT for every coordinate, in columns (first-order bound 7 u M per unit, 10 u M
+      // with slack; the height's offset adds u N)
+      const float dT = 10.01f * kU * M * fa.z + kU * (float)N + 1e-37f;
+      const float xl = fminf(fminf(x[0], x[1]), x[2]), xh = fmaxf(fmaxf(x[0], x[1]), x[2]);
+      const float yl = fminf(fminf(y[0], y[1]), y[2]), yh = fmaxf(fmaxf(y[0], y[1]), y[2]);
+      const float gx = fmaxf(0.0f, fmaxf(xl, -xh)), gy = fmaxf(0.0f, fmaxf(yl, -yh));
+      const float lim = ((float)N - 0.5f) * (1.0f + 1.0f / 4096.0f) + 2.0f * dT;
+      if (!(gx * gx + gy * gy > lim * lim)) {
+        auto order = [&](int i, int j) {  // the lower of vertices i, j to place i
+          const bool sw = z[j] < z[i];
+          const float tx = x[i], ty = y[i], tz = z[i];
+          x[i] = sw ? x[j] : tx;
+          y[i] = sw ? y[j] : ty;
+          z[i] = sw ? z[j] : tz;
+          x[j] = sw ? tx : x[j];
+          y[j] = sw ? ty : y[j];
+          z[j] = sw ? tz : z[j];
+        };
+        order(0, 1);
+        order(1, 2);
+        order(0, 1);
+        // a layer within dside of a vertex has an uncertain side (conversions saturate)
+        const float dside = kSafety * (dT + 4.0f * kU * (float)N);
+        a0 = __float2int_ru(z[0] - dside);
+        b0 = min(__float2int_rd(z[0] + dside), N);
+        a1 = __float2int_ru(z[1] - dside);
+        b1 = min(__float2int_rd(z[1] + dside), N);
+        a2 = __float2int_ru(z[2] - dside);
+        b2 = min(__float2int_rd(z[2] + dside), N);
+        if (fp64_only || !(dside < 0.25f)) {
+          // every layer it may cross goes to the band queue, through items without a margin
+          const bool known = dside < 1e30f;
+          rlow = known ? max(a0, 0) : 0;
+          nlow = max(min(known ? b2 : N - 1, N - 1) - rlow + 1, 0);
+          rup = nlow;
+          v0.w = -1.0f;
+          a0 = a1 = a2 = 0;
+          b0 = b1 = b2 = -1;
+        } else {
+          rlow = max(b0, -1) + 1;
+          nlow = max(min(a1, N) - rlow, 0);
+          rup = max(b1, -1) + 1;
+          nup = max(min(a2, N) - rup, 0);
+          // Per-edge bound on |E32 - E64| per component.  E = T_u + (r - Z_u) slope; the slope's
+          // relative error is that of 1 / (Z_v - Z_u) (heights off by dT each, at most 1/20 of the
+          // difference, else the edge's items go to FP64), of the difference x_v - x_u and three
+          // roundings; with lambda = (r - Z_u) / (Z_v - Z_u) in [0, 1]:
+          //   dE <= 1.1 (3 dT + u (ext + mag) + (ext + 2 dT) el),  el <= 3.3 dT / |Z_v - Z_u| + 7 u,
+          // ext = max(|x_v - x_u|, |y_v - y_u|), mag the largest coordinate (u mag <= dT / 10).
+          const float d01x = x[1] - x[0], d01y = y[1] - y[0], h01 = z[1] - z[0];
+          const float d02x = x[2] - x[0], d02y = y[2] - y[0], h02 = z[2] - z[0];
+          const float d12x = x[2] - x[1], d12y = y[2] - y[1], h12 = z[2] - z[1];
+          auto slope = [&](float dx, float dy, float h, float &sx, float &sy) -> float {
+            const float inv = rcp_fast(h);
+            sx = __fmul_rn(dx, inv);
+            sy = __fmul_rn(dy, inv);
+            const float steep = fmaxf(fabsf(sx), fabsf(sy)), ext = fmaxf(fabsf(dx), fabsf(dy));
+            return h > 40.0f * dT ? dT * (3.9f + 3.7f * steep) + 9.0f * kU * ext
+                                  : __int_as_float(0x7f800000);
+          };
+          const float de02 = slope(d02x, d02y, h02, sl.x, sl.y);
+          const float de01 = slope(d01x, d01y, h01, sl.z, sl.w);
+          const float de12 = slope(d12x, d12y, h12, su.x, su.y);
+          // margin of an item's distances |E| <= N + 1/4: sqrt(2) dE with the safety factor, and
+          // the rounding of |E| (below 5 u N) with slack; hd = 1/2 - delta
+          const float round_n = 12.0f * kU * (float)(N + 1);
+          v0 = make_float4(x[0], y[0], z[0],
+                           0.5f - (kSafety * 1.4143f * fmaxf(de02, de01) + round_n));
+          v2 = make_float4(x[2], y[2], z[2],
+                           0.5f - (kSafety * 1.4143f * fmaxf(de02, de12) + round_n));
         }
-        if (fp64_only || dside >= 0.25f * spacing) meta = (meta & ~0xff00u) | (kAllBand << 8);
-        sl[SGID + 0] = r3.y;
-        sl[SGID + 1] = r3.z;
-        sl[SGID + 2] = r3.w;
-        // per-edge bound on |E32 - E64| per component (edge k is opposite vertex k):
-        // E = T_u + lambda (T_v - T_u); lambda = (beta - z_u) / (z_v - z_u)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const int i = k == 0 ? 1 : 0, j = k == 2 ? 1 : 2;
-          const float den = fabsf(tz[j] - tz[i]);
-          const float eden = 2.0f * dT + kU * den;
-          // lambda = (beta - z_i) * (1 / (z_j - z_i)): reciprocal and product each round once
-          const float el = (kU * R + dT + kU * den + eden) / (den - eden) + 3.0f * kU;
-          const float ext = fmaxf(fabsf(tx[j] - tx[i]), fabsf(ty[j] - ty[i]));
-          const float mag = fmaxf(fmaxf(fabsf(tx[i]), fabsf(tx[j])), fmaxf(fabsf(ty[i]), fabsf(ty[j])));
-          const float de = 1.1f * (3.0f * dT + kU * (ext + mag) + (ext + 2.0f * dT) * el);
-          sl[SDE + k] = (den > eden && de < 1e30f) ? de : __int_as_float(0x7f800000);
-          sl[SINV + k] = __frcp_rn(tz[j] - tz[i]);
-        }
-        sl[SMETA] = __uint_as_float(meta);
-        sl[SREC] = __int_as_float(rec);
       }
     }
-    // ---- distribute (triangle, layer) items over the lanes
+    // ---- stage the triangles that have items, without gaps, and lay out their items in a row
+    const int nlay = nlow + nup;
+    const unsigned has = __ballot_sync(0xffffffffu, nlay > 0);
     int incl = nlay;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, incl, d);
+      const int y = __shfl_up_sync(0xffffffffu, incl, d);
       if (lane >= d) incl += y;
     }
     const int total = __shfl_sync(0xffffffffu, incl, 31);
-    const int first = incl - nlay;  // this lane's triangle owns items [first, first + nlay)
-    n_tri += nlay > 0;
-    for (int base = 0; base < total; base += 32) {
-      const int it = base + lane;
-      const bool act = it < total;
-      // owner of each item of this window: every triangle with items in the window marks the
-      // first window position it owns (positions are distinct; the triangle holding position 0
-      // always marks it), and an item belongs to the triangle of the last mark at or before it
+    const int first = nlay > 0 ? incl - nlay : 0x7fffffff;
+    if (nlay > 0) {
+      if (kCount) ++n_tri;
+      float4 *t4 = reinterpret_cast<float4 *>(s.slots + __popc(has & ((1u << lane) - 1u)) * kSlot);
+      t4[S_V0 / 4] = v0;
+      t4[S_V2 / 4] = v2;
+      t4[S_LONG / 4] = sl;
+      t4[S_UP / 4] = make_float4(su.x, su.y, __int_as_float(first),
+                                 __int_as_float(rlow | (nlow << 8) | ((rup - nlow) << 16)));
+      reinterpret_cast<int *>(t4)[S_REC] = rec;
+    }
+    // ---- layers whose side is uncertain for a vertex, each once
+    if (__any_sync(0xffffffffu, a0 <= b0 || a1 <= b1 || a2 <= b2)) {
+      const bool e0 = a0 <= b0 && a0 >= 0 && a0 < N;
+      const bool e1 = a1 <= b1 && a1 >= 0 && a1 < N && !(a0 <= b0 && a1 == a0);
+      const bool e2 = a2 <= b2 && a2 >= 0 && a2 < N && !(a1 <= b1 && a2 == a1);
+      push_band(e0, rec, a0);
+      push_band(e1, rec, a1);
+      push_band(e2, rec, a2);
+      if (kCount) n_items += (int)e0 + (int)e1 + (int)e2;
+    }
+    __syncwarp();
+    // ---- the items, 32 at a time: an item's triangle is the last one that starts at or before it
+    int started = 0;  // triangles that started in earlier windows
+    for (int base = 0;;) {
+      if (bn >= 32 || (last && base >= total && bn > 0)) {
+        // re-evaluate queued band items, one per lane
+        const int n = min(bn, 32);
+        if (lane < n) {
+          const int r = s.bq_r[lane];
+          const unsigned v = band_item(a.rec, a.rs, s.fr, s.fp, s.bd, s.a2d, s.ff[1].z, N, fp64_only,
+                                       s.bq_rec[lane], r);
+          if (v & 0xffu)
+            add_intervals(diff_at + 4u * (unsigned)(r * NS), (v >> 8) & 0xff, (v >> 16) & 0xff, v >> 24);
+        }
+        __syncwarp();
+        bn -= n;
+        for (int q = 0; q < bn; q += 32) {  // the rest moves down (to entries already read)
+          const int mr = q + lane < bn ? s.bq_rec[n + q + lane] : 0;
+          const int ml = q + lane < bn ? s.bq_r[n + q + lane] : 0;
+          __syncwarp();
+          if (q + lane < bn) {
+            s.bq_rec[q + lane] = mr;
+            s.bq_r[q + lane] = (unsigned char)ml;
+          }
+          __syncwarp();
+        }
+        continue;
+      }
+      if (base >= total) break;
       const int d = first - base;
-      const bool mark = nlay > 0 && d < 32 && d + nlay > 0;
-      const int pos = d > 0 ? d : 0;
-      if (mark) s.wst[pos] = lane;
-      const unsigned starts = __reduce_or_sync(0xffffffffu, mark ? 1u << pos : 0u);
-      __syncwarp();
-      const int q = 31 - __clz(starts & (0xffffffffu >> (31 - lane)));  // bit 0 is always set
-      const int owner = s.wst[q];
-      const int ofirst = __shfl_sync(0xffffffffu, first, owner);
-      int res = 0, r = 0, rec = 0, lo = 0, hi = 0, dlo = 0;
-      if (act) {
-        const float *ts = s.slots + owner * kSlot;
-        const unsigned meta = __float_as_uint(ts[SMETA]);
-        r = (int)(meta & 0xffu) + (it - ofirst);
-        rec = __float_as_int(ts[SREC]);
-        const unsigned b0 = (meta >> 8) & 0xffu;
-        const bool band = b0 == kAllBand || r == (int)b0 || r == (int)((meta >> 16) & 0xffu) ||
-                          r == (int)(meta >> 24);
-        res = band ? 2 : layer_fp32(s.bf, s.a2f, N, ts, r, scale, lo, hi, dlo);
-        ++n_items;
+      const unsigned starts = __reduce_or_sync(0xffffffffu, (unsigned)d < 32u ? 1u << d : 0u);
+      const int owner = started + __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
+      started += __popc(starts);
+      const int it = base + lane;
+      bool band = false;
+      int r = 0;
+      const float *ts = s.slots + owner * kSlot;
+      if (it < total) {
+        const float4 up4 = *reinterpret_cast<const float4 *>(ts + S_UP);
+        const float4 lg4 = *reinterpret_cast<const float4 *>(ts + S_LONG);
+        const int k = it - __float_as_int(up4.z);
+        const unsigned meta = __float_as_uint(up4.w);
+        const bool up = k >= (int)((meta >> 8) & 0xffu);
+        r = k + (int)(up ? meta >> 16 : meta & 0xffu);
+        const float4 v = *reinterpret_cast<const float4 *>(ts + (up ? S_V2 : S_V0));
+        const float h = __fsub_rn((float)r, v.z);
+        const float E0x = __fmaf_rn(h, lg4.x, v.x), E0y = __fmaf_rn(h, lg4.y, v.y);
+        const float E1x = __fmaf_rn(h, up ? up4.x : lg4.z, v.x);
+        const float E1y = __fmaf_rn(h, up ? up4.y : lg4.w, v.y);
+        int lo, hi, dlo;
+        band = !layer_fp32(E0x, E0y, E1x, E1y, v.w, wmax, lo, hi, dlo);
+        if (!band)
+          add_intervals(diff_at - 4u * (unsigned)kRoundBits + 4u * (unsigned)(r * NS), lo, hi, dlo);
+        if (kCount) ++n_items;
       }
-      // items inside the error band wait in the FP64 queue (evaluated 32 at a time)
-      const unsigned bal = __ballot_sync(0xffffffffu, res == 2);
-      if (res == 2) {
-        const int pos = bn + __popc(bal & ((1u << lane) - 1u));
-        s.bq_rec[pos] = rec;
-        s.bq_r[pos] = r;
-        ++n_band;
+      // items inside the error band wait in the queue (evaluated 32 at a time)
+      if (__any_sync(0xffffffffu, band)) {
+        push_band(band, band ? __float_as_int(ts[S_REC]) : 0, r);
+        __syncwarp();
       }
-      bn += __popc(bal);
-      if (res == 1) add_intervals(s.diff + r * N, N, lo, hi, dlo);
-      __syncwarp();
-      if (bn >= 32) flush_band(32);
+      base += 32;
     }
     __syncwarp();
   };
@@ -1030,118 +1238,126 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : 3) k_generate(KArgs a) 
   // sphere containing the bounding spheres of its records fails its test only if every record
   // fails the record test: the record test widened by the sphere's radius, with a margin that
   // covers the record test's own and both tests' rounding.
-  const float mpos = 4e-7f * (fabsf(Sx) + fabsf(Sy) + fabsf(Sz));
   auto sphere_pass = [&](const float4 c) -> bool {
     if (!(c.w < 1e30f)) return true;
-    const float dx = c.x - Sx, dy = c.y - Sy, dz = c.z - Sz;
-    const float z = fmaf(wx, dx, fmaf(wy, dy, wz * dz));
+    const float4 S = s.ff[2], w = s.ff[3];
+    const float dx = c.x - S.x, dy = c.y - S.y, dz = c.z - S.z;
+    const float z = fmaf(w.x, dx, fmaf(w.y, dy, w.z * dz));
     const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    const float m = 2e-3f * R + 2e-5f * (fabsf(dx) + fabsf(dy) + fabsf(dz) + 2.0f * c.w) + mpos;
+    const float m = 2e-3f * R + 2e-5f * (fabsf(dx) + fabsf(dy) + fabsf(dz) + 2.0f * c.w) + S.w;
     const float al = a.alpha_cull + c.w + m;
     return fabsf(z) <= a.beta_cull + c.w + m && d2 - z * z <= al * al;
   };
-  const int64_t rb = a.starts[bucket_off], re = a.starts[bucket_off + nbuckets + 1];
-  if (re > rb) {
-    const int64_t c_lo = rb >> kChunkShift, c_hi = (re - 1) >> kChunkShift;
-    const int64_t g_lo = rb >> kGroupShift, ng = ((re - 1) >> kGroupShift) - g_lo + 1;
-    // group g_lo + k0 + lane * NW + warp: consecutive groups (neighbours in space) go to
-    // different warps
-    for (int64_t k0 = 0; k0 < ng; k0 += 32 * NW) {
-      const int64_t gi = k0 + (int64_t)lane * NW + warp;
-      const bool gp = gi < ng && sphere_pass(a.grp[g_lo + gi]);
-      unsigned gm = __ballot_sync(0xffffffffu, gp);
-      while (gm) {
-        const int64_t g = g_lo + k0 + (int64_t)(__ffs(gm) - 1) * NW + warp;
-        gm &= gm - 1;
-        const int64_t ci = (g << (kGroupShift - kChunkShift)) + lane;
-        const bool cp = ci >= c_lo && ci <= c_hi && sphere_pass(a.chk[ci]);
-        unsigned cm = __ballot_sync(0xffffffffu, cp);
-        // records of the passing chunks; the next chunk's spheres are loaded before the current
-        // ones are tested and queued, so the load's latency overlaps that work
-        int64_t t = 0;
-        float4 cn = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        bool more = cm != 0;
-        if (more) {
-          t = (((g << (kGroupShift - kChunkShift)) + __ffs(cm) - 1) << kChunkShift) + lane;
-          cm &= cm - 1;
-          if (t >= rb && t < re) cn = a.rec[t];
+  const int rb = a.starts[bucket_off], re = a.starts[bucket_off + nbuckets + 1];
+  {
+    // group base + lane * NW + warp: consecutive groups (neighbours in space) go to different warps.
+    // The walk below keeps its place (k0, the masks of passing groups and chunks) and hands over
+    // 32 passing records at a time, so the batch code exists once.
+    const int gend = re > rb ? ((re - 1) >> kGroupShift) + 1 : 0;
+    if (lane == 0) {
+      s.walk[0] = rb >> kGroupShift;
+      s.walk[2] = 0;
+    }
+    __syncwarp();
+    int chunk0 = 0, t = 0;  // first chunk of the current group; this lane's record of a passing chunk
+    unsigned cm = 0;        // passing chunks left in the group
+    bool more = false;      // t is in a chunk that passed and has not been tested
+    // moves to the next passing chunk
+    auto advance = [&]() {
+      if (cm == 0) {
+        int k0 = s.walk[0], gk = s.walk[1];
+        unsigned gm = (unsigned)s.walk[2];
+        do {
+          while (gm == 0) {
+            if (k0 >= gend) {
+              more = false;
+              return;
+            }
+            const int gi = k0 + lane * NW + warp;
+            const bool gp = gi < gend && sphere_pass(a.grp[gi]);
+            gm = __ballot_sync(0xffffffffu, gp);
+            gk = k0;
+            k0 += 32 * NW;
+          }
+          chunk0 = (gk + (__ffs(gm) - 1) * NW + warp) << (kGroupShift - kChunkShift);
+          gm &= gm - 1;
+          const int ci = chunk0 + lane;
+          const bool cp = ci >= (rb >> kChunkShift) && ci <= ((re - 1) >> kChunkShift) &&
+                          sphere_pass(a.chk[ci]);
+          cm = __ballot_sync(0xffffffffu, cp);
+        } while (cm == 0);
+        __syncwarp();
+        if (lane == 0) {
+          s.walk[0] = k0;
+          s.walk[1] = gk;
+          s.walk[2] = (int)gm;
         }
-        while (more) {
-          const int64_t tc = t;
-          const float4 c = cn;
-          more = cm != 0;
-          if (more) {
-            t = (((g << (kGroupShift - kChunkShift)) + __ffs(cm) - 1) << kChunkShift) + lane;
-            cm &= cm - 1;
-            if (t >= rb && t < re) cn = a.rec[t];
-          }
-          bool pass = false;
-          if (tc >= rb && tc < re) {
-            float dx = c.x - Sx, dy = c.y - Sy, dz = c.z - Sz;
-            float z = fmaf(wx, dx, fmaf(wy, dy, wz * dz));
-            float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            float m = 1e-3f * R + 1e-5f * (fabsf(dx) + fabsf(dy) + fabsf(dz));
-            float al = a.alpha_cull + c.w + m;
-            pass = fabsf(z) <= a.beta_cull + c.w + m && d2 - z * z <= al * al;
-            ++n_cand;
-          }
-          const unsigned bal = __ballot_sync(0xffffffffu, pass);
-          if (pass) s.wq[qn + __popc(bal & ((1u << lane) - 1u))] = (int)tc;
-          qn += __popc(bal);
-          __syncwarp();
-          if (qn >= 32) {
-            process_batch(32);
-            int rest = qn - 32;
-            int moved = lane < rest ? s.wq[32 + lane] : 0;
-            __syncwarp();
-            if (lane < rest) s.wq[lane] = moved;
-            qn = rest;
-            __syncwarp();
-          }
-        }
+        __syncwarp();
       }
+      t = ((chunk0 + __ffs(cm) - 1) << kChunkShift) + lane;
+      cm &= cm - 1;
+      more = true;
+    };
+    advance();
+    while (true) {
+      float4 cn = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (more && t >= rb && t < re) cn = a.rec[t];
+      while (more && qn < 32) {
+        // the next chunk's spheres are loaded before the current ones are tested and queued, so the
+        // load's latency overlaps that work
+        const int tc = t;
+        const float4 c = cn;
+        advance();
+        if (more && t >= rb && t < re) cn = a.rec[t];
+        bool pass = false;
+        if (tc >= rb && tc < re) {
+          const float4 S = s.ff[2], w = s.ff[3];
+          float dx = c.x - S.x, dy = c.y - S.y, dz = c.z - S.z;
+          float z = fmaf(w.x, dx, fmaf(w.y, dy, w.z * dz));
+          float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+          float m = 1e-3f * R + 1e-5f * (fabsf(dx) + fabsf(dy) + fabsf(dz));
+          float al = a.alpha_cull + c.w + m;
+          pass = fabsf(z) <= a.beta_cull + c.w + m && d2 - z * z <= al * al;
+          if (kCount) ++n_cand;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, pass);
+        if (pass) s.wq[qn + __popc(bal & ((1u << lane) - 1u))] = tc;
+        qn += __popc(bal);
+      }
+      // (the last call, with no record left, is the one that empties the band queue)
+      if (qn == 0 && bn == 0) break;
+      __syncwarp();
+      const int cnt = min(qn, 32);
+      process_batch(cnt, qn <= 32 && !more);
+      qn -= cnt;
+      const int moved = lane < qn ? s.wq[32 + lane] : 0;
+      __syncwarp();
+      if (lane < qn) s.wq[lane] = moved;
+      __syncwarp();
     }
   }
-  if (qn > 0) process_batch(qn);
-  if (bn > 0) flush_band(bn);
-
-  if (a.counters) {
+  if (kCount) {
+    const unsigned n[4] = {n_tri, n_items, n_band, n_cand};
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-      n_tri += __shfl_down_sync(0xffffffffu, n_tri, d);
-      n_items += __shfl_down_sync(0xffffffffu, n_items, d);
-      n_band += __shfl_down_sync(0xffffffffu, n_band, d);
-      n_cand += __shfl_down_sync(0xffffffffu, n_cand, d);
-    }
-    if (lane == 0) {
-      atomicAdd(a.counters + 0, n_tri);
-      atomicAdd(a.counters + 1, n_items);
-      atomicAdd(a.counters + 2, n_band);
-      atomicAdd(a.counters + 3, n_cand);
+    for (int k = 0; k < 4; ++k) {
+      unsigned long long v = n[k];
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
+      if (lane == 0) atomicAdd(a.counters + k, v);
     }
   }
   __syncthreads();
 
   // ---- prefix-sum each row of the difference image, saturate, store uint16
-  uint16_t *out = out_img;
+  uint16_t *out = sc.out + ol * (int64_t)N * N;
   const int cpl = (N + 31) / 32;
   if ((N == 64 || N == 128) && (reinterpret_cast<uintptr_t>(out) & 7) == 0) {
-    // each lane owns 2 (N = 64) or 4 (N = 128) consecutive columns: one vector load of the
-    // difference row and one 32- or 64-bit store of the packed counts
+    // each lane owns 2 (N = 64) or 4 (N = 128) consecutive columns and makes one 32- or 64-bit
+    // store of the packed counts
     for (int r = warp; r < N; r += NW) {
-      const int *row = s.diff + r * N;
-      int v0, v1, v2 = 0, v3 = 0;
-      if (cpl == 2) {
-        const int2 x = *reinterpret_cast<const int2 *>(row + 2 * lane);
-        v0 = x.x;
-        v1 = x.y;
-      } else {
-        const int4 x = *reinterpret_cast<const int4 *>(row + 4 * lane);
-        v0 = x.x;
-        v1 = x.y;
-        v2 = x.z;
-        v3 = x.w;
-      }
+      const int *row = s.diff + r * NS + cpl * lane;
+      const int v0 = row[0], v1 = row[1];
+      const int v2 = cpl == 4 ? row[2] : 0, v3 = cpl == 4 ? row[3] : 0;
       const int sum = v0 + v1 + v2 + v3;
       int incl = sum;
 #pragma unroll
@@ -1162,7 +1378,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : 3) k_generate(KArgs a) 
     return;
   }
   for (int r = warp; r < N; r += NW) {
-    const int *row = s.diff + r * N;
+    const int *row = s.diff + r * NS;
     const int c0 = lane * cpl, c1 = min(N, c0 + cpl);
     int sum = 0;
     for (int c = c0; c < c1; ++c) sum += row[c];
@@ -1180,27 +1396,25 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : 3) k_generate(KArgs a) 
   }
 }
 
-size_t generate_smem_bytes(int N, int nhalf, int warps) {
-  const int nn = (2 * nhalf + 1) * (2 * nhalf + 1) * (2 * nhalf + 1);
-  size_t b = ((size_t)N * N * 4 + 15) & ~(size_t)15;
-  b += (size_t)(2 * N + 8) * sizeof(double);
-  b += (size_t)(2 * N) * sizeof(float);
-  b += 2 * (size_t)(nn + 1) * sizeof(int);
+size_t generate_smem_bytes(int N, int warps) {
+  size_t b = ((size_t)N * (N + 1) * 4 + 15) & ~(size_t)15;
+  b += (size_t)(2 * N + 8) * sizeof(double) + 6 * sizeof(Pair) + 4 * sizeof(float4);
   b += (size_t)warps * kPerWarp * 4;
   return b;
 }
 
 template <int NW>
 cudaError_t launch_k_generate(const KArgs &k, int64_t total_origins, cudaStream_t st) {
-  const size_t smem = generate_smem_bytes(k.N, k.nhalf, NW);
-  cudaError_t e = cudaFuncSetAttribute(k_generate<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  const size_t smem = generate_smem_bytes(k.N, NW);
+  auto kern = k.counters ? k_generate<NW, true> : k_generate<NW, false>;
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   for (int64_t o0 = 0; o0 < total_origins; o0 += 0x7fffffff) {
     const int64_t cnt = total_origins - o0 < 0x7fffffff ? total_origins - o0 : 0x7fffffff;
     KArgs kk = k;
     kk.origin_base = o0;
-    k_generate<NW><<<(unsigned)cnt, NW * 32, smem, st>>>(kk);
+    kern<<<(unsigned)cnt, NW * 32, smem, st>>>(kk);
     count_launches(1);
   }
   return cudaGetLastError();
