@@ -266,6 +266,27 @@ constexpr int64_t generate_workspace_bytes(int64_t num_triangles) {
 
 __device__ __forceinline__ void set_status(int *status, int bits) { atomicOr(status, bits); }
 
+// Images whose pixels a warp may read 8 at a time: rows of a multiple of 8 pixels that divide 256,
+// 16-byte aligned.
+__host__ __device__ constexpr bool rows_of_8(int N) {
+  return N == 8 || N == 16 || N == 32 || N == 64 || N == 128;
+}
+__device__ __forceinline__ bool aligned16(const void *p) {
+  return (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+}
+
+// Warp collective: the column deltas (delta of column 0 := 0) of 256 consecutive pixels, 8 per lane
+// (w: the lane's 8 pixels), of an image with rows_of_8(N) starting at a multiple of 256; the pixel
+// before a lane's first one is the previous lane's last, and lane 0 starts a row.
+__device__ __forceinline__ void deltas8(uint4 w, int lane, int N, int (&d)[8]) {
+  const unsigned prev = __shfl_up_sync(0xffffffffu, w.w >> 16, 1);
+  const int p[8] = {(int)(w.x & 0xffffu), (int)(w.x >> 16), (int)(w.y & 0xffffu), (int)(w.y >> 16),
+                    (int)(w.z & 0xffffu), (int)(w.z >> 16), (int)(w.w & 0xffffu), (int)(w.w >> 16)};
+  d[0] = ((lane * 8) & (N - 1)) == 0 ? 0 : p[0] - (int)prev;
+#pragma unroll
+  for (int e = 1; e < 8; ++e) d[e] = p[e] - p[e - 1];
+}
+
 // Number of kernels this library has enqueued in the process (for launch accounting).
 void count_launches(int64_t n);
 

@@ -6,10 +6,10 @@
 // minimal d(i,j).  Everything is integer arithmetic, so results are exact.
 //
 // Stages:
-//   k_encode        per image: int8 column deltas (delta of column 0 := 0); for needles also
-//                   a byte mask of the non-zero deltas and per-row sums of squared deltas, for
-//                   the haystack a warp-interleaved layout (32 images per group, 16-byte chunks
-//                   chunk-major); images with any |delta| > 127 are "wide" and listed apart.
+//   k_encode_needles, k_encode_groups   per image: int8 column deltas (delta of column 0 := 0);
+//                   for needles also a byte mask of the non-zero deltas and per-row sums of
+//                   squared deltas, for the haystack groups of 32 images, piece-major; images
+//                   with any |delta| > 127 are "wide" and listed apart.
 //   k_true_distance d(i, match_i) in int64 straight from the uint16 images.
 //   k_dense         narrow x narrow pairs on CUDA cores.  Per row, sum m(a-b)^2 =
 //                   sum a^2 + sum (mb)^2 - 2 sum ab with sum a^2 precomputed and the other two
@@ -41,76 +41,65 @@ __device__ __forceinline__ int delta_at(const uint16_t *img, int N, int r, int c
   return c == 0 ? 0 : (int)img[r * N + c] - (int)img[r * N + c - 1];
 }
 
-// Byte offset of the delta at flat position k of image i in the warp-interleaved layout read by
-// k_dense: 32 consecutive images form a group, and within a group each row is stored as chunks
-// of CW 32-bit words per image, chunk-major, so the 32 lanes of a warp (32 consecutive images)
-// read the same chunk of the same row with one contiguous 32 x 4CW-byte access.
-__device__ __forceinline__ int64_t interleaved_offset(int64_t i, int N, int k) {
-  const int WPR = N / 4, CW = WPR < 4 ? WPR : 4;
-  const int r = k / N, c = k - r * N;
-  const int w = c >> 2, v = w / CW, ww = w - v * CW;
-  const int64_t g = i >> 5, l = i & 31;
-  return ((((g * N + r) * (WPR / CW) + v) * 32 + l) * CW + ww) * 4 + (c & 3);
+// Four deltas clamped to [-127, 127] as the bytes of a word.
+__device__ __forceinline__ uint32_t pack_deltas(int a, int b, int c, int d) {
+  a = min(max(a, -127), 127);
+  b = min(max(b, -127), 127);
+  c = min(max(c, -127), 127);
+  d = min(max(d, -127), 127);
+  return __byte_perm(__byte_perm((uint32_t)a, (uint32_t)b, 0x0040),
+                     __byte_perm((uint32_t)c, (uint32_t)d, 0x0040), 0x5410);
+}
+// 0xff in every byte of w that is not zero.
+__device__ __forceinline__ uint32_t nonzero_bytes(uint32_t w) {
+  const uint32_t t = (w | ((w & 0x7f7f7f7fu) + 0x7f7f7f7fu)) & 0x80808080u;  // bit 7: not zero
+  return (t >> 7) * 0xffu;
+}
+// The 8 pixels at flat position k0 (a multiple of 8) of an image; vec: one 16-byte load.
+__device__ __forceinline__ uint4 load_pixels8(const uint16_t *img, int k0, bool vec) {
+  if (vec) return *reinterpret_cast<const uint4 *>(img + k0);
+  uint32_t w[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    w[e] = (uint32_t)img[k0 + 2 * e] | ((uint32_t)img[k0 + 2 * e + 1] << 16);
+  return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Byte offset of the delta at flat position k of image i in the word-major layout read by
-// k_sparse: 32 consecutive images form a group, and within a group word w (4 deltas) of the 32
-// images is stored contiguously (128 bytes), so the 32 lanes of a warp reading the same word of
-// their images make one coalesced access whatever the word.
-__device__ __forceinline__ int64_t word_major_offset(int64_t i, int N, int k) {
-  const int64_t g = i >> 5, l = i & 31;
-  return ((g * (N * N / 4) + (k >> 2)) * 32 + l) * 4 + (k & 3);
-}
-
-// One warp per image.  interleave: 0 image-major deltas; 1 the layout of interleaved_offset (the
-// haystack of the dense kernel); 2 the layout of word_major_offset (the haystack of k_sparse).
-// row_sq (optional): per row, the sum of the squared (clamped) deltas, [n][N].
-// list (optional): encode images list[0 .. *list_count) of imgs as images 0, 1, ... (a compacted
-// subset, count read on the device; n is then an upper bound).
-__global__ void k_encode(const uint16_t *__restrict__ imgs, int64_t n, int N,
-                         int8_t *__restrict__ delta, int8_t *__restrict__ mask,
-                         int *__restrict__ wide_flag, int *__restrict__ wide_list,
-                         int *__restrict__ wide_count, int interleave, int *__restrict__ row_sq,
-                         const int *__restrict__ list = nullptr,
-                         const int *__restrict__ list_count = nullptr) {
+// Needle side of the CUDA-core forms, one warp per image, 256 pixels per pass (rows_of_8(N)):
+// image-major int8 deltas, byte masks of the non-zero ones and, with row_sq, the sum of each
+// row's squared (clamped) deltas, [n][N].
+__global__ void k_encode_needles(const uint16_t *__restrict__ imgs, int64_t n, int N,
+                                 int8_t *__restrict__ delta, int8_t *__restrict__ mask,
+                                 int *__restrict__ wide_flag, int *__restrict__ wide_list,
+                                 int *__restrict__ wide_count, int *__restrict__ row_sq) {
   const int lane = threadIdx.x & 31;
   const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int K = N * N;
-  if (list) n = *list_count < n ? *list_count : n;
-  // rows of a multiple of 32 positions: every pass of the warp lies in one row, so the row sums
-  // of squared (clamped) deltas come from one warp reduction per pass
-  const bool rows_by_pass = N % 32 == 0;
+  const int K = N * N, rl = N / 8;  // rl: lanes of a row (a power of two, at most 16)
+  const bool vec = aligned16(imgs);
   for (int64_t i = w; i < n; i += nw) {
-    const uint16_t *img = imgs + (list ? (int64_t)list[i] : i) * K;
-    int wide = 0, row_acc = 0;
-    for (int k = lane; k < K; k += 32) {
-      int r = k / N, c = k - r * N;
-      int d = delta_at(img, N, r, c);
-      wide |= (d > 127 || d < -127);
-      int dc = d > 127 ? 127 : (d < -127 ? -127 : d);
-      const int64_t off = interleave == 1   ? interleaved_offset(i, N, k)
-                          : interleave == 2 ? word_major_offset(i, N, k)
-                                            : i * K + k;
-      delta[off] = (int8_t)dc;
-      if (mask) mask[i * K + k] = (int8_t)(d != 0 ? -1 : 0);
-      if (row_sq && rows_by_pass) {
-        row_acc += (int)__reduce_add_sync(0xffffffffu, (unsigned)(dc * dc));
-        if (c - lane + 32 == N) {  // the row's last pass (uniform over the warp)
-          if (lane == 0) row_sq[i * N + r] = row_acc;
-          row_acc = 0;
-        }
+    const uint16_t *img = imgs + i * K;
+    int wide = 0;
+#pragma unroll 4
+    for (int base = 0; base < K; base += 256) {
+      const int k0 = base + lane * 8;
+      const bool in = k0 < K;
+      int d[8];
+      deltas8(in ? load_pixels8(img, k0, vec) : make_uint4(0, 0, 0, 0), lane, N, d);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) wide |= d[e] > 127 || d[e] < -127;
+      const uint2 a = make_uint2(pack_deltas(d[0], d[1], d[2], d[3]),
+                                 pack_deltas(d[4], d[5], d[6], d[7]));
+      if (in) {
+        *reinterpret_cast<uint2 *>(delta + i * K + k0) = a;
+        // from the deltas themselves: a wide delta is not zero
+        *reinterpret_cast<uint2 *>(mask + i * K + k0) =
+            make_uint2(nonzero_bytes(a.x), nonzero_bytes(a.y));
       }
-    }
-    if (row_sq && !rows_by_pass) {
-      for (int r = lane; r < N; r += 32) {
-        int sq = 0;
-        for (int c = 1; c < N; ++c) {
-          int d = delta_at(img, N, r, c);
-          d = d > 127 ? 127 : (d < -127 ? -127 : d);
-          sq += d * d;
-        }
-        row_sq[i * N + r] = sq;
+      if (row_sq) {
+        int sq = __dp4a((int)a.x, (int)a.x, __dp4a((int)a.y, (int)a.y, 0));
+        for (int k = 1; k < rl; k <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, k);
+        if (in && (lane & (rl - 1)) == 0) row_sq[i * N + k0 / N] = sq;
       }
     }
     wide = __any_sync(0xffffffffu, wide);
@@ -121,22 +110,115 @@ __global__ void k_encode(const uint16_t *__restrict__ imgs, int64_t n, int N,
   }
 }
 
-// Exact int64 distance of one pair, one warp.
+// Haystack side of the CUDA-core forms: int8 deltas of groups of 32 consecutive images, so that the
+// 32 lanes of a warp (one image each) read the same piece of their images with one contiguous
+// access.  Within a group the 32-bit words (4 deltas) of an image are cut into pieces of CW words,
+// piece-major: piece v of image l is at word (v * 32 + l) * CW.
+//   CW = min(4, N / 4)  k_dense: pieces of 16 bytes within a row (a warp reads 512 bytes)
+//   CW = 1              k_sparse: any word of the 32 images is one 128-byte line
+// list (optional): encode images list[0 .. *list_count) of imgs as images 0, 1, ... (a compacted
+// subset, count read on the device; n is then an upper bound).  Images past the last are zero.
+// One block per group; 256 pixels of its images at a time cross through shared memory, so that
+// both the reads (512 bytes of an image) and the writes are contiguous.  Writing from one warp
+// per image instead left 1 or 16 bytes in every 128-byte line (262,144 images of 64 x 64:
+// 2.2 ms with CW = 1, 1.5 ms per 90,000 with CW = 4).
+constexpr int kGroupWarps = 8;
+template <int CW>
+__global__ void __launch_bounds__(kGroupWarps * 32) k_encode_groups(
+    const uint16_t *__restrict__ imgs, int64_t n, int N, int8_t *__restrict__ delta,
+    int *__restrict__ wide_flag, int *__restrict__ wide_list, int *__restrict__ wide_count,
+    const int *__restrict__ list, const int *__restrict__ list_count) {
+  constexpr int kPerW = 32 / kGroupWarps;  // images of a warp
+  __shared__ uint32_t tile[64][33];        // [word of the 256 pixels][image]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int K = N * N;
+  if (list) n = *list_count < n ? *list_count : n;
+  const bool vec = aligned16(imgs);
+  for (int64_t g = blockIdx.x; g * 32 < n; g += gridDim.x) {
+    int wide[kPerW];
+    const uint16_t *img[kPerW];
+#pragma unroll
+    for (int q = 0; q < kPerW; ++q) {
+      const int64_t i = g * 32 + warp * kPerW + q;
+      wide[q] = 0;
+      img[q] = i < n ? imgs + (list ? (int64_t)list[i] : i) * K : nullptr;
+    }
+    uint32_t *out = reinterpret_cast<uint32_t *>(delta) + g * (int64_t)(K / 4) * 32;
+    for (int base = 0; base < K; base += 256) {
+      const int k0 = base + lane * 8;
+      uint4 px[kPerW];
+#pragma unroll
+      for (int q = 0; q < kPerW; ++q)
+        px[q] = k0 < K && img[q] ? load_pixels8(img[q], k0, vec) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int q = 0; q < kPerW; ++q) {
+        int d[8];
+        deltas8(px[q], lane, N, d);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) wide[q] |= d[e] > 127 || d[e] < -127;
+        tile[2 * lane][warp * kPerW + q] = pack_deltas(d[0], d[1], d[2], d[3]);
+        tile[2 * lane + 1][warp * kPerW + q] = pack_deltas(d[4], d[5], d[6], d[7]);
+      }
+      __syncthreads();
+      const int nv = min(64, (K - base) / 4) / CW;  // pieces of these pixels
+      for (int v = warp; v < nv; v += kGroupWarps) {
+        uint32_t *dst = out + ((int64_t)(base / 4 / CW + v) * 32 + lane) * CW;
+        if constexpr (CW == 4)
+          *reinterpret_cast<uint4 *>(dst) = make_uint4(tile[4 * v][lane], tile[4 * v + 1][lane],
+                                                       tile[4 * v + 2][lane], tile[4 * v + 3][lane]);
+        else if constexpr (CW == 2)
+          *reinterpret_cast<uint2 *>(dst) = make_uint2(tile[2 * v][lane], tile[2 * v + 1][lane]);
+        else
+          *dst = tile[v][lane];
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int q = 0; q < kPerW; ++q) {
+      const int any = __any_sync(0xffffffffu, wide[q]);
+      const int64_t i = g * 32 + warp * kPerW + q;
+      if (lane == 0 && i < n) {
+        wide_flag[i] = any;
+        if (any) wide_list[atomicAdd(wide_count, 1)] = (int)i;
+      }
+    }
+  }
+}
+
+// Exact int64 distance of one pair, one warp: 256 pixels per pass where both images can be read 8
+// at a time, else 32.
 __device__ int64_t warp_crss(const uint16_t *n, const uint16_t *h, int N) {
   const int lane = threadIdx.x & 31;
-  long long s = 0;
-  for (int k = lane; k < N * N; k += 32) {
-    int r = k / N, c = k - r * N;
-    if (c == 0) continue;
-    int a = delta_at(n, N, r, c);
-    if (a != 0) {
-      long long d = (long long)a - (long long)delta_at(h, N, r, c);
-      s += d * d;
+  const int K = N * N;
+  unsigned long long s = 0;
+  if (rows_of_8(N) && aligned16(n) && aligned16(h)) {
+#pragma unroll 4
+    for (int base = 0; base < K; base += 256) {
+      const int k0 = base + lane * 8;
+      const bool in = k0 < K;
+      int a[8], b[8];
+      deltas8(in ? load_pixels8(n, k0, true) : make_uint4(0, 0, 0, 0), lane, N, a);
+      deltas8(in ? load_pixels8(h, k0, true) : make_uint4(0, 0, 0, 0), lane, N, b);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const unsigned x = a[e] != 0 ? (unsigned)abs(a[e] - b[e]) : 0u;  // at most 131,070
+        s += (unsigned long long)x * x;
+      }
+    }
+  } else {
+    for (int k = lane; k < K; k += 32) {
+      int r = k / N, c = k - r * N;
+      if (c == 0) continue;
+      int a = delta_at(n, N, r, c);
+      if (a != 0) {
+        long long d = (long long)a - (long long)delta_at(h, N, r, c);
+        s += (unsigned long long)(d * d);
+      }
     }
   }
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
-  return __shfl_sync(0xffffffffu, s, 0);
+  return (int64_t)__shfl_sync(0xffffffffu, s, 0);
 }
 
 __global__ void k_true_distance(const SearchScene *__restrict__ tab, const int *__restrict__ qscene,
@@ -1056,12 +1138,27 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
       default: return launch_dense<128>(nd, nm, nrs, nexcl, Q, hd, hexcl, H, dt, nflags, rank, best, cnt, st, hcount, hmap, gate);
     }
   };
+  // the haystack of a single scene (or its images list[0 .. *count)) for k_dense, for k_sparse
+  const int group_blocks = (int)((H + 31) / 32 < 152 * 32 ? (H + 31) / 32 : 152 * 32);
+  auto encode_rows = [&](int8_t *out, int *flag, int *wlist, int *wcount, const int *list,
+                         const int *count) {
+    auto kern = N == 8 ? k_encode_groups<2> : k_encode_groups<4>;
+    kern<<<group_blocks, kGroupWarps * 32, 0, st>>>(scenes[0].haystack, H, N, out, flag, wlist,
+                                                    wcount, list, count);
+    count_launches(1);
+  };
+  auto encode_words = [&](int8_t *out, int *flag, int *wlist, int *wcount) {
+    k_encode_groups<1><<<group_blocks, kGroupWarps * 32, 0, st>>>(scenes[0].haystack, H, N, out,
+                                                                  flag, wlist, wcount, nullptr,
+                                                                  nullptr);
+    count_launches(1);
+  };
   if (tensor) {
     const SearchScene &s0 = scenes[0];
     if (mid) {
       // CUDA-core encode of every needle (the fp16-class ones are int8-class too)
-      k_encode<<<blocks_for(Q), 32 * wpb, 0, st>>>(s0.needles, Q, N, nd, nm, mid_nflag, mid_list,
-                                                   counts + 2, 0, nrs);
+      k_encode_needles<<<blocks_for(Q), 32 * wpb, 0, st>>>(s0.needles, Q, N, nd, nm, mid_nflag,
+                                                           mid_list, counts + 2, nrs);
       count_launches(1);
     }
     if (autom) {
@@ -1083,10 +1180,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
       // the haystack images outside the fp16 class, compacted in list order (list and count
       // from the tensor-core encode); narrow needles x those images on CUDA cores, and the
       // int64 kernel only for the compacted images outside the int8 class
-      k_encode<<<blocks_for(H), 32 * wpb, 0, st>>>(s0.haystack, H, N, hd, nullptr, mid_hflag,
-                                                   mid_list + Q, counts + 3, 1, nullptr, wh_list,
-                                                   counts + 1);
-      count_launches(1);
+      encode_rows(hd, mid_hflag, mid_list + Q, counts + 3, wh_list, counts + 1);
       // (AUTO: counts[5] = 0 when no needle is left for the tensor-core side)
       if ((e = run_dense(autom ? excl_dense : nwide, mid_hflag, counts + 1, wh_list,
                          autom ? counts + 5 : nullptr)) != cudaSuccess)
@@ -1099,9 +1193,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
     if (autom) {
       // the sparse-needle form for its needles against every int8-class image (the encode's list
       // of images outside int8 goes to wh_list, whose readers above precede it on the stream)
-      k_encode<<<blocks_for(H), 32 * wpb, 0, st>>>(s0.haystack, H, N, hword, nullptr, auto_hflag,
-                                                   wh_list, counts + 4, 2, nullptr);
-      count_launches(1);
+      encode_words(hword, auto_hflag, wh_list, counts + 4);
       if ((e = launch_sparse(sent, scount, excl_sparse, Q, hword, auto_hflag, H, N, dt, nflags,
                              rank, best, cnt, st)) != cudaSuccess)
         return e;
@@ -1116,22 +1208,20 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   } else if (dense) {
     // single scene: launch-wide indices are the scene's own
     const SearchScene &s0 = scenes[0];
-    k_encode<<<blocks_for(Q), 32 * wpb, 0, st>>>(s0.needles, Q, N, nd, nm, nwide, wn_list,
-                                                 counts + 0, 0, nrs);
-    k_encode<<<blocks_for(H), 32 * wpb, 0, st>>>(s0.haystack, H, N, hd, nullptr, hwide, wh_list,
-                                                 counts + 1, 1, nullptr);
-    count_launches(2);
+    k_encode_needles<<<blocks_for(Q), 32 * wpb, 0, st>>>(s0.needles, Q, N, nd, nm, nwide, wn_list,
+                                                         counts + 0, nrs);
+    count_launches(1);
+    encode_rows(hd, hwide, wh_list, counts + 1, nullptr, nullptr);
     if ((e = run_dense(nwide, hwide, nullptr, nullptr)) != cudaSuccess) return e;
     wide(0);
     wide(1);
   } else if (sparse) {
     const SearchScene &s0 = scenes[0];
-    k_encode<<<blocks_for(Q), 32 * wpb, 0, st>>>(s0.needles, Q, N, nd, nm, nwide, wn_list,
-                                                 counts + 0, 0, nullptr);
-    k_encode<<<blocks_for(H), 32 * wpb, 0, st>>>(s0.haystack, H, N, hd, nullptr, hwide, wh_list,
-                                                 counts + 1, 2, nullptr);
+    k_encode_needles<<<blocks_for(Q), 32 * wpb, 0, st>>>(s0.needles, Q, N, nd, nm, nwide, wn_list,
+                                                         counts + 0, nullptr);
+    encode_words(hd, hwide, wh_list, counts + 1);
     k_sparse_needles<<<blocks_for(Q), 32 * wpb, 0, st>>>(nd, nm, Q, N, sent, scount);
-    count_launches(3);
+    count_launches(2);
     if ((e = launch_sparse(sent, scount, nwide, Q, hd, hwide, H, N, dt, nflags, rank, best, cnt,
                            st)) != cudaSuccess)
       return e;

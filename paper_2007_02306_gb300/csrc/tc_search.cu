@@ -196,29 +196,52 @@ __global__ void k_tc_encode(const SearchScene *__restrict__ tab, const int *__re
                                       : sc.haystack + (i - sc.hoff) * K0;
     __half *row = op + i * (int64_t)(2 * K0);
     const int lim = needle_side ? kNarrowA : kNarrowB;
-    int wide = 0, a2 = 0, s1 = 0;  // needles: a2 = sum a^2; haystack: a2 = S2_j, s1 = S1_j
+    // needles: a2 = sum a^2; haystack: a2 = S2_j, s1 = S1_j (wrapped, and not used, for an image
+    // with a wide delta; its operand row is garbage that no result reads)
+    unsigned a2 = 0, s1 = 0;
+    int wide = 0;
     const bool write = needle_side ? !(skip_tile && skip_tile[i / kBM]) : hay_written;
-    for (int k0 = lane * 8; k0 < K0; k0 += 32 * 8) {
-      __align__(16) __half lo[8], hi[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int k = k0 + e;
-        const int r = k / N, c = k - r * N;
-        const int d = c == 0 ? 0 : (int)img[r * N + c] - (int)img[r * N + c - 1];
-        const bool nar = d >= -lim && d <= lim;
-        wide |= !nar;
-        const int dc = nar ? d : 0;
-        a2 += dc * dc;
-        if (needle_side) {
-          lo[e] = __int2half_rn(dc != 0 ? 1 : 0);
-          hi[e] = __int2half_rn(dc);
+    const bool vec = aligned16(img);
+#pragma unroll 4
+    for (int base = 0; base < K0; base += 256) {
+      const int k0 = base + lane * 8;
+      const bool in = k0 < K0;
+      int d[8];
+      uint4 px = make_uint4(0, 0, 0, 0);
+      if (in) {
+        if (vec) {
+          px = *reinterpret_cast<const uint4 *>(img + k0);
         } else {
-          s1 += dc < 0 ? -dc : dc;
-          lo[e] = __int2half_rn(dc * dc);
-          hi[e] = __int2half_rn(-2 * dc);
+          const uint16_t *q = img + k0;
+          px = make_uint4(q[0] | (uint32_t)q[1] << 16, q[2] | (uint32_t)q[3] << 16,
+                          q[4] | (uint32_t)q[5] << 16, q[6] | (uint32_t)q[7] << 16);
         }
       }
-      if (write) {
+      deltas8(px, lane, N, d);
+      __align__(16) __half2 lo[4], hi[4];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        wide |= d[e] < -lim || d[e] > lim;
+        a2 += (unsigned)d[e] * (unsigned)d[e];
+        if (!needle_side) s1 += (unsigned)abs(d[e]);
+      }
+      // |d| <= 127 as halves without conversions: 0x6600 + d are the bits of 1536 + d (0x6400 is
+      // 1024, steps of 1); differences, products and doubles of such integers are exact
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const uint32_t bits = __byte_perm((uint32_t)(0x6600 + d[2 * e]),
+                                          (uint32_t)(0x6600 + d[2 * e + 1]), 0x5410);
+        const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&bits),
+                                  __floats2half2_rn(1536.0f, 1536.0f));
+        if (needle_side) {
+          lo[e] = __hne2(h, __floats2half2_rn(0.0f, 0.0f));
+          hi[e] = h;
+        } else {
+          lo[e] = __hmul2(h, h);
+          hi[e] = __hmul2(h, __floats2half2_rn(-2.0f, -2.0f));
+        }
+      }
+      if (write && in) {
         *reinterpret_cast<int4 *>(row + k0) = *reinterpret_cast<int4 *>(lo);
         *reinterpret_cast<int4 *>(row + K0 + k0) = *reinterpret_cast<int4 *>(hi);
       }
@@ -233,7 +256,7 @@ __global__ void k_tc_encode(const SearchScene *__restrict__ tab, const int *__re
       if (!needle_side && (int64_t)a2 + 2ll * kNarrowA * s1 >= kExactSum) wide = 1;
       wide_flag[i] = wide;
       if (wide) wide_list[atomicAdd(wide_count, 1)] = (int)i;
-      if (asum) asum[i] = a2;
+      if (asum) asum[i] = (int)a2;
       if (valid_mask && !wide) atomicOr(&valid_mask[i >> 5], 1u << (i & 31));
     }
   }
