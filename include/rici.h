@@ -67,9 +67,11 @@ extern "C" {
                                    powers of two) for needles with every |delta| <= 127 and
                                    haystack images with every |delta| <= 45 and
                                    sum b^2 + 254 sum |b| < 2^24 (all partial sums exact in FP32);
-                                   single-scene calls run the other int8-class pairs on the dense
-                                   CUDA-core kernel, and pairs with |delta| > 127 (multi-scene
-                                   calls: any pair outside the fp16 class) in exact int64 */
+                                   single-scene calls take haystack images with |delta| <= 127 and
+                                   that sum in a second GEMM (b^2 split in two), run the other
+                                   int8-class pairs on the dense CUDA-core kernel, and pairs with
+                                   |delta| > 127 (multi-scene calls: any pair outside the fp16
+                                   class) in exact int64 */
 #define RICI_SEARCH_SPARSE 4    /* Listing 1 over each needle's non-zero delta words only (the
                                    positions where a != 0, Section 3.2), on CUDA cores: words
                                    heaviest first, early exit after every word; single-scene

@@ -191,9 +191,11 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
 
 // Tensor-core search (tc_search.cu): operand encoding + persistent tcgen05 GEMM with the rank /
 // top-1 epilogue for narrow x narrow pairs of every scene.  Fills nwide/hwide and the wide
-// lists/counts (launch-wide indices).
+// lists/counts (launch-wide indices).  With split_haystack (single scene): the haystack images outside
+// the fp16 class that only exceed its limit on one delta are ranked too, by a second GEMM with a
+// split square, and left_list / *left_count (zeroed before) receive the other ones.
 bool tc_supported(int N);
-int64_t tc_workspace_bytes(int64_t Q, int64_t H, int N);
+int64_t tc_workspace_bytes(int64_t Q, int64_t H, int N, bool single_scene);
 cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, const int *qscene,
                                       const int *hscene, int64_t Qtot, int64_t Htot,
                                       int64_t tiles_total, int N, void *ws, int *nwide, int *hwide,
@@ -202,7 +204,9 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
                                       unsigned long long *best, int *status, int test_withhold,
                                       cudaStream_t st, const int *skip_needle = nullptr,
                                       const int *skip_tile = nullptr,
-                                      const int *any_tile = nullptr);
+                                      const int *any_tile = nullptr,
+                                      const uint16_t *split_haystack = nullptr,
+                                      int *left_list = nullptr, int *left_count = nullptr);
 
 // Integer tensor-core search (i8_search.cu): int8 operand encoding + mma.sync s8 GEMM with the
 // rank / top-1 epilogue for int8-narrow x int8-narrow pairs of every scene (the tiles of the

@@ -1024,11 +1024,12 @@ int64_t search_batch_workspace_bytes(int num_scenes, int64_t Q, int64_t H, int N
   c.take<int>(Q);                        // ranks
   c.take<int4>(sparse || autom ? Q * (K / 4) : 0);  // sparse needle entries (a slab per needle)
   c.take<int>(sparse || autom ? Q : 0);  // sparse entries per needle
-  c.take<char>(tensor ? tc_workspace_bytes(Q, H, N) : 0);
+  c.take<char>(tensor ? tc_workspace_bytes(Q, H, N, num_scenes == 1) : 0);
   c.take<char>(i8 ? i8_workspace_bytes(Q, H, N) : 0);
   c.take<int>(mid ? Q : 0);      // int8 class flags of the needles (dense middle pass)
   c.take<int>(mid ? H : 0);      // int8 class flags of the compacted haystack images
   c.take<int>(mid ? Q + H : 0);  // lists written by its encodes
+  c.take<int>(mid ? H : 0);      // images of neither tensor-core class
   c.take<int8_t>(autom ? (H + 31) / 32 * 32 * K : 0);  // word-major haystack of the sparse form
   c.take<int>(autom ? H : 0);     // its int8 class flags
   c.take<int>(autom ? 3 * Q : 0);  // per-needle choice and the two exclusions
@@ -1059,9 +1060,9 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
                       b.num_scenes == 1;
   const bool sparse = packed && mode == RICI_SEARCH_SPARSE;
   const bool dense = packed && !sparse;
-  // single-scene tensor-core calls: pairs of a narrow needle with a haystack image outside the
-  // fp16 class but inside int8 (32 < |delta| <= 127) run on the dense CUDA-core kernel over a
-  // compacted haystack instead of the int64 kernel
+  // single-scene tensor-core calls: pairs of a narrow needle with a haystack image outside both
+  // tensor-core classes but inside int8 run on the dense CUDA-core kernel over a compacted haystack
+  // instead of the int64 kernel
   const bool mid = tensor && b.num_scenes == 1 && dense_supported(N);
   Carver c(ws);
   SearchScene *tab = c.take<SearchScene>(b.num_scenes);
@@ -1083,11 +1084,12 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   int *rank = c.take<int>(Q);
   int4 *sent = c.take<int4>(sparse || autom ? Q * (K / 4) : 0);
   int *scount = c.take<int>(sparse || autom ? Q : 0);
-  char *tc_ws = tensor ? c.take<char>(tc_workspace_bytes(Q, H, N)) : nullptr;
+  char *tc_ws = tensor ? c.take<char>(tc_workspace_bytes(Q, H, N, b.num_scenes == 1)) : nullptr;
   char *i8_ws = i8 ? c.take<char>(i8_workspace_bytes(Q, H, N)) : nullptr;
   int *mid_nflag = c.take<int>(mid ? Q : 0);
   int *mid_hflag = c.take<int>(mid ? H : 0);
   int *mid_list = c.take<int>(mid ? Q + H : 0);
+  int *left_list = c.take<int>(mid ? H : 0);
   int8_t *hword = c.take<int8_t>(autom ? (H + 31) / 32 * 32 * K : 0);
   int *auto_hflag = c.take<int>(autom ? H : 0);
   int *auto_n = c.take<int>(autom ? 3 * Q : 0);
@@ -1121,9 +1123,11 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   if ((e = cudaFuncSetAttribute(k_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)wide_smem)) != cudaSuccess)
     return e;
-  auto wide = [&](int pass, const int *sub_list = nullptr, const int *sub_count = nullptr) {
+  auto wide = [&](int pass, const int *sub_list = nullptr, const int *sub_count = nullptr,
+                  const int *list = nullptr) {
     k_wide<<<152 * 8, kWideThreads, wide_smem, st>>>(tab, qscene, hscene, Q, b.Hmax, N, pass,
-                                                   nwide, wn_list, counts + 0, wh_list,
+                                                   nwide, wn_list, counts + 0,
+                                                   list ? list : wh_list,
                                                    counts + 1, dt, nflags, rank, best, t1flag, cnt,
                                                    sub_list, sub_count);
     count_launches(1);
@@ -1173,20 +1177,22 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
     if ((e = launch_tc_encode_and_rank(tab, b.num_scenes, qscene, hscene, Q, H, b.tiles_total, N,
                                        tc_ws, nwide, hwide, wn_list, wh_list, counts, nflags, dt,
                                        rank, best, b.status, withhold, st, sparse_of,
-                                       autom ? skip_tile : nullptr, counts + 5)) != cudaSuccess)
+                                       autom ? skip_tile : nullptr, counts + 5,
+                                       mid ? s0.haystack : nullptr, left_list, counts + 6)) !=
+        cudaSuccess)
       return e;
     wide(0);  // needles outside the fp16 class against the whole haystack (int64)
     if (mid) {
-      // the haystack images outside the fp16 class, compacted in list order (list and count
-      // from the tensor-core encode); narrow needles x those images on CUDA cores, and the
+      // the haystack images of neither tensor-core class, compacted in list order (list and
+      // count from the tensor-core encodes); narrow needles x those images on CUDA cores, and the
       // int64 kernel only for the compacted images outside the int8 class
-      encode_rows(hd, mid_hflag, mid_list + Q, counts + 3, wh_list, counts + 1);
+      encode_rows(hd, mid_hflag, mid_list + Q, counts + 3, left_list, counts + 6);
       // (AUTO: counts[5] = 0 when no needle is left for the tensor-core side)
-      if ((e = run_dense(autom ? excl_dense : nwide, mid_hflag, counts + 1, wh_list,
+      if ((e = run_dense(autom ? excl_dense : nwide, mid_hflag, counts + 6, left_list,
                          autom ? counts + 5 : nullptr)) != cudaSuccess)
         return e;
       // the compacted encode listed its images outside the int8 class (compact indices)
-      wide(1, mid_list + Q, counts + 3);
+      wide(1, mid_list + Q, counts + 3, left_list);
     } else {
       wide(1);
     }

@@ -12,8 +12,17 @@
 // b^2 <= 2025 < 2^11, |2b| <= 90), every product is an exact integer, and every partial sum of
 // any subset of the products m_ik b_jk^2 - 2 a_ik b_jk is an integer of magnitude at most
 // S2_j + 2 * 127 * S1_j < 2^24, so the FP32 accumulation in TMEM is exact in any order.  Pairs
-// with a side outside the class go to the CUDA-core kernels (dense int8 or exact int64).  The rank test S_ij < d(i,match_i) - A_i, and the top-1 key
-// (A_i + S_ij, j), are evaluated in the GEMM epilogue; S is never written to memory.
+// with a side outside the class go to the CUDA-core kernels (dense int8 or exact int64).  The rank
+// test S_ij < d(i,match_i) - A_i, and the top-1 key (A_i + S_ij, j), are evaluated in the GEMM
+// epilogue; S is never written to memory.
+//
+// Split-square class (single-scene calls): haystack images with some 45 < |b| <= 127 and the same
+// bound S2_j + 254 S1_j < 2^24.  b^2 = 128 q + r with r < 128, q <= 126, and 128 q is exact in fp16
+// (7 significant bits), so S = [m | a | m] x [r | -2b | 128 q]^T with K = 3 N^2 has the same exact
+// partial sums; the third block of the needle row is its first one again, so only the haystack rows
+// are new.  On the 5M-triangle scene 7 % of the images are in this class: 1.5 times a fp16-class
+// pair's work on the tensor cores, against CUDA cores at a ninth of that rate (8,192 needles x
+// 262,144 of its images: 35.7 ms with those pairs on k_dense, 24.5 ms here).
 //
 // Kernel structure (one CTA per SM, persistent over 128 x 256 output tiles):
 //   warp 0: TMA producer (128B-swizzled K-major tiles, 4-stage mbarrier pipeline)
@@ -262,6 +271,83 @@ __global__ void k_tc_encode(const SearchScene *__restrict__ tab, const int *__re
   }
 }
 
+// The haystack images outside the fp16 class (list[0 .. *count)), one warp each: those of the
+// split-square class get a row [r | -2b | 128 q] of op (at most cap rows) and an entry of map, the
+// others an entry of left.
+__global__ void k_tc_encode_split(const uint16_t *__restrict__ imgs, int N,
+                                  const int *__restrict__ list, const int *__restrict__ count,
+                                  int cap, __half *__restrict__ op, int *__restrict__ map,
+                                  int *__restrict__ map_count, int *__restrict__ left,
+                                  int *__restrict__ left_count, const int *__restrict__ any_tile) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int64_t n = *count;
+  const int K0 = N * N;
+  const bool wanted = !any_tile || *any_tile != 0;
+  for (int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; p < n; p += nw) {
+    const int j = list[p];
+    const uint16_t *img = imgs + (int64_t)j * K0;
+    const bool vec = aligned16(img);
+    auto pixels = [&](int k0) {
+      if (k0 >= K0) return make_uint4(0, 0, 0, 0);
+      if (vec) return *reinterpret_cast<const uint4 *>(img + k0);
+      const uint16_t *q = img + k0;
+      return make_uint4(q[0] | (uint32_t)q[1] << 16, q[2] | (uint32_t)q[3] << 16,
+                        q[4] | (uint32_t)q[5] << 16, q[6] | (uint32_t)q[7] << 16);
+    };
+    unsigned s2 = 0, s1 = 0;
+    int wide = !wanted;
+    for (int base = 0; base < K0; base += 256) {
+      int d[8];
+      deltas8(pixels(base + lane * 8), lane, N, d);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        wide |= d[e] < -kNarrowA || d[e] > kNarrowA;
+        s2 += (unsigned)d[e] * (unsigned)d[e];
+        s1 += (unsigned)abs(d[e]);
+      }
+    }
+    wide = __any_sync(0xffffffffu, wide);
+    s2 = __reduce_add_sync(0xffffffffu, s2);
+    s1 = __reduce_add_sync(0xffffffffu, s1);
+    if ((int64_t)s2 + 2ll * kNarrowA * s1 >= kExactSum) wide = 1;  // (s2, s1 exact when not wide)
+    int at = cap;
+    if (lane == 0) {
+      if (!wide) at = atomicAdd(map_count, 1);
+      if (at < cap) map[at] = j;
+      else left[atomicAdd(left_count, 1)] = j;
+    }
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (at >= cap) continue;
+    __half *row = op + (int64_t)at * (3 * K0);
+    for (int base = 0; base < K0; base += 256) {
+      const int k0 = base + lane * 8;
+      int d[8];
+      deltas8(pixels(k0), lane, N, d);
+      __align__(16) __half r[8], b[8], q[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int sq = d[e] * d[e];
+        r[e] = __int2half_rn(sq & 127);
+        b[e] = __int2half_rn(-2 * d[e]);
+        q[e] = __int2half_rn(sq & ~127);
+      }
+      if (k0 < K0) {
+        *reinterpret_cast<int4 *>(row + k0) = *reinterpret_cast<int4 *>(r);
+        *reinterpret_cast<int4 *>(row + K0 + k0) = *reinterpret_cast<int4 *>(b);
+        *reinterpret_cast<int4 *>(row + 2 * K0 + k0) = *reinterpret_cast<int4 *>(q);
+      }
+    }
+  }
+}
+
+// Rows kept for split-square images: an eighth of the haystack, in whole tiles (3 KB of workspace per
+// image at N = 64; images beyond that go to the CUDA cores).
+int split_capacity(int64_t H) {
+  const int64_t want = (H / 8 + kBN) / kBN * kBN;
+  return (int)(want < H ? want : H);
+}
+
 // ---------------------------------------------------------------- GEMM + rank epilogue (S3, S5)
 
 struct TcArgs {
@@ -273,7 +359,7 @@ struct TcArgs {
   const int *nflags;              // per-needle state (0 = searchable)
   const int *asum;                // A_i
   const int64_t *dtrue;           // d(i, match_i)
-  const uint32_t *hvalid;         // bit j: haystack image j is narrow
+  const uint32_t *hvalid;         // bit j: haystack image j is narrow (null: every one is)
   int *rank;
   unsigned long long *best;
   int *status;
@@ -282,6 +368,10 @@ struct TcArgs {
   const int *skip_needle;   // optional: 1 = this needle is ranked by another form
   const int *skip_tile;     // optional (single scene): 1 = needle tile m has no needle here
   const int *any_tile;      // with skip_tile: 0 = every tile is skipped (the grid returns at once)
+  int ka_blocks;            // k-blocks of a needle row (block kb of K reads block kb % ka_blocks)
+  const int *hcount;        // optional (single scene): the haystack is min(*hcount, hcap) rows
+  int hcap;
+  const int *hmap;          // optional: column j is haystack image hmap[j] of the caller
 };
 
 // Tiles and their order: search_tile_of (common.cuh).
@@ -306,10 +396,21 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
   int *abort_flag = reinterpret_cast<int *>(tmem_slot + 1);
 
+  __shared__ SearchScene counted;  // hcount: the table entry with that many haystack rows
   // nothing to rank: return before any barrier, TMEM or TMA work (uniform over the grid)
   if (a.any_tile && *a.any_tile == 0) return;
+  int64_t tiles = a.tiles;
+  const SearchScene *tab = a.tab;
+  if (a.hcount) {
+    SearchScene sc = a.tab[0];
+    sc.H = *a.hcount < a.hcap ? *a.hcount : a.hcap;
+    sc.tiles_n = (int)((sc.H + kBN - 1) / kBN);
+    tiles = (int64_t)sc.tiles_m * sc.tiles_n;
+    if (threadIdx.x == 0) counted = sc;
+    tab = &counted;
+  }
+  if (blockIdx.x >= tiles) return;  // (uniform over the block)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t tiles = a.tiles;
   const int kblocks = a.KT / kBK;
 
   if (threadIdx.x == 0) {
@@ -342,7 +443,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       uint32_t it = 0;
       bool ok = true;
       for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-        const TcTile tt = tile_of(a.tab, a.num_scenes, t, a.group_m);
+        const TcTile tt = tile_of(tab, a.num_scenes, t, a.group_m);
         if (a.skip_tile && a.skip_tile[tt.m]) continue;  // every role skips the same tiles
         const int ya = (int)(tt.qbeg + tt.m * kBM), yb = (int)(tt.hbeg + tt.n * kBN);
         for (int kb = 0; kb < kblocks; ++kb, ++it) {
@@ -353,7 +454,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           }
           if (a.withhold_first_load && blockIdx.x == 0 && it == 0) continue;
           mbar_arrive_expect_tx(&full[s], kStageA + kStageB);
-          tma_load_2d(sA + s * kStageA, &map_a, &full[s], kb * kBK, ya);
+          tma_load_2d(sA + s * kStageA, &map_a, &full[s],
+                      (kb < a.ka_blocks ? kb : kb - a.ka_blocks) * kBK, ya);
           tma_load_2d(sB + s * kStageB, &map_b, &full[s], kb * kBK, yb);
         }
       }
@@ -371,7 +473,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       uint32_t it = 0, lt = 0;
       bool ok = true;
       for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-        if (a.skip_tile && a.skip_tile[tile_of(a.tab, a.num_scenes, t, a.group_m).m]) continue;
+        if (a.skip_tile && a.skip_tile[tile_of(tab, a.num_scenes, t, a.group_m).m]) continue;
         const uint32_t buf = lt & 1, use = lt >> 1;
         ++lt;  // local count of processed tiles (selects the accumulator buffer)
         if (!mbar_wait(&tempty[buf], (use & 1) ^ 1, a.status, abort_flag)) break;
@@ -405,7 +507,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int row = quarter * 32 + lane;
     uint32_t lt = 0;
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-      const TcTile tt = tile_of(a.tab, a.num_scenes, t, a.group_m);
+      const TcTile tt = tile_of(tab, a.num_scenes, t, a.group_m);
       if (a.skip_tile && a.skip_tile[tt.m]) continue;
       const uint32_t buf = lt & 1, use = lt >> 1;
       ++lt;
@@ -436,9 +538,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         uint32_t vm = 0;  // bit e: column j0 + e is a narrow haystack image of this scene
         if (row_ok && j0 < tt.H) {
           const int64_t g0 = tt.hbeg + j0;   // launch-wide index (any alignment)
-          const uint32_t lo = a.hvalid[g0 >> 5], hi = a.hvalid[(g0 >> 5) + 1];
-          const int sh = (int)(g0 & 31);
-          vm = sh ? (lo >> sh) | (hi << (32 - sh)) : lo;
+          vm = 0xffffffffu;
+          if (a.hvalid) {
+            const uint32_t lo = a.hvalid[g0 >> 5], hi = a.hvalid[(g0 >> 5) + 1];
+            const int sh = (int)(g0 & 31);
+            vm = sh ? (lo >> sh) | (hi << (32 - sh)) : lo;
+          }
           const int64_t rem = tt.H - j0;
           if (rem < 32) vm &= (1u << rem) - 1u;
         }
@@ -449,7 +554,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           cnt += (ok && sv < thr);
           if (ok && sv <= thr) {
             const unsigned long long dist = (unsigned long long)(asum + (int64_t)sv);
-            const unsigned long long key = (dist << 32) | (unsigned long long)(uint32_t)(j0 + e);
+            const uint32_t j = a.hmap ? (uint32_t)a.hmap[j0 + e] : (uint32_t)(j0 + e);
+            const unsigned long long key = (dist << 32) | (unsigned long long)j;
             bestk = key < bestk ? key : bestk;
           }
         }
@@ -501,13 +607,16 @@ cudaError_t encode_map(CUtensorMap *map, const void *base, int64_t rows, int KT,
 
 bool tc_supported(int N) { return N == 8 || N == 16 || N == 32 || N == 64 || N == 128; }
 
-int64_t tc_workspace_bytes(int64_t Q, int64_t H, int N) {
+int64_t tc_workspace_bytes(int64_t Q, int64_t H, int N, bool single_scene) {
   const int64_t KT = 2ll * N * N;
+  const int cap = single_scene ? split_capacity(H) : 0;
   Carver c(nullptr);
   c.take<__half>(Q * KT);
   c.take<__half>(H * KT);
   c.take<int>(Q);                 // A_i
   c.take<uint32_t>((H + 31) / 32 + 2);
+  c.take<__half>(cap * (KT / 2 * 3));  // split-square rows
+  c.take<int>(cap);                    // their images
   return c.off + 256;
 }
 
@@ -518,13 +627,19 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
                                       const int *nflags, const int64_t *dtrue, int *rank,
                                       unsigned long long *best, int *status, int test_withhold,
                                       cudaStream_t st, const int *skip_needle,
-                                      const int *skip_tile, const int *any_tile) {
+                                      const int *skip_tile, const int *any_tile,
+                                      const uint16_t *split_haystack, int *left_list,
+                                      int *left_count) {
   const int64_t KT = 2ll * N * N;
+  const int cap = num_scenes == 1 ? split_capacity(H) : 0;
   Carver c(ws);
   __half *opa = c.take<__half>(Q * KT);
   __half *opb = c.take<__half>(H * KT);
   int *asum = c.take<int>(Q);
   uint32_t *hvalid = c.take<uint32_t>((H + 31) / 32 + 2);
+  __half *ops = c.take<__half>(cap * (KT / 2 * 3));
+  int *smap = c.take<int>(cap);
+  int *const scount = counts + 7;  // their number (zeroed by the caller with the other counts)
   cudaError_t e;
   if ((e = cudaMemsetAsync(hvalid, 0, sizeof(uint32_t) * ((H + 31) / 32 + 2), st)) != cudaSuccess)
     return e;
@@ -532,11 +647,18 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
     int64_t b = (warps + 7) / 8;
     return (int)(b < 152 * 64 ? (b > 0 ? b : 1) : 152 * 64);
   };
+  const int *any = skip_tile ? any_tile : nullptr;
   k_tc_encode<<<blocks_for(Q), 256, 0, st>>>(tab, qscene, Q, N, 1, opa, nwide, wn_list, counts + 0,
                                              asum, nullptr, skip_tile, nullptr);
   k_tc_encode<<<blocks_for(H), 256, 0, st>>>(tab, hscene, H, N, 0, opb, hwide, wh_list, counts + 1,
-                                             nullptr, hvalid, nullptr, skip_tile ? any_tile : nullptr);
+                                             nullptr, hvalid, nullptr, any);
   count_launches(2);
+  if (split_haystack) {
+    k_tc_encode_split<<<blocks_for(cap), 256, 0, st>>>(split_haystack, N, wh_list, counts + 1, cap,
+                                                       ops, smap, scount, left_list, left_count,
+                                                       any);
+    count_launches(1);
+  }
   if (tiles_total == 0) return cudaGetLastError();
   CUtensorMap ma, mb;
   if ((e = encode_map(&ma, opa, Q, (int)KT, kBM)) != cudaSuccess) return e;
@@ -558,7 +680,11 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
   a.group_m = current_tuning().tc_group_m;
   a.skip_needle = skip_needle;
   a.skip_tile = skip_tile;
-  a.any_tile = skip_tile ? any_tile : nullptr;
+  a.any_tile = any;
+  a.ka_blocks = (int)(KT / kBK);
+  a.hcount = nullptr;
+  a.hcap = cap;
+  a.hmap = nullptr;
   const size_t smem = 1024 + kStages * (kStageA + kStageB) + 256;
   if ((e = cudaFuncSetAttribute(k_tc_rank, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem)) != cudaSuccess)
@@ -569,6 +695,17 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
   const int grid = (int)(tiles_total < sms ? tiles_total : sms);
   k_tc_rank<<<grid, kTcThreads, smem, st>>>(ma, mb, a);
   count_launches(1);
+  if (split_haystack) {
+    // the needles' tiles against the compacted split-square images (count on the device)
+    if ((e = encode_map(&mb, ops, cap, (int)(KT / 2 * 3), kBN)) != cudaSuccess) return e;
+    a.KT = (int)(KT / 2 * 3);
+    a.hcount = scount;
+    a.hvalid = nullptr;
+    a.hmap = smap;
+    a.withhold_first_load = 0;
+    k_tc_rank<<<grid, kTcThreads, smem, st>>>(ma, mb, a);
+    count_launches(1);
+  }
   return cudaGetLastError();
 }
 
