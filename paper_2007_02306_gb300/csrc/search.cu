@@ -924,6 +924,73 @@ __global__ void k_distances(const uint16_t *__restrict__ nimg, int64_t Q,
   }
 }
 
+// A whole small search of one scene in one launch: block i ranks needle i, one warp per pair, every
+// distance exact in int64 (so no classes, lists or fallbacks).
+constexpr int kSmallWarps = 8;
+__global__ void __launch_bounds__(kSmallWarps * 32) k_search_small(SearchScene sc, int N,
+                                                                   int64_t *__restrict__ distances,
+                                                                   int *status) {
+  __shared__ int64_t dt_s;
+  __shared__ int cnt_s[kSmallWarps];
+  __shared__ int64_t bd_s[kSmallWarps], bj_s[kSmallWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t K = (int64_t)N * N, i = blockIdx.x;
+  const uint16_t *needle = sc.needles + i * K;
+  const int64_t m = sc.match ? sc.match[i] : i;
+  const bool valid = m >= 0 && m < sc.H;
+  if (warp == 0) {
+    const int64_t d = valid ? warp_crss(needle, sc.haystack + m * K, N) : -1;
+    if (lane == 0) {
+      dt_s = d;
+      if (!valid) set_status(status, RICI_ERR_INDEX_OUT_OF_RANGE);
+    }
+  }
+  __syncthreads();
+  const int64_t dt = dt_s;
+  int cnt = 0;
+  int64_t bd = INT64_MAX, bj = -1;
+  if (valid || distances) {
+    for (int64_t j = warp; j < sc.H; j += kSmallWarps) {
+      const int64_t d = warp_crss(needle, sc.haystack + j * K, N);
+      cnt += d < dt;
+      if (d < bd) {  // j ascends: the smallest index of a minimum stays
+        bd = d;
+        bj = j;
+      }
+      if (distances && lane == 0) distances[i * sc.H + j] = d;
+    }
+  }
+  if (lane == 0) {
+    cnt_s[warp] = cnt;
+    bd_s[warp] = bd;
+    bj_s[warp] = bj;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kSmallWarps; ++w) {
+      cnt += cnt_s[w];
+      if (bj_s[w] >= 0 && (bd_s[w] < bd || (bd_s[w] == bd && bj_s[w] < bj))) {
+        bd = bd_s[w];
+        bj = bj_s[w];
+      }
+    }
+    sc.rank[i] = valid ? cnt : -1;
+    if (sc.dtrue) sc.dtrue[i] = dt;
+    if (sc.top1) sc.top1[i] = valid ? (int32_t)bj : -1;
+  }
+}
+
+// Whether a call takes k_search_small: the forms that leave the choice to the library (DEFAULT,
+// AUTO), no work counters, and so little work that launches decide: at most 2^19 pixel pairs per
+// block and 2^28 in all.  162 x 162 images of 32 x 32 with the distance matrix: 114 us in the
+// general sequence of 19 launches, 35 us here (most of it the call's host side); at the limits the
+// kernel takes as long as that sequence.
+bool small_search(const SearchBatch &b) {
+  const int64_t K = (int64_t)b.N * b.N;
+  return (b.mode == RICI_SEARCH_DEFAULT || b.mode == RICI_SEARCH_AUTO) && b.num_scenes == 1 &&
+         !b.counters && b.Htot * K <= (1 << 19) && b.Qtot * b.Htot * K <= (1 << 28);
+}
+
 bool dense_supported(int N) { return N == 8 || N == 16 || N == 32 || N == 64 || N == 128; }
 
 template <int N>
@@ -1047,6 +1114,11 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   const int N = b.N;
   const int64_t K = (int64_t)N * N;
   if (Q == 0) return cudaSuccess;
+  if (small_search(b)) {
+    k_search_small<<<(unsigned)Q, kSmallWarps * 32, 0, st>>>(scenes[0], N, out_distances, b.status);
+    count_launches(1);
+    return cudaGetLastError();
+  }
   const int withhold = (b.mode & RICI_SEARCH_TEST_WITHHOLD_LOAD) ? 1 : 0;
   const int mode = b.mode & 0xff;
   // RICI_SEARCH_AUTO (single scene): each needle ranked by the fp16 tensor cores or by the
