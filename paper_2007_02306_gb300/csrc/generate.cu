@@ -182,6 +182,24 @@ __global__ void k_tri_bbox(const GenScene *__restrict__ tab, int ns, int64_t nt_
   }
 }
 
+// Morton bin of a bounding-sphere centre on a 2^L grid over the box bb (ints of float_order) of its
+// scene's centres, 8^L <= nbuckets.
+__device__ __forceinline__ uint32_t morton_bin(const TriSphere &s, const int *bb, uint32_t nbuckets) {
+  const float lo[3] = {order_float(bb[0]), order_float(bb[1]), order_float(bb[2])};
+  const float ext = fmaxf(fmaxf(order_float(bb[3]) - lo[0], order_float(bb[4]) - lo[1]),
+                          order_float(bb[5]) - lo[2]);
+  const int L = (31 - __clz(nbuckets)) / 3;
+  const float top = (float)((1 << L) - 1);
+  const float scale = (ext > 0.0f && ext < 1e30f) ? (float)(1 << L) / ext : 0.0f;
+  const float c[3] = {s.cx, s.cy, s.cz};
+  uint32_t q[3];
+  for (int k = 0; k < 3; ++k) {
+    const float f = scale > 0.0f ? floorf((c[k] - lo[k]) * scale) : 0.0f;
+    q[k] = (uint32_t)fminf(fmaxf(f, 0.0f), top);
+  }
+  return spread3(q[0]) | (spread3(q[1]) << 1) | (spread3(q[2]) << 2);
+}
+
 // Bins every triangle by its bounding sphere.  With bbox == nullptr (clutter measure, spin
 // images): a hashed uniform grid of cell edge 1 / inv_cell, wide triangles in the scene's big
 // list.  Otherwise (generation): every triangle by the Morton code of its centre on a 2^L grid
@@ -216,20 +234,7 @@ __global__ void k_tri_bin(const GenScene *__restrict__ tab, int ns, int64_t nt_t
     TriSphere s = tri_sphere(v);
     uint32_t b = sc.nbuckets;  // the scene's big list
     if (bbox) {
-      const int *bb = bbox + 8 * (int64_t)scene_of_tri(tab, ns, t);
-      const float lo[3] = {order_float(bb[0]), order_float(bb[1]), order_float(bb[2])};
-      const float ext = fmaxf(fmaxf(order_float(bb[3]) - lo[0], order_float(bb[4]) - lo[1]),
-                              order_float(bb[5]) - lo[2]);
-      const int L = (31 - __clz(sc.nbuckets)) / 3;
-      const float top = (float)((1 << L) - 1);
-      const float scale = (ext > 0.0f && ext < 1e30f) ? (float)(1 << L) / ext : 0.0f;
-      const float c[3] = {s.cx, s.cy, s.cz};
-      uint32_t q[3];
-      for (int k = 0; k < 3; ++k) {
-        const float f = scale > 0.0f ? floorf((c[k] - lo[k]) * scale) : 0.0f;
-        q[k] = (uint32_t)fminf(fmaxf(f, 0.0f), top);
-      }
-      b = spread3(q[0]) | (spread3(q[1]) << 1) | (spread3(q[2]) << 2);
+      b = morton_bin(s, bbox + 8 * (int64_t)scene_of_tri(tab, ns, t), sc.nbuckets);
     } else {
       const float lim = kCellClamp - 4.0f;
       bool big = s.r > g.r_big || !(fabsf(s.cx * g.inv_cell) < lim) ||
@@ -423,6 +428,138 @@ __global__ void k_scan_final(const int *__restrict__ in, int64_t n, const int *_
     run += v[k];
   }
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = partials[gridDim.x];
+}
+
+// ------------------------------------------------------------------ small meshes
+
+// The whole preparation of one small scene in one block: table entry, box of centres, Morton bins,
+// scan, sorted records, bounding spheres (the steps of k_tri_bbox .. k_chunk_spheres, with the
+// bins in shared memory).  Nine dependent launches of a few microseconds each cost more than the
+// work of up to kSmallTris triangles: 162 images of a 320-triangle mesh 62 us with them, 37 us
+// with this launch and the generation's (most of it the call's host side).
+constexpr int kSmallTris = 8192;
+constexpr int kSmallBins = 4096;  // 8^L bins in use: L <= 4 for up to 2^14 buckets
+__global__ void __launch_bounds__(1024) k_sort_small(GenScene sc, GenScene *__restrict__ tab,
+                                                     uint32_t *__restrict__ tb,
+                                                     int *__restrict__ ts,
+                                                     int *__restrict__ starts,
+                                                     float4 *rec, float4 *__restrict__ chk,
+                                                     float4 *__restrict__ grp, int *status) {
+  __shared__ int bins[kSmallBins];
+  __shared__ int bb[6];
+  __shared__ int ws[32];
+  __shared__ int tot;
+  __shared__ float4 cs[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nt = (int)sc.nt;
+  for (int b = tid; b < kSmallBins; b += 1024) bins[b] = 0;
+  if (tid < 6) bb[tid] = tid < 3 ? 0x7fffffff : (int)0x80000000;
+  if (tid == 0) *tab = sc;
+  __syncthreads();
+  // reads a triangle; false when it is skipped (`report`: its status bits are raised)
+  auto read = [&](int t, int (&id)[3], float (&v)[9], bool report) -> bool {
+    for (int k = 0; k < 3; ++k) id[k] = sc.tris[3 * (int64_t)t + k];
+    if (id[0] < 0 || id[0] >= sc.nv || id[1] < 0 || id[1] >= sc.nv || id[2] < 0 || id[2] >= sc.nv) {
+      if (report) set_status(status, RICI_ERR_INDEX_OUT_OF_RANGE);
+      return false;
+    }
+    bool fin = true;
+    for (int k = 0; k < 3; ++k)
+      for (int d = 0; d < 3; ++d) {
+        v[3 * k + d] = sc.V[3 * (int64_t)id[k] + d];
+        fin = fin && isfinite(v[3 * k + d]);
+      }
+    if (!fin && report) set_status(status, RICI_ERR_NONFINITE_INPUT);
+    return fin;
+  };
+  float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+  for (int t = tid; t < nt; t += 1024) {
+    int id[3];
+    float v[9];
+    if (!read(t, id, v, true)) continue;
+    const TriSphere s = tri_sphere(v);
+    const float c[3] = {s.cx, s.cy, s.cz};
+    for (int k = 0; k < 3; ++k) {
+      lo[k] = fminf(lo[k], c[k]);
+      hi[k] = fmaxf(hi[k], c[k]);
+    }
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], d));
+      hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], d));
+    }
+  if (lane == 0 && lo[0] <= hi[0])
+    for (int k = 0; k < 3; ++k) {
+      atomicMin(&bb[k], float_order(lo[k]));
+      atomicMax(&bb[3 + k], float_order(hi[k]));
+    }
+  __syncthreads();
+  for (int t = tid; t < nt; t += 1024) {
+    int id[3];
+    float v[9];
+    uint32_t b = kSkip;
+    if (read(t, id, v, false)) {
+      b = morton_bin(tri_sphere(v), bb, sc.nbuckets);
+      ts[t] = atomicAdd(&bins[b], 1);
+    }
+    tb[t] = b;
+  }
+  __syncthreads();
+  {  // exclusive scan of the bins, 4 per thread
+    int c[4], s = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      c[k] = bins[4 * tid + k];
+      s += c[k];
+    }
+    int run = block_exclusive_scan(s, ws, &tot);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      bins[4 * tid + k] = run;
+      run += c[k];
+    }
+  }
+  __syncthreads();
+  const int n = tot;
+  // the scene's record range: all that k_generate reads of the bin starts
+  if (tid == 0) {
+    starts[0] = 0;
+    starts[sc.nbuckets + 1] = n;
+  }
+  for (int t = tid; t < nt; t += 1024) {
+    const uint32_t b = tb[t];
+    if (b == kSkip) continue;
+    int id[3];
+    float v[9];
+    read(t, id, v, false);
+    const TriSphere s = tri_sphere(v);
+    const int64_t pos = bins[b] + ts[t];
+    rec[pos] = make_float4(s.cx, s.cy, s.cz, s.r);
+    rec[nt + pos] = make_float4(v[0], v[1], v[2], v[3]);
+    rec[2 * (int64_t)nt + pos] = make_float4(v[4], v[5], v[6], v[7]);
+    rec[3 * (int64_t)nt + pos] = make_float4(v[8], __int_as_float(id[0]), __int_as_float(id[1]),
+                                             __int_as_float(id[2]));
+  }
+  __syncthreads();
+  for (int g = 0; g * 1024 < n; ++g) {
+    const int ci = g * 32 + warp, t = ci * 32 + lane;
+    // written by this block before the barrier: read past the first-level cache
+    const float4 c = t < n ? __ldcg(rec + t) : make_float4(0.0f, 0.0f, 0.0f, -1.0f);
+    const float4 sp = sphere_of_spheres(c);
+    if (lane == 0) {
+      cs[warp] = sp;
+      if (sp.w >= 0.0f) chk[ci] = sp;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const float4 gs = sphere_of_spheres(cs[lane]);
+      if (lane == 0 && gs.w >= 0.0f) grp[g] = gs;
+    }
+    __syncthreads();
+  }
 }
 
 // ------------------------------------------------------------------ generation kernel
@@ -1918,7 +2055,8 @@ static cudaError_t bin_triangles(const GenScene *scenes, int num_scenes, int64_t
   float4 *grp = c.take<float4>((nt + 1023) / 1024);
 
   cudaError_t e;
-  for (int s0 = 0; s0 < num_scenes; s0 += kFillChunk) {
+  const bool small = morton && num_scenes == 1 && nt <= kSmallTris;
+  for (int s0 = 0; s0 < num_scenes && !small; s0 += kFillChunk) {
     GenFill f;
     f.n = num_scenes - s0 < kFillChunk ? num_scenes - s0 : kFillChunk;
     for (int i = 0; i < f.n; ++i) f.e[i] = scenes[s0 + i];
@@ -1940,11 +2078,16 @@ static cudaError_t bin_triangles(const GenScene *scenes, int num_scenes, int64_t
   gp.inv_cell = (float)(1.0 / cell);
   gp.mask = 0;
 
-  if ((e = cudaMemsetAsync(counts, 0, sizeof(int) * TB, st)) != cudaSuccess) return e;
+  if (small) {
+    k_sort_small<<<1, 1024, 0, st>>>(scenes[0], tab, tb, ts, starts, rec, chk, grp, status);
+    count_launches(1);
+  } else if ((e = cudaMemsetAsync(counts, 0, sizeof(int) * TB, st)) != cudaSuccess) {
+    return e;
+  }
   const int tpb = 256;
   const int64_t want = (nt + tpb - 1) / tpb;
   const int grid = (int)(want < 152 * 32 ? (want > 0 ? want : 1) : 152 * 32);
-  if (nt > 0) {
+  if (nt > 0 && !small) {
     if (morton) {
       k_tri_bbox<<<grid, tpb, 0, st>>>(tab, num_scenes, nt, bbox);
       count_launches(1);
@@ -1954,11 +2097,13 @@ static cudaError_t bin_triangles(const GenScene *scenes, int num_scenes, int64_t
     count_launches(1);
   }
   const int nb = (int)((TB + kScanItems - 1) / kScanItems);
-  k_scan_partials<<<nb, 256, 0, st>>>(counts, TB, partials);
-  k_scan_top<<<1, 1024, 0, st>>>(partials, nb);
-  k_scan_final<<<nb, 256, 0, st>>>(counts, TB, partials, starts);
-  count_launches(3);
-  if (nt > 0) {
+  if (!small) {
+    k_scan_partials<<<nb, 256, 0, st>>>(counts, TB, partials);
+    k_scan_top<<<1, 1024, 0, st>>>(partials, nb);
+    k_scan_final<<<nb, 256, 0, st>>>(counts, TB, partials, starts);
+    count_launches(3);
+  }
+  if (nt > 0 && !small) {
     k_tri_scatter<<<grid, tpb, 0, st>>>(tab, num_scenes, nt, tb, ts, starts, rec);
     count_launches(1);
     if (morton) {
