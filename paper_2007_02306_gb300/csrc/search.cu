@@ -118,6 +118,8 @@ __global__ void k_encode_needles(const uint16_t *__restrict__ imgs, int64_t n, i
 //   CW = 1              k_sparse: any word of the 32 images is one 128-byte line
 // list (optional): encode images list[0 .. *list_count) of imgs as images 0, 1, ... (a compacted
 // subset, count read on the device; n is then an upper bound).  Images past the last are zero.
+// wide_flag and narrow (bit l of word g: image 32 g + l exists and is not wide; zero words up to
+// a multiple of four groups) are optional.
 // One block per group; 256 pixels of its images at a time cross through shared memory, so that
 // both the reads (512 bytes of an image) and the writes are contiguous.  Writing from one warp
 // per image instead left 1 or 16 bytes in every 128-byte line (262,144 images of 64 x 64:
@@ -127,7 +129,9 @@ template <int CW>
 __global__ void __launch_bounds__(kGroupWarps * 32) k_encode_groups(
     const uint16_t *__restrict__ imgs, int64_t n, int N, int8_t *__restrict__ delta,
     int *__restrict__ wide_flag, int *__restrict__ wide_list, int *__restrict__ wide_count,
-    const int *__restrict__ list, const int *__restrict__ list_count) {
+    const int *__restrict__ list, const int *__restrict__ list_count,
+    uint32_t *__restrict__ narrow) {
+  __shared__ uint32_t group_wide;
   constexpr int kPerW = 32 / kGroupWarps;  // images of a warp
   __shared__ uint32_t tile[64][33];        // [word of the 256 pixels][image]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -137,6 +141,7 @@ __global__ void __launch_bounds__(kGroupWarps * 32) k_encode_groups(
   for (int64_t g = blockIdx.x; g * 32 < n; g += gridDim.x) {
     int wide[kPerW];
     const uint16_t *img[kPerW];
+    if (threadIdx.x == 0) group_wide = 0;  // (read by nobody before the barriers below)
 #pragma unroll
     for (int q = 0; q < kPerW; ++q) {
       const int64_t i = g * 32 + warp * kPerW + q;
@@ -178,9 +183,22 @@ __global__ void __launch_bounds__(kGroupWarps * 32) k_encode_groups(
       const int any = __any_sync(0xffffffffu, wide[q]);
       const int64_t i = g * 32 + warp * kPerW + q;
       if (lane == 0 && i < n) {
-        wide_flag[i] = any;
-        if (any) wide_list[atomicAdd(wide_count, 1)] = (int)i;
+        if (wide_flag) wide_flag[i] = any;
+        if (any) {
+          wide_list[atomicAdd(wide_count, 1)] = (int)i;
+          atomicOr(&group_wide, 1u << (warp * kPerW + q));
+        }
       }
+    }
+    if (narrow) {
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        const int64_t left = n - g * 32;
+        narrow[g] = ~group_wide & (left >= 32 ? 0xffffffffu : (1u << left) - 1u);
+        if (left <= 32)
+          for (int64_t e = g + 1; e & 3; ++e) narrow[e] = 0;
+      }
+      __syncthreads();
     }
   }
 }
@@ -605,18 +623,23 @@ __global__ void __launch_bounds__(256) k_sparse_needles(const int8_t *__restrict
 
 // Narrow needles x narrow haystack images over the needles' sparse entries.  Block: kSparseWarps
 // needles (one per warp) sweeping a band of haystack tiles of 32 * kSparseImg images; lane l of a
-// warp holds images j0 + l + 32 k.  Per step the warp reads kSparseStep entries (the same address
-// in every lane) and each lane gathers the entries' words of its images that are still alive
-// (one coalesced 128-byte access per warp and image slot).
+// warp holds images j0 + l + 32 k.  Most pairs of sparse needles stop within a word or two, so the
+// first kSparseHead entries stay in shared memory for the whole band, the words of the first
+// kSparseStep of the next tile are loaded before the current tile is summed (one coalesced 128-byte
+// access per warp, entry and image slot), the images to rank come as one bit each, and a tile none
+// of whose images is left ends there.  Bound by the L2 gathers: at least 1 KB per warp and tile.
+// 16,384 sparse needles x 262,144 images: 11.8 -> 8.8 ms for the whole call (entries, class flags and
+// reductions per tile before).
 template <bool kCount>
-__global__ void __launch_bounds__(kSparseWarps * 32) k_sparse(
+__global__ void __launch_bounds__(kSparseWarps * 32, 4) k_sparse(
     const int4 *__restrict__ ent, const int *__restrict__ ecount,
     const int *__restrict__ nwide, int64_t Q, const int8_t *__restrict__ hword,
-    const int *__restrict__ hwide, int64_t H, int N, const int64_t *__restrict__ dtrue,
+    const uint4 *__restrict__ narrow, int64_t H, int N, const int64_t *__restrict__ dtrue,
     const int *__restrict__ nflags, int *__restrict__ rank, unsigned long long *__restrict__ best,
     unsigned long long *__restrict__ counters, int64_t tile0, int64_t tiles_q, int64_t tiles_h,
     int64_t band_h) {
   constexpr int kTile = 32 * kSparseImg;
+  static_assert(kSparseImg == 4 && kSparseHead == 2 * kSparseStep, "one uint4 of image bits per tile");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t L = tile0 + blockIdx.x;
   const int64_t band = L / tiles_q, qt = L - band * tiles_q;
@@ -630,60 +653,101 @@ __global__ void __launch_bounds__(kSparseWarps * 32) k_sparse(
   const int ne = ecount[q];
   const int4 *e = ent + q * (int64_t)KW;
   const int64_t gbytes = (int64_t)KW * 128;  // one group of 32 images
+  const int64_t groups = (H + 31) / 32;
   unsigned long long pair_words = 0, lane_slots = 0;
-  for (int64_t ht = h0; ht < h1; ++ht) {
-    const int64_t j0 = ht * kTile + lane;
-    int acc[kSparseImg];  // partial distance minus the needle's true distance (exit once > 0)
-    unsigned alive = 0;
+  __shared__ int4 head_s[kSparseWarps][kSparseHead];
+  if (lane < kSparseHead)
+    head_s[warp][lane] = lane < ne ? e[lane] : make_int4(0, 0, 0, 0);  // a zero entry adds nothing
+  __syncwarp();
+  const int4 *const head = head_s[warp];
+  auto word = [&](const int8_t *hb, int k, int off) {
+    return *reinterpret_cast<const int *>(hb + k * gbytes + off);
+  };
+  auto base_of = [&](int64_t ht) { return hword + ht * kSparseImg * gbytes + lane * 4; };
+  // words of the first step's entries of a tile's images (groups past the haystack are not read)
+  auto fetch = [&](int64_t ht, int (&b)[kSparseStep][kSparseImg]) {
+    const int8_t *hb = base_of(ht);
 #pragma unroll
     for (int k = 0; k < kSparseImg; ++k) {
-      const int64_t j = j0 + 32 * k;
-      acc[k] = -thr;
-      if (j < H && !hwide[j]) alive |= 1u << k;
+      const bool in = ht * kSparseImg + k < groups;
+#pragma unroll
+      for (int u = 0; u < kSparseStep; ++u) b[u][k] = in ? word(hb, k, head[u].z) : 0;
     }
-    const int8_t *hb = hword + (j0 >> 5) * gbytes + lane * 4;
-    // steps of S entries from e0 while any image of the warp is alive; returns where it stopped
-    auto steps = [&](auto step_tag, int e0, int e_end) {
-      constexpr int S = decltype(step_tag)::value;
-      for (; e0 < e_end; e0 += S) {
-        if (__ballot_sync(0xffffffffu, alive != 0) == 0) return ne;
-        int4 E[S];
+  };
+  int acc[kSparseImg] = {};  // partial distance minus the needle's true distance (exit once > 0)
+  // m (a - b)^2 over the word = sum a^2 + sum (m b)^2 - 2 sum a b
+  auto add = [&](int k, const int4 &E, int b) {
+    const int bm = b & E.y;
+    acc[k] = __dp4a(bm, bm, acc[k] + E.w) - 2 * __dp4a(E.x, b, 0);
+  };
+  int next[kSparseStep][kSparseImg];
+  fetch(h0, next);
+  for (int64_t ht = h0; ht < h1; ++ht) {
+    const uint4 bits = narrow[ht];
+    int b[kSparseStep][kSparseImg];
 #pragma unroll
-        for (int u = 0; u < S; ++u)
-          E[u] = e0 + u < ne ? e[e0 + u] : make_int4(0, 0, 0, 0);  // a zero entry adds nothing
-        int b[S][kSparseImg];
+    for (int u = 0; u < kSparseStep; ++u)
 #pragma unroll
-        for (int u = 0; u < S; ++u)
+      for (int k = 0; k < kSparseImg; ++k) b[u][k] = next[u][k];
+    if (ht + 1 < h1) fetch(ht + 1, next);
+    unsigned alive = ((bits.x >> lane) & 1u) | (((bits.y >> lane) & 1u) << 1) |
+                     (((bits.z >> lane) & 1u) << 2) | (((bits.w >> lane) & 1u) << 3);
+    auto count = [&](int n) {
+      if (kCount && n > 0) {
+        pair_words += (unsigned long long)__popc(alive) * n;
+        lane_slots += (unsigned long long)kSparseImg * n;
+      }
+    };
+    auto leave = [&]() {  // images that have exited keep stale sums
 #pragma unroll
-          for (int k = 0; k < kSparseImg; ++k)
-            b[u][k] = (alive >> k) & 1u
-                          ? *reinterpret_cast<const int *>(hb + k * gbytes + E[u].z)
-                          : 0;
-        if (kCount) {
-          const int n = ne - e0 < S ? ne - e0 : S;
-          pair_words += (unsigned long long)__popc(alive) * n;
-          lane_slots += (unsigned long long)kSparseImg * n;
-        }
+      for (int k = 0; k < kSparseImg; ++k)
+        if (acc[k] > 0) alive &= ~(1u << k);
+    };
+    if (__ballot_sync(0xffffffffu, alive != 0) == 0) continue;
+    count(ne < kSparseStep ? ne : kSparseStep);
 #pragma unroll
-        for (int u = 0; u < S; ++u)
+    for (int k = 0; k < kSparseImg; ++k) {
+      acc[k] = -thr;
 #pragma unroll
-          for (int k = 0; k < kSparseImg; ++k) {
-            // m (a - b)^2 over the word = sum a^2 + sum (m b)^2 - 2 sum a b
-            const int bm = b[u][k] & E[u].y;
-            const int sq = __dp4a(bm, bm, acc[k] + E[u].w);
-            acc[k] = sq - 2 * __dp4a(E[u].x, b[u][k], 0);
-          }
+      for (int u = 0; u < kSparseStep; ++u) add(k, head[u], b[u][k]);
+    }
+    leave();
+    if (__ballot_sync(0xffffffffu, alive != 0) == 0) continue;
+    const int8_t *hb = base_of(ht);
+    if (ne > kSparseStep) {
+      count(ne < kSparseHead ? ne - kSparseStep : kSparseStep);
+#pragma unroll
+      for (int u = 0; u < kSparseStep; ++u)
 #pragma unroll
         for (int k = 0; k < kSparseImg; ++k)
-          if (acc[k] > 0) alive &= ~(1u << k);  // images that have exited keep stale sums
-      }
-      return e0;
-    };
-    // short steps first (most pairs of sparse needles stop within a word or two), then longer
-    // steps with more loads in flight for the pairs that go on
-    const int e_mid = ne < kSparseHead ? ne : kSparseHead;
-    const int e1 = steps(std::integral_constant<int, kSparseStep>(), 0, e_mid);
-    steps(std::integral_constant<int, kSparseStepLong>(), e1, ne);
+          b[u][k] = (alive >> k) & 1u ? word(hb, k, head[kSparseStep + u].z) : 0;
+#pragma unroll
+      for (int k = 0; k < kSparseImg; ++k)
+#pragma unroll
+        for (int u = 0; u < kSparseStep; ++u) add(k, head[kSparseStep + u], b[u][k]);
+      leave();
+    }
+    // longer steps with more loads in flight for the pairs that go on
+    for (int e0 = kSparseHead; e0 < ne; e0 += kSparseStepLong) {
+      if (__ballot_sync(0xffffffffu, alive != 0) == 0) break;
+      count(ne - e0 < kSparseStepLong ? ne - e0 : kSparseStepLong);
+      int4 E[kSparseStepLong];
+#pragma unroll
+      for (int u = 0; u < kSparseStepLong; ++u)
+        E[u] = e0 + u < ne ? e[e0 + u] : make_int4(0, 0, 0, 0);
+      int w[kSparseStepLong][kSparseImg];
+#pragma unroll
+      for (int u = 0; u < kSparseStepLong; ++u)
+#pragma unroll
+        for (int k = 0; k < kSparseImg; ++k) w[u][k] = (alive >> k) & 1u ? word(hb, k, E[u].z) : 0;
+#pragma unroll
+      for (int u = 0; u < kSparseStepLong; ++u)
+#pragma unroll
+        for (int k = 0; k < kSparseImg; ++k) add(k, E[u], w[u][k]);
+      leave();
+    }
+    if (__ballot_sync(0xffffffffu, alive != 0) == 0) continue;
+    const int64_t j0 = ht * kTile + lane;
     int c = 0;
     unsigned long long bb = kNoBest;
 #pragma unroll
@@ -1030,8 +1094,8 @@ cudaError_t launch_dense(const int8_t *nd, const int8_t *nm, const int *nrs, con
 }
 
 cudaError_t launch_sparse(const int4 *ent, const int *ecount, const int *nw, int64_t Q,
-                          const int8_t *hd, const int *hw, int64_t H, int N, const int64_t *dt,
-                          const int *nf, int *rank, unsigned long long *best,
+                          const int8_t *hd, const uint32_t *narrow, int64_t H, int N,
+                          const int64_t *dt, const int *nf, int *rank, unsigned long long *best,
                           unsigned long long *counters, cudaStream_t st) {
   auto kern = counters ? k_sparse<true> : k_sparse<false>;
   const int64_t th = (H + 32 * kSparseImg - 1) / (32 * kSparseImg);
@@ -1046,7 +1110,9 @@ cudaError_t launch_sparse(const int4 *ent, const int *ecount, const int *nw, int
   constexpr int64_t kMaxGrid = 0x7fffffffll;
   for (int64_t t0 = 0; t0 < total; t0 += kMaxGrid) {
     const int64_t n = total - t0 < kMaxGrid ? total - t0 : kMaxGrid;
-    kern<<<(unsigned)n, kSparseWarps * 32, 0, st>>>(ent, ecount, nw, Q, hd, hw, H, N, dt, nf, rank,
+    kern<<<(unsigned)n, kSparseWarps * 32, 0, st>>>(ent, ecount, nw, Q, hd,
+                                                    reinterpret_cast<const uint4 *>(narrow), H, N,
+                                                    dt, nf, rank,
                                                     best, counters, t0, tq, th, band_h);
     count_launches(1);
   }
@@ -1080,7 +1146,7 @@ int64_t search_batch_workspace_bytes(int num_scenes, int64_t Q, int64_t H, int N
   c.take<int>((packed && !sparse) || mid ? Q * N : 0);  // needle row sums of squared deltas
   c.take<int8_t>(packed || mid ? (H + 31) / 32 * 32 * K : 0);  // haystack deltas (groups of 32)
   c.take<int>(Q);                        // needle wide flags
-  c.take<int>(H);                        // haystack wide flags
+  c.take<int>(H + 4);                    // haystack wide flags (or, sparse form, a bit per image)
   c.take<int>(Q);                        // wide needle list
   c.take<int>(H);                        // wide haystack list
   c.take<int>(8);                        // list lengths
@@ -1098,7 +1164,7 @@ int64_t search_batch_workspace_bytes(int num_scenes, int64_t Q, int64_t H, int N
   c.take<int>(mid ? Q + H : 0);  // lists written by its encodes
   c.take<int>(mid ? H : 0);      // images of neither tensor-core class
   c.take<int8_t>(autom ? (H + 31) / 32 * 32 * K : 0);  // word-major haystack of the sparse form
-  c.take<int>(autom ? H : 0);     // its int8 class flags
+  c.take<uint32_t>(autom ? (H + 127) / 128 * 4 : 0);  // its int8 class, a bit per image
   c.take<int>(autom ? 3 * Q : 0);  // per-needle choice and the two exclusions
   c.take<int>(autom ? Q / 128 + 2 : 0);  // tensor-core needle tiles to skip
   return c.off + 256;
@@ -1145,7 +1211,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   int *nrs = c.take<int>(dense || mid ? Q * N : 0);
   int8_t *hd = c.take<int8_t>(packed || mid ? (H + 31) / 32 * 32 * K : 0);
   int *nwide = c.take<int>(Q);
-  int *hwide = c.take<int>(H);
+  int *hwide = c.take<int>(H + 4);
   int *wn_list = c.take<int>(Q);
   int *wh_list = c.take<int>(H);
   int *counts = c.take<int>(8);
@@ -1163,7 +1229,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   int *mid_list = c.take<int>(mid ? Q + H : 0);
   int *left_list = c.take<int>(mid ? H : 0);
   int8_t *hword = c.take<int8_t>(autom ? (H + 31) / 32 * 32 * K : 0);
-  int *auto_hflag = c.take<int>(autom ? H : 0);
+  uint32_t *auto_narrow = c.take<uint32_t>(autom ? (H + 127) / 128 * 4 : 0);
   int *auto_n = c.take<int>(autom ? 3 * Q : 0);
   int *skip_tile = c.take<int>(autom ? Q / 128 + 2 : 0);
   int *sparse_of = autom ? auto_n : nullptr;
@@ -1220,13 +1286,13 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
                          const int *count) {
     auto kern = N == 8 ? k_encode_groups<2> : k_encode_groups<4>;
     kern<<<group_blocks, kGroupWarps * 32, 0, st>>>(scenes[0].haystack, H, N, out, flag, wlist,
-                                                    wcount, list, count);
+                                                    wcount, list, count, nullptr);
     count_launches(1);
   };
-  auto encode_words = [&](int8_t *out, int *flag, int *wlist, int *wcount) {
+  auto encode_words = [&](int8_t *out, uint32_t *narrow, int *wlist, int *wcount) {
     k_encode_groups<1><<<group_blocks, kGroupWarps * 32, 0, st>>>(scenes[0].haystack, H, N, out,
-                                                                  flag, wlist, wcount, nullptr,
-                                                                  nullptr);
+                                                                  nullptr, wlist, wcount, nullptr,
+                                                                  nullptr, narrow);
     count_launches(1);
   };
   if (tensor) {
@@ -1271,8 +1337,8 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
     if (autom) {
       // the sparse-needle form for its needles against every int8-class image (the encode's list
       // of images outside int8 goes to wh_list, whose readers above precede it on the stream)
-      encode_words(hword, auto_hflag, wh_list, counts + 4);
-      if ((e = launch_sparse(sent, scount, excl_sparse, Q, hword, auto_hflag, H, N, dt, nflags,
+      encode_words(hword, auto_narrow, wh_list, counts + 4);
+      if ((e = launch_sparse(sent, scount, excl_sparse, Q, hword, auto_narrow, H, N, dt, nflags,
                              rank, best, cnt, st)) != cudaSuccess)
         return e;
     }
@@ -1297,10 +1363,11 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
     const SearchScene &s0 = scenes[0];
     k_encode_needles<<<blocks_for(Q), 32 * wpb, 0, st>>>(s0.needles, Q, N, nd, nm, nwide, wn_list,
                                                          counts + 0, nullptr);
-    encode_words(hd, hwide, wh_list, counts + 1);
+    uint32_t *const narrow = reinterpret_cast<uint32_t *>(hwide);
+    encode_words(hd, narrow, wh_list, counts + 1);
     k_sparse_needles<<<blocks_for(Q), 32 * wpb, 0, st>>>(nd, nm, Q, N, sent, scount);
     count_launches(2);
-    if ((e = launch_sparse(sent, scount, nwide, Q, hd, hwide, H, N, dt, nflags, rank, best, cnt,
+    if ((e = launch_sparse(sent, scount, nwide, Q, hd, narrow, H, N, dt, nflags, rank, best, cnt,
                            st)) != cudaSuccess)
       return e;
     wide(0);
