@@ -318,7 +318,7 @@ RICI_API int rici_clutter(const float *vertices, const float *normals, int64_t n
  *              exactly as an integer number of units of 2^-24 (rounding error <= 2^-25 per
  *              weight; the sums do not depend on the order of the samples), so each bin differs
  *              from the FP64 definition by at most the rounding of those FP32 steps.
- * Workspace: rici_clutter_workspace_size bytes (the clutter measure's grid), or NULL.
+ * Workspace: rici_clutter_workspace_size bytes, or NULL.
  * Errors: as rici_generate (a zero image for an oriented point with a bad index or a
  * non-finite coordinate).
  */
@@ -371,17 +371,16 @@ RICI_API int64_t rici_kernel_launches(void);
  * paper has no counterpart (it fixes one kernel configuration for its GPU). */
 struct RiciTuning {
   int32_t gen_cells_per_reach; /* 2, 3 or 4: grid cells per triangle reach (the support
-                                  sphere's radius plus the largest binned triangle's) of the
-                                  clutter measure and spin images, which scan up to 7^3 cells
-                                  around each oriented point (at most 3 per reach). Image
-                                  generation sorts its triangles along a space-filling curve
-                                  and culls them by bounding spheres of runs of 32 and 1024
-                                  instead, and ignores this field. Default 2. */
-  float gen_big_radius;        /* in [1/16, 1]: in the clutter measure and spin images,
-                                  triangles whose bounding radius exceeds this fraction of the
-                                  support sphere's radius are checked by every oriented point
-                                  instead of being binned (image generation ignores it).
-                                  Default 0.25. */
+                                  sphere's radius plus the largest binned triangle's) of spin
+                                  images, which scan up to 7^3 cells around each oriented point
+                                  (at most 3 per reach). Image generation and the clutter
+                                  measure sort their triangles along a space-filling curve and
+                                  cull them by bounding spheres of runs of 32 and 1024 instead,
+                                  and ignore this field. Default 2. */
+  float gen_big_radius;        /* in [1/16, 1]: in spin images, triangles whose bounding radius
+                                  exceeds this fraction of the support sphere's radius are
+                                  checked by every oriented point instead of being binned (the
+                                  others ignore it). Default 0.25. */
   int32_t gen_warps;           /* 4 or 8 warps per oriented point (image generation). Default 4. */
   int32_t tc_group_m;          /* 1..64: needle tiles of 128 that the tensor-core search sweeps
                                   together over the haystack (L2 reuse). Default 8. */
