@@ -1045,14 +1045,16 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_search_small(SearchScene s
 }
 
 // Whether a call takes k_search_small: the forms that leave the choice to the library (DEFAULT,
-// AUTO), no work counters, and so little work that launches decide: at most 2^19 pixel pairs per
-// block and 2^28 in all.  162 x 162 images of 32 x 32 with the distance matrix: 114 us in the
-// general sequence of 19 launches, 35 us here (most of it the call's host side); at the limits the
-// kernel takes as long as that sequence.
+// AUTO), no work counters, and so little work that launches decide.  A pair costs a warp about
+// 0.45 us and 0.11 us per 256 pixels, one after another, so the haystack is limited (256 images of up
+// to 32 x 32, 64 of 64 x 64, 16 of 128 x 128), and with it the work in all.  162 x 162 images of 32 x
+// 32 with the distance matrix: 114 us in the general sequence of 19 launches, 35 us here (most of
+// it the call's host side).  Past the limits it loses: 64 x 512 images of 32 x 32 80 against 93 us,
+// 512 x 512 190 against 95 us, 16 x 2,048 of 16 x 16 146 against 85 us.
 bool small_search(const SearchBatch &b) {
-  const int64_t K = (int64_t)b.N * b.N;
+  const int64_t K = (int64_t)b.N * b.N < 1024 ? 1024 : (int64_t)b.N * b.N;
   return (b.mode == RICI_SEARCH_DEFAULT || b.mode == RICI_SEARCH_AUTO) && b.num_scenes == 1 &&
-         !b.counters && b.Htot * K <= (1 << 19) && b.Qtot * b.Htot * K <= (1 << 28);
+         !b.counters && b.Htot * K <= (1 << 18) && b.Qtot * b.Htot * K <= (1 << 26);
 }
 
 bool dense_supported(int N) { return N == 8 || N == 16 || N == 32 || N == 64 || N == 128; }
