@@ -24,7 +24,7 @@
 // pair's work on the tensor cores, against CUDA cores at a ninth of that rate (8,192 needles x
 // 262,144 of its images: 35.7 ms with those pairs on k_dense, 24.5 ms here).
 //
-// Kernel structure (one CTA per SM, persistent over 128 x 256 output tiles):
+// Kernel structure of k_tc_rank (one CTA per SM, persistent over 128 x 256 output tiles):
 //   warp 0: TMA producer (128B-swizzled K-major tiles, 4-stage mbarrier pipeline)
 //   warp 1: TMEM allocator and single-thread tcgen05.mma issuer (M=128, N=256, K=16)
 //   warps 2-5: epilogue; tcgen05.ld of the accumulator (double-buffered: 2 x 256 columns)
@@ -145,12 +145,13 @@ constexpr uint32_t kIdesc = (1u << 4)                      // D format F32
                             | ((uint32_t)(kBN >> 3) << 17) // N / 8
                             | ((uint32_t)(kBM >> 4) << 24);// M / 16
 
+template <uint32_t kDesc = kIdesc>
 __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
                                        uint32_t accumulate) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate));
+      "l"(adesc), "l"(bdesc), "r"(kDesc), "r"(accumulate));
 }
 
 __device__ __forceinline__ void tc_commit(uint64_t *bar) {
@@ -578,12 +579,352 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   }
 }
 
+// ---------------------------------------------------------------- few needles: encode and GEMM in one
+//
+// With few needles the GEMM is short and the haystack's operand rows (16 KB per image at N = 64, from
+// 8 KB of pixels) cost the time: written by one kernel, read by the next.  Here the pixels go from
+// global to shared memory once and become operand tiles there; nothing of the haystack is written
+// back but the list of the images outside the fp16 class.
+//
+// Persistent over items of (needle tile of 128, haystack tile of 128 images), needle tiles of one
+// haystack tile next to each other (its pixels come from L2 then).  K runs in chunks of 64 pixels:
+//   warp 0      TMA of the pixels: 128 images x 64 pixels, 128-byte swizzle, 3 stages
+//   warp 1      TMEM allocator and MMA issuer: m x b^2 and a x (-2 b), M = N = 128, K = 64 each
+//   warps 2-5   epilogue, as in k_tc_rank (double-buffered: 2 x 128 TMEM columns)
+//   warps 6-21  converters: four threads per image, 16 pixels each, from the pixel stage to the two
+//               operand tiles (K-major, same swizzle), and the image's class
+//   warp 22     TMA of the needles' operand blocks [m | a] of the chunk, 2 stages
+// Shared-memory bandwidth bounds it: per chunk 48 KB arrive, 48 KB pass through the converters and the
+// MMAs read 64 KB, 1,250 cycles at 128 bytes each against 1,376 measured (0.2 ms for 90,001 images of
+// 64 x 64 and a needle tile; their pixels alone take 0.11 ms of HBM).  Whole calls, operand rows
+// written by an encode and read by k_tc_rank against this kernel: 100 needles 715 -> 355 us, 256
+// 754 -> 554 us, 512 959 -> 916 us, 1,024 1,357 -> 1,712 us; 90,001 images of 32 x 32: 128 needles 262 ->
+// 147 us, 512 352 -> 305 us; so up to 512 needles take it.
+constexpr int kQN = 128;          // haystack images per tile
+constexpr int kQRaw = 3;          // pixel stages (16 KB)
+constexpr int kQOps = 2;          // operand stages (needles 32 KB, haystack 32 KB)
+constexpr int kQConvWarps = 16;
+constexpr int kQThreads = (7 + kQConvWarps) * 32;
+constexpr uint32_t kQTile = 128 * 128;  // one operand or pixel block: 128 rows of 128 bytes
+constexpr uint32_t kIdescQ = (1u << 4) | ((uint32_t)(kQN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
+
+struct QueryArgs {
+  int64_t Q, H;
+  int N, tiles_m;
+  int64_t items;
+  const int *nwide, *nflags, *asum;
+  const int64_t *dtrue;
+  int *rank;
+  unsigned long long *best;
+  int *hwide, *wh_list, *wh_count;
+  int *status;
+};
+
+__global__ void __launch_bounds__(kQThreads, 1)
+    k_tc_query(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_px,
+               QueryArgs a) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char *smem = reinterpret_cast<unsigned char *>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  unsigned char *s_px = smem;                          // kQRaw tiles
+  unsigned char *s_a = s_px + kQRaw * kQTile;          // kQOps x (m, a)
+  unsigned char *s_b = s_a + kQOps * 2 * kQTile;       // kQOps x (b^2, -2b)
+  uint64_t *px_full = reinterpret_cast<uint64_t *>(s_b + kQOps * 2 * kQTile);
+  uint64_t *px_empty = px_full + kQRaw;
+  uint64_t *a_full = px_empty + kQRaw;
+  uint64_t *b_full = a_full + kQOps;
+  uint64_t *op_empty = b_full + kQOps;
+  uint64_t *tfull = op_empty + kQOps;
+  uint64_t *tempty = tfull + 2;
+  uint64_t *cls_full = tempty + 2;
+  uint64_t *drain = cls_full + 2;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
+  int *abort_flag = reinterpret_cast<int *>(tmem_slot + 1);
+  unsigned char *cls = reinterpret_cast<unsigned char *>(abort_flag + 1);  // [2][kQN]: fp16 class
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int K0 = a.N * a.N, chunks = K0 / 64;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kQRaw; ++s) {
+      mbar_init(&px_full[s], 1);
+      mbar_init(&px_empty[s], kQConvWarps);
+    }
+    for (int s = 0; s < kQOps; ++s) {
+      mbar_init(&a_full[s], 1);
+      mbar_init(&b_full[s], kQConvWarps);
+      mbar_init(&op_empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&tfull[b], 1);
+      mbar_init(&tempty[b], 4);
+      mbar_init(&cls_full[b], kQConvWarps);
+    }
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(256));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    // ---------------- pixels
+    if (lane == 0) {
+      uint32_t it = 0;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < a.items && ok; t += gridDim.x) {
+        const int y = (int)(t / a.tiles_m * kQN);
+        for (int c = 0; c < chunks; ++c, ++it) {
+          const uint32_t s = it % kQRaw, round = it / kQRaw;
+          if (!mbar_wait(&px_empty[s], (round & 1) ^ 1, a.status, abort_flag)) {
+            ok = false;
+            break;
+          }
+          mbar_arrive_expect_tx(&px_full[s], kQTile);
+          tma_load_2d(s_px + s * kQTile, &map_px, &px_full[s], c * 64, y);
+        }
+      }
+      for (uint32_t j = 1; j <= (uint32_t)kQRaw && j <= it; ++j)
+        mbar_drain(&px_full[(it - j) % kQRaw], ((it - j) / kQRaw) & 1, a.status);
+    }
+  } else if (warp == 6 + kQConvWarps) {
+    // ---------------- needle operands
+    if (lane == 0) {
+      uint32_t it = 0;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < a.items && ok; t += gridDim.x) {
+        const int y = (int)(t % a.tiles_m * kBM);
+        for (int c = 0; c < chunks; ++c, ++it) {
+          const uint32_t s = it % kQOps, round = it / kQOps;
+          if (!mbar_wait(&op_empty[s], (round & 1) ^ 1, a.status, abort_flag)) {
+            ok = false;
+            break;
+          }
+          mbar_arrive_expect_tx(&a_full[s], 2 * kQTile);
+          tma_load_2d(s_a + s * 2 * kQTile, &map_a, &a_full[s], c * 64, y);
+          tma_load_2d(s_a + s * 2 * kQTile + kQTile, &map_a, &a_full[s], K0 + c * 64, y);
+        }
+      }
+      for (uint32_t j = 1; j <= (uint32_t)kQOps && j <= it; ++j)
+        mbar_drain(&a_full[(it - j) % kQOps], ((it - j) / kQOps) & 1, a.status);
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer (one thread)
+    if (lane == 0) {
+      uint32_t it = 0, lt = 0;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < a.items && ok; t += gridDim.x) {
+        const uint32_t buf = lt & 1, use = lt >> 1;
+        ++lt;
+        if (!mbar_wait(&tempty[buf], (use & 1) ^ 1, a.status, abort_flag)) break;
+        tc_fence_after();
+        const uint32_t tacc = tmem + buf * kQN;
+        for (int c = 0; c < chunks; ++c, ++it) {
+          const uint32_t s = it % kQOps, round = it / kQOps;
+          if (!mbar_wait(&a_full[s], round & 1, a.status, abort_flag) ||
+              !mbar_wait(&b_full[s], round & 1, a.status, abort_flag)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t a0 = smem_u32(s_a + s * 2 * kQTile), b0 = smem_u32(s_b + s * 2 * kQTile);
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk) {  // 4 steps of K = 16 in either block
+            const uint32_t off = (kk >> 2) * kQTile + (kk & 3) * 32;
+            tc_mma<kIdescQ>(tacc, smem_desc(a0 + off), smem_desc(b0 + off),
+                            (c > 0 || kk > 0) ? 1u : 0u);
+          }
+          tc_commit(&op_empty[s]);
+        }
+        if (!ok) break;
+        tc_commit(&tfull[buf]);
+      }
+      tc_commit(drain);
+      mbar_drain(drain, 0, a.status);
+    }
+  } else if (warp >= 6) {
+    // ---------------- converters: image `row` of the tile, 16 pixels from 16 `quad` of a chunk.  Two
+    // pixels at a time: with w = (p0, p1) and v = (p before, p0), w - v + 0x66006600 are the bits of
+    // the halves 1536 + d0, 1536 + d1 (as in k_tc_encode; the low half lends nothing to the high one
+    // as long as |d0| < 0x6600), so a pair costs nine instructions in all.  Deltas past the halves'
+    // range give halves past the class limit, infinities or NaN; pixels of 32,768 and more, whose
+    // differences could wrap around, put the image outside the class too (the split-square encode
+    // looks at those again).
+    const int ct = threadIdx.x - 6 * 32, row = ct >> 2, quad = ct & 3;
+    const __half2 k1536 = __floats2half2_rn(1536.0f, 1536.0f), km2 = __floats2half2_rn(-2.0f, -2.0f);
+    uint32_t it = 0, lt = 0;
+    bool ok = true;
+    for (int64_t t = blockIdx.x; t < a.items && ok; t += gridDim.x) {
+      const uint32_t buf = lt & 1, use = lt >> 1;
+      ++lt;
+      unsigned any = 0, last = 0;
+      int s2 = 0, s1 = 0;
+      __half2 top = __floats2half2_rn(0.0f, 0.0f);
+      for (int c = 0; c < chunks; ++c, ++it) {
+        const uint32_t s = it % kQRaw, o = it % kQOps;
+        ok = __all_sync(0xffffffffu,
+                        mbar_wait(&px_full[s], (it / kQRaw) & 1, a.status, abort_flag) &&
+                            mbar_wait(&op_empty[o], ((it / kQOps) & 1) ^ 1, a.status, abort_flag));
+        if (!ok) break;
+        const unsigned char *src = s_px + s * kQTile + row * 128;
+        unsigned char *dst = s_b + o * 2 * kQTile + row * 128;
+        uint32_t w[8];
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          const uint4 x = *reinterpret_cast<const uint4 *>(src + (((quad * 2 + v) ^ (row & 7)) << 4));
+          w[4 * v] = x.x;
+          w[4 * v + 1] = x.y;
+          w[4 * v + 2] = x.z;
+          w[4 * v + 3] = x.w;
+        }
+        // the word before the first: the previous thread's last one, of this chunk, or (first thread;
+        // only rows of 128 pixels continue there) of the chunk before
+        const unsigned left = __shfl_up_sync(0xffffffffu, w[7], 1);
+        const unsigned carry = __shfl_down_sync(0xffffffffu, last, 3);
+        last = w[7];
+        uint32_t prev = quad ? left : carry;
+        __half2 sum = __floats2half2_rn(0.0f, 0.0f);  // sum |b| of the chunk's pairs: at most 8 x 45
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          // rows start at multiples of N pixels, so only at the first pixel of 8: delta 0 there
+          if (((c * 64 + quad * 16 + v * 8) & (a.N - 1)) == 0) prev = w[4 * v] << 16;
+          uint32_t sq[4], dbl[4], bits[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const uint32_t x = w[4 * v + e];
+            bits[e] = x - __funnelshift_l(prev, x, 16) + 0x66006600u;
+            prev = x;
+            any |= x;
+            const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&bits[e]), k1536);
+            const __half2 ha = __habs2(h);
+            top = __hmax2_nan(top, ha);
+            sum = __hadd2(sum, ha);
+            const __half2 hs = __hmul2(h, h), hd = __hmul2(h, km2);
+            sq[e] = *reinterpret_cast<const uint32_t *>(&hs);
+            dbl[e] = *reinterpret_cast<const uint32_t *>(&hd);
+          }
+#pragma unroll
+          for (int e = 0; e < 4; e += 2) {  // the low bytes of the halves' bits are the deltas'
+            const int d4 = (int)__byte_perm(bits[e], bits[e + 1], 0x6420);
+            s2 = __dp4a(d4, d4, s2);
+          }
+          const int at = ((quad * 2 + v) ^ (row & 7)) << 4;
+          *reinterpret_cast<uint4 *>(dst + at) = make_uint4(sq[0], sq[1], sq[2], sq[3]);
+          *reinterpret_cast<uint4 *>(dst + kQTile + at) = make_uint4(dbl[0], dbl[1], dbl[2], dbl[3]);
+        }
+        const float2 sf = __half22float2(sum);
+        s1 += (int)fminf(sf.x + sf.y, 65536.0f);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(&px_empty[s]);
+          mbar_arrive(&b_full[o]);
+        }
+      }
+      if (!ok) break;
+      // the image's class, once the epilogue has read the buffer's previous one
+      ok = __all_sync(0xffffffffu, mbar_wait(&tempty[buf], (use & 1) ^ 1, a.status, abort_flag));
+      if (!ok) break;
+      const float2 tf = __half22float2(top);
+      int wide = !(tf.x <= (float)kNarrowB && tf.y <= (float)kNarrowB) || (any & 0x80008000u) != 0;
+#pragma unroll
+      for (int k = 1; k < 4; k <<= 1) {
+        wide |= __shfl_xor_sync(0xffffffffu, wide, k);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, k);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, k);
+      }
+      // (s2, s1 exact when every |b| <= 45)
+      if ((int64_t)s2 + 2ll * kNarrowA * s1 >= kExactSum) wide = 1;
+      const int64_t j = t / a.tiles_m * kQN + row;
+      if (quad == 0) {
+        cls[buf * kQN + row] = j < a.H && !wide;
+        if (j < a.H && t % a.tiles_m == 0) {
+          a.hwide[j] = wide;
+          if (wide) a.wh_list[atomicAdd(a.wh_count, 1)] = (int)j;
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&cls_full[buf]);
+    }
+  } else {
+    // ---------------- epilogue: warps 2..5, TMEM lane quarter = warp % 4
+    const int quarter = warp & 3;
+    const int row = quarter * 32 + lane;
+    uint32_t lt = 0;
+    for (int64_t t = blockIdx.x; t < a.items; t += gridDim.x) {
+      const uint32_t buf = lt & 1, use = lt >> 1;
+      ++lt;
+      const bool ready = __all_sync(
+          0xffffffffu, mbar_wait(&tfull[buf], use & 1, a.status, abort_flag) &&
+                           mbar_wait(&cls_full[buf], use & 1, a.status, abort_flag));
+      if (!ready) break;
+      tc_fence_after();
+      const int64_t i = t % a.tiles_m * kBM + row;
+      const bool row_ok = i < a.Q && a.nflags[i] == 0 && !a.nwide[i];
+      float thr = 0.0f;
+      int64_t asum = 0;
+      if (row_ok) {
+        asum = a.asum[i];
+        const int64_t thr_i = a.dtrue[i] - asum;
+        // fp16-class S values are integers with |S| < 2^24; clamping keeps S < thr exact
+        thr = (float)(thr_i > (1ll << 25) ? (1ll << 25) : (thr_i < -(1ll << 25) ? -(1ll << 25) : thr_i));
+      }
+      int cnt = 0;
+      unsigned long long bestk = kNoBestTc;
+      const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + buf * kQN;
+#pragma unroll 1
+      for (int c0 = 0; c0 < kQN; c0 += 32) {
+        uint32_t v[32];
+        tmem_ld32(taddr + c0, v);
+        const uint32_t in = __ballot_sync(0xffffffffu, cls[buf * kQN + c0 + lane] != 0);
+        const uint32_t vm = row_ok ? in : 0;
+        const int64_t j0 = t / a.tiles_m * kQN + c0;
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+          const float sv = __uint_as_float(v[e]);
+          const bool in_e = (vm >> e) & 1u;
+          cnt += (in_e && sv < thr);
+          if (in_e && sv <= thr) {
+            const unsigned long long dist = (unsigned long long)(asum + (int64_t)sv);
+            const unsigned long long key = (dist << 32) | (unsigned long long)(uint32_t)(j0 + e);
+            bestk = key < bestk ? key : bestk;
+          }
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tempty[buf]);
+      if (row_ok) {
+        if (cnt) atomicAdd(&a.rank[i], cnt);
+        if (bestk != kNoBestTc) atomicMin(&a.best[i], bestk);
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256));
+  }
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                   const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                                   const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-cudaError_t encode_map(CUtensorMap *map, const void *base, int64_t rows, int KT, int box_rows) {
+// Row-major 16-bit matrix [rows][KT] in boxes of 64 x box_rows, 128-byte swizzle.
+cudaError_t encode_map(CUtensorMap *map, const void *base, int64_t rows, int KT, int box_rows,
+                       bool half = true) {
   static EncodeTiledFn fn = nullptr;
   if (!fn) {
     cudaDriverEntryPointQueryResult q;
@@ -597,13 +938,16 @@ cudaError_t encode_map(CUtensorMap *map, const void *base, int64_t rows, int KT,
   cuuint64_t strides[1] = {(cuuint64_t)KT * 2};
   cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
-  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void *>(base), dims, strides,
+  CUresult r = fn(map, half ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, const_cast<void *>(base), dims, strides,
                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 }  // namespace
+
+// Most needles of a call that k_tc_query takes (measured above).
+constexpr int64_t kQueryNeedles = 512;
 
 bool tc_supported(int N) { return N == 8 || N == 16 || N == 32 || N == 64 || N == 128; }
 
@@ -650,8 +994,41 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
   const int *any = skip_tile ? any_tile : nullptr;
   k_tc_encode<<<blocks_for(Q), 256, 0, st>>>(tab, qscene, Q, N, 1, opa, nwide, wn_list, counts + 0,
                                              asum, nullptr, skip_tile, nullptr);
-  k_tc_encode<<<blocks_for(H), 256, 0, st>>>(tab, hscene, H, N, 0, opb, hwide, wh_list, counts + 1,
-                                             nullptr, hvalid, nullptr, any);
+  // few needles of one scene: the haystack's operands are built inside the GEMM kernel
+  const bool query = split_haystack && !skip_tile && !test_withhold && Q <= kQueryNeedles &&
+                     (reinterpret_cast<uintptr_t>(split_haystack) & 15) == 0;  // (TMA)
+  if (query) {
+    CUtensorMap mq, mp;
+    if ((e = encode_map(&mq, opa, Q, (int)KT, kBM)) != cudaSuccess) return e;
+    if ((e = encode_map(&mp, split_haystack, H, (int)(KT / 2), kQN, false)) != cudaSuccess) return e;
+    QueryArgs q;
+    q.Q = Q;
+    q.H = H;
+    q.N = N;
+    q.tiles_m = (int)((Q + kBM - 1) / kBM);
+    q.items = q.tiles_m * ((H + kQN - 1) / kQN);
+    q.nwide = nwide;
+    q.nflags = nflags;
+    q.asum = asum;
+    q.dtrue = dtrue;
+    q.rank = rank;
+    q.best = best;
+    q.hwide = hwide;
+    q.wh_list = wh_list;
+    q.wh_count = counts + 1;
+    q.status = status;
+    const size_t smem_q = 1024 + (kQRaw + 4 * kQOps) * kQTile + 512;
+    if ((e = cudaFuncSetAttribute(k_tc_query, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)smem_q)) != cudaSuccess)
+      return e;
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    k_tc_query<<<(unsigned)(q.items < sms ? q.items : sms), kQThreads, smem_q, st>>>(mq, mp, q);
+  } else {
+    k_tc_encode<<<blocks_for(H), 256, 0, st>>>(tab, hscene, H, N, 0, opb, hwide, wh_list,
+                                               counts + 1, nullptr, hvalid, nullptr, any);
+  }
   count_launches(2);
   if (split_haystack) {
     k_tc_encode_split<<<blocks_for(cap), 256, 0, st>>>(split_haystack, N, wh_list, counts + 1, cap,
@@ -693,8 +1070,10 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = (int)(tiles_total < sms ? tiles_total : sms);
-  k_tc_rank<<<grid, kTcThreads, smem, st>>>(ma, mb, a);
-  count_launches(1);
+  if (!query) {
+    k_tc_rank<<<grid, kTcThreads, smem, st>>>(ma, mb, a);
+    count_launches(1);
+  }
   if (split_haystack) {
     // the needles' tiles against the compacted split-square images (count on the device)
     if ((e = encode_map(&mb, ops, cap, (int)(KT / 2 * 3), kBN)) != cudaSuccess) return e;
