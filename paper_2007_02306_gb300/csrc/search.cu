@@ -321,7 +321,7 @@ __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
 
 // Narrow x narrow pairs.  Block: kTQ needles (deltas + masks in shared memory) x
 // kDenseThreads * kImg haystack images (kImg per thread, in consecutive groups of 32).
-template <int N, int kTQ, int kImg, bool kCount>
+template <int N, int kTQ, int kImg, bool kCount, bool kCounted>
 __global__ void __launch_bounds__(kDenseThreads, (N * kImg <= 64 ? 4 : 2) * 256 / kDenseThreads)
     k_dense(
     const int8_t *__restrict__ ndelta, const int8_t *__restrict__ nmask,
@@ -330,10 +330,11 @@ __global__ void __launch_bounds__(kDenseThreads, (N * kImg <= 64 ? 4 : 2) * 256 
     const int *__restrict__ hwide, int64_t H, const int64_t *__restrict__ dtrue,
     const int *__restrict__ nflags, int *__restrict__ rank, unsigned long long *__restrict__ best,
     unsigned long long *__restrict__ counters, int64_t tile0, int64_t tiles_q, int64_t tiles_h,
-    int64_t band_h, const int *__restrict__ hcount, const int *__restrict__ hmap,
-    const int *__restrict__ gate) {
-  // hcount (optional): the haystack holds *hcount images (H is then an upper bound); hmap
-  // (optional): haystack image j is image hmap[j] of the caller's haystack (a compacted subset);
+    int64_t band_h, int64_t blocks, const int *__restrict__ hcount,
+    const int *__restrict__ hmap, const int *__restrict__ gate) {
+  // kCounted: the haystack holds *hcount images (H is an upper bound), usually far fewer, so the grid
+  // is bounded and its blocks step through the `blocks` work items (a grid for H took 0.1-0.2 ms to
+  // find nothing to do in 131,072 blocks); otherwise one block per item.  hmap (optional): haystack image j is image hmap[j] of the caller's haystack (a compacted subset);
   // gate (optional): *gate == 0 means no needle is ranked here, and every block returns at once
   constexpr int WPR = N / 4;  // 32-bit words per row
   constexpr int K = N * N;
@@ -350,15 +351,18 @@ __global__ void __launch_bounds__(kDenseThreads, (N * kImg <= 64 ? 4 : 2) * 256 
   // haystack tiles of one band; consecutive blocks take consecutive needle tiles of the same band,
   // so a band's haystack images are read from DRAM once and reused from L2 by every needle tile,
   // and the needle tile's set-up (shared-memory fill, row order) is paid once per band.
-  const int64_t L = tile0 + blockIdx.x;
+  if (gate && *gate == 0) return;  // uniform over the grid
+  if (kCounted) H = *hcount < H ? *hcount : H;
+  int64_t L = tile0 + blockIdx.x;
+  do {
   const int64_t band = L / tiles_q, qt = L - band * tiles_q;
   const int64_t h0 = band * band_h;
   const int64_t h1 = tiles_h - h0 < band_h ? tiles_h : h0 + band_h;
   const int64_t q0 = qt * kTQ;
-  if (gate && *gate == 0) return;  // uniform over the grid
-  if (hcount) {
-    H = *hcount < H ? *hcount : H;
-    if (h0 * (int64_t)(kDenseThreads * kImg) >= H) return;  // uniform over the block
+  if (kCounted) {
+    // bands ascend: nothing is left for this block (uniform over the block)
+    if (h0 * (int64_t)(kDenseThreads * kImg) >= H) return;
+    __syncthreads();  // the item before is done with the shared arrays
   }
 
   bool act = false;
@@ -369,7 +373,7 @@ __global__ void __launch_bounds__(kDenseThreads, (N * kImg <= 64 ? 4 : 2) * 256 
     thr_s[tid] = t > 0x7fffffffll ? 0x7fffffff : (int)t;
     act_s[tid] = act;
   }
-  if (!__syncthreads_or(act)) return;  // no needle of this tile is ranked here
+  if (!__syncthreads_or(act)) continue;  // no needle of this tile is ranked here
   for (int x = tid; x < kTQ * (K / 4); x += kDenseThreads) {
     int q = x / (K / 4), wd = x - q * (K / 4);
     int a = 0, m = 0;
@@ -548,6 +552,7 @@ __global__ void __launch_bounds__(kDenseThreads, (N * kImg <= 64 ? 4 : 2) * 256 
       if (lane == 0 && lane_slots) atomicAdd(counters + 3, 32ull * lane_slots);
     }
   }
+  } while (kCounted && (L += gridDim.x) < blocks);
 }
 
 // Sparse-needle form.  Listing 1 only touches positions where the needle's delta is non-zero, so
@@ -806,11 +811,34 @@ __global__ void __launch_bounds__(kWideThreads) k_wide(
     if (pass != 1 && ch * kWideThreads >= sc.H) continue;     // uniform over the block
     const int64_t il = i - sc.qoff;
     const uint16_t *n = sc.needles + il * K;
-    // compact the needle's non-zero deltas (row-major order)
+    // compact the needle's non-zero deltas (any order: the sum is exact)
     __syncthreads();
     if (tid == 0) nnz_s = 0;
     __syncthreads();
-    for (int64_t base = 0; base < K; base += kWideThreads) {
+    if (rows_of_8(N)) {  // 256 pixels per warp and pass
+      const bool vec = aligned16(n);
+      for (int base = (tid >> 5) * 256; base < K; base += kWideThreads * 8) {
+        const int k0 = base + lane * 8;
+        int d[8];
+        deltas8(k0 < K ? load_pixels8(n, k0, vec) : make_uint4(0, 0, 0, 0), lane, N, d);
+        int c = 0;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) c += d[e] != 0;
+        int at = c;  // entries of the lanes up to this one
+#pragma unroll
+        for (int m = 1; m < 32; m <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, at, m);
+          if (lane >= m) at += y;
+        }
+        int wbase = 0;
+        if (lane == 31) wbase = atomicAdd(&nnz_s, at);
+        at += __shfl_sync(0xffffffffu, wbase, 31) - c;
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if (d[e] != 0) nz[at++] = make_int2(k0 + e, d[e]);
+      }
+    }
+    for (int64_t base = rows_of_8(N) ? K : 0; base < K; base += kWideThreads) {
       int k = (int)(base + tid);
       int a = 0;
       if (k < K) {
@@ -1072,7 +1100,10 @@ cudaError_t launch_dense(const int8_t *nd, const int8_t *nm, const int *nrs, con
   constexpr int kTQ = N <= 64 ? 4 : 2;  // N = 128: 64 KB of needle tile, two blocks per SM
   constexpr int kImg = N <= 64 ? 4 : 1;
   const size_t smem = sizeof(int2) * kTQ * (N * N / 4);
-  auto kern = counters ? k_dense<N, kTQ, kImg, true> : k_dense<N, kTQ, kImg, false>;
+  auto kern = hcount ? (counters ? k_dense<N, kTQ, kImg, true, true>
+                                 : k_dense<N, kTQ, kImg, false, true>)
+                     : (counters ? k_dense<N, kTQ, kImg, true, false>
+                                 : k_dense<N, kTQ, kImg, false, false>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int64_t th = (H + kDenseThreads * kImg - 1) / (kDenseThreads * kImg);
@@ -1084,11 +1115,11 @@ cudaError_t launch_dense(const int8_t *nd, const int8_t *nm, const int *nrs, con
   int64_t band_h = th * tq / ((int64_t)sms * 2 * 4);
   band_h = band_h < 1 ? 1 : (band_h > kBandMax ? kBandMax : band_h);
   const int64_t total = (th + band_h - 1) / band_h * tq;
-  constexpr int64_t kMaxGrid = 0x7fffffffll;
-  for (int64_t t0 = 0; t0 < total; t0 += kMaxGrid) {
+  const int64_t kMaxGrid = hcount ? (int64_t)sms * 32 : 0x7fffffffll;
+  for (int64_t t0 = 0; t0 < total; t0 += hcount ? total : kMaxGrid) {
     const int64_t n = total - t0 < kMaxGrid ? total - t0 : kMaxGrid;
     kern<<<(unsigned)n, kDenseThreads, smem, st>>>(nd, nm, nrs, nw, Q, hd, hw, H, dt, nf, rank,
-                                                   best, counters, t0, tq, th, band_h, hcount,
+                                                   best, counters, t0, tq, th, band_h, total, hcount,
                                                    hmap, gate);
     count_launches(1);
   }
@@ -1167,6 +1198,7 @@ int64_t search_batch_workspace_bytes(int num_scenes, int64_t Q, int64_t H, int N
   c.take<int>(mid ? H : 0);      // images of neither tensor-core class
   c.take<int8_t>(autom ? (H + 31) / 32 * 32 * K : 0);  // word-major haystack of the sparse form
   c.take<uint32_t>(autom ? (H + 127) / 128 * 4 : 0);  // its int8 class, a bit per image
+  c.take<int>(autom ? H : 0);      // the images outside it
   c.take<int>(autom ? 3 * Q : 0);  // per-needle choice and the two exclusions
   c.take<int>(autom ? Q / 128 + 2 : 0);  // tensor-core needle tiles to skip
   return c.off + 256;
@@ -1232,6 +1264,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   int *left_list = c.take<int>(mid ? H : 0);
   int8_t *hword = c.take<int8_t>(autom ? (H + 31) / 32 * 32 * K : 0);
   uint32_t *auto_narrow = c.take<uint32_t>(autom ? (H + 127) / 128 * 4 : 0);
+  int *auto_list = c.take<int>(autom ? H : 0);
   int *auto_n = c.take<int>(autom ? 3 * Q : 0);
   int *skip_tile = c.take<int>(autom ? Q / 128 + 2 : 0);
   int *sparse_of = autom ? auto_n : nullptr;
@@ -1264,11 +1297,11 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
                                 (int)wide_smem)) != cudaSuccess)
     return e;
   auto wide = [&](int pass, const int *sub_list = nullptr, const int *sub_count = nullptr,
-                  const int *list = nullptr) {
+                  const int *list = nullptr, const int *list_count = nullptr) {
     k_wide<<<152 * 8, kWideThreads, wide_smem, st>>>(tab, qscene, hscene, Q, b.Hmax, N, pass,
                                                    nwide, wn_list, counts + 0,
                                                    list ? list : wh_list,
-                                                   counts + 1, dt, nflags, rank, best, t1flag, cnt,
+                                                   list_count ? list_count : counts + 1, dt, nflags, rank, best, t1flag, cnt,
                                                    sub_list, sub_count);
     count_launches(1);
   };
@@ -1306,6 +1339,10 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
       count_launches(1);
     }
     if (autom) {
+      // the haystack of the sparse-needle form; its list of the images outside int8 also serves the
+      // int64 pass below, so the tensor-core class encode has nothing to do when no needle is left
+      // for it
+      encode_words(hword, auto_narrow, auto_list, counts + 4);
       // each needle's form, decided before the tensor-core kernel runs
       k_sparse_needles<<<blocks_for(Q), 32 * wpb, 0, st>>>(nd, nm, Q, N, sent, scount);
       k_auto_assign<<<blocks_for(Q / 32 + 1), 256, 0, st>>>(scount, mid_nflag, Q, (int)(K / 4),
@@ -1331,15 +1368,15 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
       if ((e = run_dense(autom ? excl_dense : nwide, mid_hflag, counts + 6, left_list,
                          autom ? counts + 5 : nullptr)) != cudaSuccess)
         return e;
-      // the compacted encode listed its images outside the int8 class (compact indices)
-      wide(1, mid_list + Q, counts + 3, left_list);
+      // images outside the int8 class: AUTO's word encode has listed them, the compacted encode (as
+      // compact indices) those of its images
+      if (autom) wide(1, nullptr, nullptr, auto_list, counts + 4);
+      else wide(1, mid_list + Q, counts + 3, left_list);
     } else {
       wide(1);
     }
     if (autom) {
-      // the sparse-needle form for its needles against every int8-class image (the encode's list
-      // of images outside int8 goes to wh_list, whose readers above precede it on the stream)
-      encode_words(hword, auto_narrow, wh_list, counts + 4);
+      // the sparse-needle form for its needles against every int8-class image
       if ((e = launch_sparse(sent, scount, excl_sparse, Q, hword, auto_narrow, H, N, dt, nflags,
                              rank, best, cnt, st)) != cudaSuccess)
         return e;

@@ -194,9 +194,10 @@ __global__ void k_tc_encode(const SearchScene *__restrict__ tab, const int *__re
                             uint32_t *__restrict__ valid_mask, const int *__restrict__ skip_tile,
                             const int *__restrict__ any_tile) {
   const int lane = threadIdx.x & 31;
-  // operand rows no tile will load are not written (the classes are still computed): needle
-  // rows of skipped needle tiles, and every haystack row when no needle tile is left
+  // operand rows no tile will load are not written: needle rows of skipped needle tiles (their
+  // classes are still computed), and the haystack's when no needle tile is left
   const bool hay_written = needle_side || !any_tile || *any_tile != 0;
+  if (!hay_written) return;  // nor does anything read the haystack's classes then
   const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int K0 = N * N;
@@ -210,7 +211,7 @@ __global__ void k_tc_encode(const SearchScene *__restrict__ tab, const int *__re
     // with a wide delta; its operand row is garbage that no result reads)
     unsigned a2 = 0, s1 = 0;
     int wide = 0;
-    const bool write = needle_side ? !(skip_tile && skip_tile[i / kBM]) : hay_written;
+    const bool write = !(needle_side && skip_tile && skip_tile[i / kBM]);
     const bool vec = aligned16(img);
 #pragma unroll 4
     for (int base = 0; base < K0; base += 256) {
