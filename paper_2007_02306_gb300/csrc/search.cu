@@ -564,10 +564,8 @@ __global__ void __launch_bounds__(kDenseThreads, (N * kImg <= 64 ? 4 : 2) * 256 
 // The order decides only when a pair stops, never its result.
 constexpr int kSparseWarps = 8;   // needles per block, one per warp
 constexpr int kSparseImg = 4;     // haystack images per lane
-constexpr int kSparseStep = 2;    // needle words per step over the first kSparseHead words
-constexpr int kSparseHead = 4;
-constexpr int kSparseStepLong = 4;  // needle words per step after them (loads of a step are in
-                                    // flight together)
+constexpr int kSparseStepLong = 2;  // needle words per step after the first two (loads of a step are
+                                    // in flight together)
 constexpr int64_t kSparseBandMax = 64;  // haystack tiles per band of the sparse work order
 
 __device__ __forceinline__ int sparse_class(int wsq) {  // 0 = heaviest
@@ -628,23 +626,87 @@ __global__ void __launch_bounds__(256) k_sparse_needles(const int8_t *__restrict
 
 // Narrow needles x narrow haystack images over the needles' sparse entries.  Block: kSparseWarps
 // needles (one per warp) sweeping a band of haystack tiles of 32 * kSparseImg images; lane l of a
-// warp holds images j0 + l + 32 k.  Most pairs of sparse needles stop within a word or two, so the
-// first kSparseHead entries stay in shared memory for the whole band, the words of the first
-// kSparseStep of the next tile are loaded before the current tile is summed (one coalesced 128-byte
-// access per warp, entry and image slot), the images to rank come as one bit each, and a tile none
-// of whose images is left ends there.  Bound by the L2 gathers: at least 1 KB per warp and tile.
-// 16,384 sparse needles x 262,144 images: 11.8 -> 8.8 ms for the whole call (entries, class flags and
-// reductions per tile before).
-template <bool kCount>
+// warp holds images j0 + l + 32 k.  Most pairs of sparse needles stop within a word or two, so a tile
+// is decided by the needle's first two words where it can be: both stay in registers for the band,
+// their words of the next tile are loaded (one coalesced 128-byte access per entry and 32 images, at
+// constant distances from one running address) before the current tile is summed, and where every
+// image is narrow and none is left the tile ends at one vote.  Bound by instruction issue (as fast on
+// 32 x 32 images with a quarter of the words).  16,384 sparse needles x 262,144 images of 64 x 64, whole
+// calls: 7.8 ms with early loads alone, 4.4 ms with the constant distances and the single vote (64
+// registers, four blocks per SM; three 5.2 ms).  Groups held in shared memory instead of gathers
+// were slower (+0.8 ms), as was deciding by one word (+0.65 ms).
+// The images of a tile that the needle's first two words leave: the further entries, kSparseStepLong
+// per step with their loads in flight together, then the count and the minimum.  Warp collective;
+// returns the words this lane evaluated.  (Inlined: as a call it spilled the sweep's registers.)
+template <int N, bool kCount>
+__device__ __forceinline__ unsigned long long sparse_rest(const int8_t *tile, const int4 *e, int ne,
+                                                       int4 acc4, unsigned alive, int thr, int j0,
+                                                       int *rank, unsigned long long *best,
+                                                       unsigned long long &lane_slots) {
+  constexpr int kGroup = N * N / 4 * 128;
+  const int lane = threadIdx.x & 31;
+  int acc[kSparseImg] = {acc4.x, acc4.y, acc4.z, acc4.w};
+  unsigned long long pair_words = 0;
+  for (int i = 2; i < ne; i += kSparseStepLong) {
+    if (__ballot_sync(0xffffffffu, alive != 0) == 0) return pair_words;
+    if (kCount) {
+      const int n = ne - i < kSparseStepLong ? ne - i : kSparseStepLong;
+      pair_words += (unsigned long long)__popc(alive) * n;
+      lane_slots += (unsigned long long)kSparseImg * n;
+    }
+    int4 E[kSparseStepLong];
+#pragma unroll
+    for (int u = 0; u < kSparseStepLong; ++u) E[u] = i + u < ne ? e[i + u] : make_int4(0, 0, 0, 0);
+    int w[kSparseStepLong][kSparseImg];
+#pragma unroll
+    for (int u = 0; u < kSparseStepLong; ++u)
+#pragma unroll
+      for (int k = 0; k < kSparseImg; ++k)
+        w[u][k] =
+            (alive >> k) & 1u ? *reinterpret_cast<const int *>(tile + E[u].z + k * kGroup) : 0;
+#pragma unroll
+    for (int u = 0; u < kSparseStepLong; ++u)
+#pragma unroll
+      for (int k = 0; k < kSparseImg; ++k) {
+        const int bm = w[u][k] & E[u].y;
+        acc[k] = __dp4a(bm, bm, acc[k] + E[u].w) - 2 * __dp4a(E[u].x, w[u][k], 0);
+      }
+#pragma unroll
+    for (int k = 0; k < kSparseImg; ++k)
+      if (acc[k] > 0) alive &= ~(1u << k);  // images that have exited keep stale sums
+  }
+  if (__ballot_sync(0xffffffffu, alive != 0) == 0) return pair_words;
+  int c = 0;
+  unsigned long long bb = kNoBest;
+#pragma unroll
+  for (int k = 0; k < kSparseImg; ++k) {
+    const bool fin = (alive >> k) & 1u;
+    c += fin && acc[k] < 0;
+    const unsigned long long bk = fin ? pack_best(acc[k] + thr, j0 + 32 * k) : kNoBest;
+    bb = bk < bb ? bk : bb;
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) c += __shfl_down_sync(0xffffffffu, c, d);
+  bb = warp_min_u64(bb);
+  if (lane == 0) {
+    if (c) atomicAdd(rank, c);
+    if (bb != kNoBest) atomicMin(best, bb);
+  }
+  return pair_words;
+}
+
+template <int N, bool kCount>
 __global__ void __launch_bounds__(kSparseWarps * 32, 4) k_sparse(
     const int4 *__restrict__ ent, const int *__restrict__ ecount,
     const int *__restrict__ nwide, int64_t Q, const int8_t *__restrict__ hword,
-    const uint4 *__restrict__ narrow, int64_t H, int N, const int64_t *__restrict__ dtrue,
+    const uint4 *__restrict__ narrow, int64_t H, const int64_t *__restrict__ dtrue,
     const int *__restrict__ nflags, int *__restrict__ rank, unsigned long long *__restrict__ best,
     unsigned long long *__restrict__ counters, int64_t tile0, int64_t tiles_q, int64_t tiles_h,
     int64_t band_h) {
   constexpr int kTile = 32 * kSparseImg;
-  static_assert(kSparseImg == 4 && kSparseHead == 2 * kSparseStep, "one uint4 of image bits per tile");
+  static_assert(kSparseImg == 4, "one uint4 of image bits per tile");
+  constexpr int KW = N * N / 4;
+  constexpr int kGroup = KW * 128;  // bytes of a group of 32 images
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t L = tile0 + blockIdx.x;
   const int64_t band = L / tiles_q, qt = L - band * tiles_q;
@@ -654,121 +716,67 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 4) k_sparse(
   if (q >= Q || nflags[q] != 0 || nwide[q]) return;  // the whole warp leaves; no block barrier follows
   const int64_t tq = dtrue[q];
   const int thr = tq > 0x7fffffffll ? 0x7fffffff : (int)tq;
-  const int KW = N * N / 4;
   const int ne = ecount[q];
   const int4 *e = ent + q * (int64_t)KW;
-  const int64_t gbytes = (int64_t)KW * 128;  // one group of 32 images
-  const int64_t groups = (H + 31) / 32;
+  const int4 zero = make_int4(0, 0, 0, 0);  // a zero entry adds nothing
+  const int4 e0 = ne > 0 ? e[0] : zero, e1 = ne > 1 ? e[1] : zero;
+  const int start = e0.w + e1.w - thr;
   unsigned long long pair_words = 0, lane_slots = 0;
-  __shared__ int4 head_s[kSparseWarps][kSparseHead];
-  if (lane < kSparseHead)
-    head_s[warp][lane] = lane < ne ? e[lane] : make_int4(0, 0, 0, 0);  // a zero entry adds nothing
-  __syncwarp();
-  const int4 *const head = head_s[warp];
-  auto word = [&](const int8_t *hb, int k, int off) {
-    return *reinterpret_cast<const int *>(hb + k * gbytes + off);
-  };
-  auto base_of = [&](int64_t ht) { return hword + ht * kSparseImg * gbytes + lane * 4; };
-  // words of the first step's entries of a tile's images (groups past the haystack are not read)
-  auto fetch = [&](int64_t ht, int (&b)[kSparseStep][kSparseImg]) {
-    const int8_t *hb = base_of(ht);
+  // words of the first two entries of the next tile's images; the haystack is padded to whole tiles
+  const int8_t *at = hword + h0 * (int64_t)(kSparseImg * kGroup) + lane * 4;
+  int n0[kSparseImg], n1[kSparseImg];
+  auto fetch = [&]() {
+    const int8_t *p0 = at + e0.z, *p1 = at + e1.z;
 #pragma unroll
     for (int k = 0; k < kSparseImg; ++k) {
-      const bool in = ht * kSparseImg + k < groups;
-#pragma unroll
-      for (int u = 0; u < kSparseStep; ++u) b[u][k] = in ? word(hb, k, head[u].z) : 0;
+      n0[k] = *reinterpret_cast<const int *>(p0 + k * kGroup);
+      n1[k] = *reinterpret_cast<const int *>(p1 + k * kGroup);
     }
   };
-  int acc[kSparseImg] = {};  // partial distance minus the needle's true distance (exit once > 0)
-  // m (a - b)^2 over the word = sum a^2 + sum (m b)^2 - 2 sum a b
-  auto add = [&](int k, const int4 &E, int b) {
-    const int bm = b & E.y;
-    acc[k] = __dp4a(bm, bm, acc[k] + E.w) - 2 * __dp4a(E.x, b, 0);
-  };
-  int next[kSparseStep][kSparseImg];
-  fetch(h0, next);
+  fetch();
+  uint4 nbits = narrow[h0];
+#pragma unroll 2
   for (int64_t ht = h0; ht < h1; ++ht) {
-    const uint4 bits = narrow[ht];
-    int b[kSparseStep][kSparseImg];
-#pragma unroll
-    for (int u = 0; u < kSparseStep; ++u)
-#pragma unroll
-      for (int k = 0; k < kSparseImg; ++k) b[u][k] = next[u][k];
-    if (ht + 1 < h1) fetch(ht + 1, next);
-    unsigned alive = ((bits.x >> lane) & 1u) | (((bits.y >> lane) & 1u) << 1) |
-                     (((bits.z >> lane) & 1u) << 2) | (((bits.w >> lane) & 1u) << 3);
-    auto count = [&](int n) {
-      if (kCount && n > 0) {
-        pair_words += (unsigned long long)__popc(alive) * n;
-        lane_slots += (unsigned long long)kSparseImg * n;
-      }
-    };
-    auto leave = [&]() {  // images that have exited keep stale sums
-#pragma unroll
-      for (int k = 0; k < kSparseImg; ++k)
-        if (acc[k] > 0) alive &= ~(1u << k);
-    };
-    if (__ballot_sync(0xffffffffu, alive != 0) == 0) continue;
-    count(ne < kSparseStep ? ne : kSparseStep);
+    const uint4 bits = nbits;
+    int b0[kSparseImg], b1[kSparseImg];
 #pragma unroll
     for (int k = 0; k < kSparseImg; ++k) {
-      acc[k] = -thr;
-#pragma unroll
-      for (int u = 0; u < kSparseStep; ++u) add(k, head[u], b[u][k]);
+      b0[k] = n0[k];
+      b1[k] = n1[k];
     }
-    leave();
-    if (__ballot_sync(0xffffffffu, alive != 0) == 0) continue;
-    const int8_t *hb = base_of(ht);
-    if (ne > kSparseStep) {
-      count(ne < kSparseHead ? ne - kSparseStep : kSparseStep);
-#pragma unroll
-      for (int u = 0; u < kSparseStep; ++u)
-#pragma unroll
-        for (int k = 0; k < kSparseImg; ++k)
-          b[u][k] = (alive >> k) & 1u ? word(hb, k, head[kSparseStep + u].z) : 0;
-#pragma unroll
-      for (int k = 0; k < kSparseImg; ++k)
-#pragma unroll
-        for (int u = 0; u < kSparseStep; ++u) add(k, head[kSparseStep + u], b[u][k]);
-      leave();
+    const int8_t *tile = at;
+    if (ht + 1 < h1) {
+      at += kSparseImg * kGroup;
+      fetch();
+      nbits = narrow[ht + 1];
     }
-    // longer steps with more loads in flight for the pairs that go on
-    for (int e0 = kSparseHead; e0 < ne; e0 += kSparseStepLong) {
-      if (__ballot_sync(0xffffffffu, alive != 0) == 0) break;
-      count(ne - e0 < kSparseStepLong ? ne - e0 : kSparseStepLong);
-      int4 E[kSparseStepLong];
-#pragma unroll
-      for (int u = 0; u < kSparseStepLong; ++u)
-        E[u] = e0 + u < ne ? e[e0 + u] : make_int4(0, 0, 0, 0);
-      int w[kSparseStepLong][kSparseImg];
-#pragma unroll
-      for (int u = 0; u < kSparseStepLong; ++u)
-#pragma unroll
-        for (int k = 0; k < kSparseImg; ++k) w[u][k] = (alive >> k) & 1u ? word(hb, k, E[u].z) : 0;
-#pragma unroll
-      for (int u = 0; u < kSparseStepLong; ++u)
-#pragma unroll
-        for (int k = 0; k < kSparseImg; ++k) add(k, E[u], w[u][k]);
-      leave();
-    }
-    if (__ballot_sync(0xffffffffu, alive != 0) == 0) continue;
-    const int64_t j0 = ht * kTile + lane;
-    int c = 0;
-    unsigned long long bb = kNoBest;
+    // partial distance minus the needle's true distance (exit once > 0); per word m (a - b)^2 =
+    // sum a^2 + sum (m b)^2 - 2 sum a b
+    int acc[kSparseImg];
 #pragma unroll
     for (int k = 0; k < kSparseImg; ++k) {
-      const bool fin = (alive >> k) & 1u;
-      c += fin && acc[k] < 0;
-      const unsigned long long bk = fin ? pack_best(acc[k] + thr, j0 + 32 * k) : kNoBest;
-      bb = bk < bb ? bk : bb;
+      const int m0 = b0[k] & e0.y, m1 = b1[k] & e1.y;
+      acc[k] = __dp4a(m1, m1, __dp4a(m0, m0, start)) -
+               2 * __dp4a(e1.x, b1[k], __dp4a(e0.x, b0[k], 0));
     }
+    const bool some = min(min(acc[0], acc[1]), min(acc[2], acc[3])) <= 0;
+    if (kCount) {
+      const int n = ne < 2 ? ne : 2;
+      pair_words += (unsigned long long)n * (((bits.x >> lane) & 1u) + ((bits.y >> lane) & 1u) +
+                                             ((bits.z >> lane) & 1u) + ((bits.w >> lane) & 1u));
+      lane_slots += (unsigned long long)n * kSparseImg;
+    }
+    if (__ballot_sync(0xffffffffu, some) == 0) continue;
+    unsigned alive = 0;
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) c += __shfl_down_sync(0xffffffffu, c, d);
-    bb = warp_min_u64(bb);
-    if (lane == 0) {
-      if (c) atomicAdd(&rank[q], c);
-      if (bb != kNoBest) atomicMin(&best[q], bb);
+    for (int k = 0; k < kSparseImg; ++k) {
+      const unsigned w = k == 0 ? bits.x : (k == 1 ? bits.y : (k == 2 ? bits.z : bits.w));
+      if (acc[k] <= 0) alive |= ((w >> lane) & 1u) << k;
     }
+    const unsigned long long more =
+        sparse_rest<N, kCount>(tile, e, ne, make_int4(acc[0], acc[1], acc[2], acc[3]), alive, thr,
+                               (int)(ht * kTile) + lane, rank + q, best + q, lane_slots);
+    if (kCount) pair_words += more;
   }
   if (kCount) {  // lane_slots is the same in every lane of the warp
 #pragma unroll
@@ -1130,7 +1138,14 @@ cudaError_t launch_sparse(const int4 *ent, const int *ecount, const int *nw, int
                           const int8_t *hd, const uint32_t *narrow, int64_t H, int N,
                           const int64_t *dt, const int *nf, int *rank, unsigned long long *best,
                           unsigned long long *counters, cudaStream_t st) {
-  auto kern = counters ? k_sparse<true> : k_sparse<false>;
+  auto pick = [&](auto n) {
+    return counters ? k_sparse<decltype(n)::value, true> : k_sparse<decltype(n)::value, false>;
+  };
+  auto kern = N == 8    ? pick(std::integral_constant<int, 8>())
+              : N == 16 ? pick(std::integral_constant<int, 16>())
+              : N == 32 ? pick(std::integral_constant<int, 32>())
+              : N == 64 ? pick(std::integral_constant<int, 64>())
+                        : pick(std::integral_constant<int, 128>());
   const int64_t th = (H + 32 * kSparseImg - 1) / (32 * kSparseImg);
   const int64_t tq = (Q + kSparseWarps - 1) / kSparseWarps;
   int dev = 0, sms = 152;
@@ -1144,8 +1159,8 @@ cudaError_t launch_sparse(const int4 *ent, const int *ecount, const int *nw, int
   for (int64_t t0 = 0; t0 < total; t0 += kMaxGrid) {
     const int64_t n = total - t0 < kMaxGrid ? total - t0 : kMaxGrid;
     kern<<<(unsigned)n, kSparseWarps * 32, 0, st>>>(ent, ecount, nw, Q, hd,
-                                                    reinterpret_cast<const uint4 *>(narrow), H, N,
-                                                    dt, nf, rank,
+                                                    reinterpret_cast<const uint4 *>(narrow), H, dt,
+                                                    nf, rank,
                                                     best, counters, t0, tq, th, band_h);
     count_launches(1);
   }
@@ -1177,7 +1192,7 @@ int64_t search_batch_workspace_bytes(int num_scenes, int64_t Q, int64_t H, int N
   c.take<int8_t>(packed || mid ? Q * K : 0);  // needle deltas (CUDA-core forms)
   c.take<int8_t>(packed || mid ? Q * K : 0);  // needle masks
   c.take<int>((packed && !sparse) || mid ? Q * N : 0);  // needle row sums of squared deltas
-  c.take<int8_t>(packed || mid ? (H + 31) / 32 * 32 * K : 0);  // haystack deltas (groups of 32)
+  c.take<int8_t>(packed || mid ? (H + 127) / 128 * 128 * K : 0);  // haystack deltas (groups of 32)
   c.take<int>(Q);                        // needle wide flags
   c.take<int>(H + 4);                    // haystack wide flags (or, sparse form, a bit per image)
   c.take<int>(Q);                        // wide needle list
@@ -1196,7 +1211,7 @@ int64_t search_batch_workspace_bytes(int num_scenes, int64_t Q, int64_t H, int N
   c.take<int>(mid ? H : 0);      // int8 class flags of the compacted haystack images
   c.take<int>(mid ? Q + H : 0);  // lists written by its encodes
   c.take<int>(mid ? H : 0);      // images of neither tensor-core class
-  c.take<int8_t>(autom ? (H + 31) / 32 * 32 * K : 0);  // word-major haystack of the sparse form
+  c.take<int8_t>(autom ? (H + 127) / 128 * 128 * K : 0);  // word-major haystack of the sparse form
   c.take<uint32_t>(autom ? (H + 127) / 128 * 4 : 0);  // its int8 class, a bit per image
   c.take<int>(autom ? H : 0);      // the images outside it
   c.take<int>(autom ? 3 * Q : 0);  // per-needle choice and the two exclusions
@@ -1243,7 +1258,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   int8_t *nd = c.take<int8_t>(packed || mid ? Q * K : 0);
   int8_t *nm = c.take<int8_t>(packed || mid ? Q * K : 0);
   int *nrs = c.take<int>(dense || mid ? Q * N : 0);
-  int8_t *hd = c.take<int8_t>(packed || mid ? (H + 31) / 32 * 32 * K : 0);
+  int8_t *hd = c.take<int8_t>(packed || mid ? (H + 127) / 128 * 128 * K : 0);
   int *nwide = c.take<int>(Q);
   int *hwide = c.take<int>(H + 4);
   int *wn_list = c.take<int>(Q);
@@ -1262,7 +1277,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   int *mid_hflag = c.take<int>(mid ? H : 0);
   int *mid_list = c.take<int>(mid ? Q + H : 0);
   int *left_list = c.take<int>(mid ? H : 0);
-  int8_t *hword = c.take<int8_t>(autom ? (H + 31) / 32 * 32 * K : 0);
+  int8_t *hword = c.take<int8_t>(autom ? (H + 127) / 128 * 128 * K : 0);
   uint32_t *auto_narrow = c.take<uint32_t>(autom ? (H + 127) / 128 * 4 : 0);
   int *auto_list = c.take<int>(autom ? H : 0);
   int *auto_n = c.take<int>(autom ? 3 * Q : 0);
