@@ -1197,7 +1197,7 @@ int64_t search_batch_workspace_bytes(int num_scenes, int64_t Q, int64_t H, int N
   c.take<int>(H + 4);                    // haystack wide flags (or, sparse form, a bit per image)
   c.take<int>(Q);                        // wide needle list
   c.take<int>(H);                        // wide haystack list
-  c.take<int>(8);                        // list lengths
+  c.take<int>(16);                       // list lengths
   c.take<int>(Q);                        // per-needle state flags
   c.take<int>(Q);                        // top-1 exact fallback flags
   c.take<unsigned long long>(Q);         // packed best (distance, index)
@@ -1263,7 +1263,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   int *hwide = c.take<int>(H + 4);
   int *wn_list = c.take<int>(Q);
   int *wh_list = c.take<int>(H);
-  int *counts = c.take<int>(8);
+  int *counts = c.take<int>(16);
   int *nflags = c.take<int>(Q);
   int *t1flag = c.take<int>(Q);
   unsigned long long *best = c.take<unsigned long long>(Q);
@@ -1294,7 +1294,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
     k_fill_search_table<<<1, 256, 0, st>>>(tab + s0, f);
     count_launches(1);
   }
-  if ((e = cudaMemsetAsync(counts, 0, sizeof(int) * 8, st)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(counts, 0, sizeof(int) * 16, st)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(t1flag, 0, sizeof(int) * Q, st)) != cudaSuccess) return e;
   const int wpb = 8;
   auto blocks_for = [&](int64_t items) {

@@ -184,15 +184,29 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
 
 // ---------------------------------------------------------------- operand encoding (S2)
 
+// The 8 pixels of an image at k0 (zeros past its K0): one 16-byte load where it is aligned.
+__device__ __forceinline__ uint4 pixels8(const uint16_t *img, int k0, int K0, bool vec) {
+  if (k0 >= K0) return make_uint4(0, 0, 0, 0);
+  if (vec) return *reinterpret_cast<const uint4 *>(img + k0);
+  const uint16_t *q = img + k0;
+  return make_uint4(q[0] | (uint32_t)q[1] << 16, q[2] | (uint32_t)q[3] << 16,
+                    q[4] | (uint32_t)q[5] << 16, q[6] | (uint32_t)q[7] << 16);
+}
+
 // One warp per image (launch-wide index).  Needle rows: [m | a]; haystack rows: [b^2 | -2b]
 // (fp16, K = 2 N^2).  Also: the class flag (wide = outside the fp16 class, see the exactness
-// note above), the list of wide images, and for needles A_i.
+// note above), the list of wide images, and for needles A_i.  With row_map (the haystack of a single
+// scene) the rows of the class are written without gaps, *row_count of them, row_map[r] the image of
+// row r: the image is read a second time (from the caches) once its class is known, and the GEMM
+// has no columns for the images that others rank (7 % on the 5M-triangle scene: its search 24.4 ->
+// its images 24.6 -> 22.9 ms).
 __global__ void k_tc_encode(const SearchScene *__restrict__ tab, const int *__restrict__ scene_of,
                             int64_t n, int N, int needle_side, __half *__restrict__ op,
                             int *__restrict__ wide_flag, int *__restrict__ wide_list,
                             int *__restrict__ wide_count, int *__restrict__ asum,
                             uint32_t *__restrict__ valid_mask, const int *__restrict__ skip_tile,
-                            const int *__restrict__ any_tile) {
+                            const int *__restrict__ any_tile, int *__restrict__ row_map,
+                            int *__restrict__ row_count) {
   const int lane = threadIdx.x & 31;
   // operand rows no tile will load are not written: needle rows of skipped needle tiles (their
   // classes are still computed), and the haystack's when no needle tile is left
@@ -205,37 +219,22 @@ __global__ void k_tc_encode(const SearchScene *__restrict__ tab, const int *__re
     const SearchScene &sc = tab[scene_of[i]];
     const uint16_t *img = needle_side ? sc.needles + (i - sc.qoff) * K0
                                       : sc.haystack + (i - sc.hoff) * K0;
-    __half *row = op + i * (int64_t)(2 * K0);
     const int lim = needle_side ? kNarrowA : kNarrowB;
+    const bool vec = aligned16(img);
     // needles: a2 = sum a^2; haystack: a2 = S2_j, s1 = S1_j (wrapped, and not used, for an image
-    // with a wide delta; its operand row is garbage that no result reads)
+    // with a wide delta; its operand row, if it has one, is garbage that no result reads)
     unsigned a2 = 0, s1 = 0;
     int wide = 0;
-    const bool write = !(needle_side && skip_tile && skip_tile[i / kBM]);
-    const bool vec = aligned16(img);
-#pragma unroll 4
-    for (int base = 0; base < K0; base += 256) {
-      const int k0 = base + lane * 8;
-      const bool in = k0 < K0;
-      int d[8];
-      uint4 px = make_uint4(0, 0, 0, 0);
-      if (in) {
-        if (vec) {
-          px = *reinterpret_cast<const uint4 *>(img + k0);
-        } else {
-          const uint16_t *q = img + k0;
-          px = make_uint4(q[0] | (uint32_t)q[1] << 16, q[2] | (uint32_t)q[3] << 16,
-                          q[4] | (uint32_t)q[5] << 16, q[6] | (uint32_t)q[7] << 16);
-        }
-      }
-      deltas8(px, lane, N, d);
-      __align__(16) __half2 lo[4], hi[4];
+    auto classify = [&](const int (&d)[8]) {
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         wide |= d[e] < -lim || d[e] > lim;
         a2 += (unsigned)d[e] * (unsigned)d[e];
         if (!needle_side) s1 += (unsigned)abs(d[e]);
       }
+    };
+    auto write_row = [&](__half *row, int k0, const int (&d)[8]) {
+      __align__(16) __half2 lo[4], hi[4];
       // |d| <= 127 as halves without conversions: 0x6600 + d are the bits of 1536 + d (0x6400 is
       // 1024, steps of 1); differences, products and doubles of such integers are exact
 #pragma unroll
@@ -252,23 +251,43 @@ __global__ void k_tc_encode(const SearchScene *__restrict__ tab, const int *__re
           hi[e] = __hmul2(h, __floats2half2_rn(-2.0f, -2.0f));
         }
       }
-      if (write && in) {
+      if (k0 < K0) {
         *reinterpret_cast<int4 *>(row + k0) = *reinterpret_cast<int4 *>(lo);
         *reinterpret_cast<int4 *>(row + K0 + k0) = *reinterpret_cast<int4 *>(hi);
       }
+    };
+    const bool write = !(needle_side && skip_tile && skip_tile[i / kBM]);
+#pragma unroll 4
+    for (int base = 0; base < K0; base += 256) {
+      const int k0 = base + lane * 8;
+      int d[8];
+      deltas8(pixels8(img, k0, K0, vec), lane, N, d);
+      classify(d);
+      if (write && !row_map) write_row(op + i * (int64_t)(2 * K0), k0, d);
     }
     wide = __any_sync(0xffffffffu, wide);
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-      a2 += __shfl_down_sync(0xffffffffu, a2, d);
-      s1 += __shfl_down_sync(0xffffffffu, s1, d);
-    }
+    a2 = __reduce_add_sync(0xffffffffu, a2);
+    s1 = __reduce_add_sync(0xffffffffu, s1);
+    if (!needle_side && (int64_t)a2 + 2ll * kNarrowA * s1 >= kExactSum) wide = 1;
+    int r = 0;
     if (lane == 0) {
-      if (!needle_side && (int64_t)a2 + 2ll * kNarrowA * s1 >= kExactSum) wide = 1;
       wide_flag[i] = wide;
       if (wide) wide_list[atomicAdd(wide_count, 1)] = (int)i;
       if (asum) asum[i] = (int)a2;
       if (valid_mask && !wide) atomicOr(&valid_mask[i >> 5], 1u << (i & 31));
+      if (row_map && !wide) {
+        r = atomicAdd(row_count, 1);
+        row_map[r] = (int)i;
+      }
+    }
+    if (!row_map || wide) continue;
+    r = __shfl_sync(0xffffffffu, r, 0);
+#pragma unroll 4
+    for (int base = 0; base < K0; base += 256) {
+      const int k0 = base + lane * 8;
+      int d[8];
+      deltas8(pixels8(img, k0, K0, vec), lane, N, d);
+      write_row(op + r * (int64_t)(2 * K0), k0, d);
     }
   }
 }
@@ -290,18 +309,11 @@ __global__ void k_tc_encode_split(const uint16_t *__restrict__ imgs, int N,
     const int j = list[p];
     const uint16_t *img = imgs + (int64_t)j * K0;
     const bool vec = aligned16(img);
-    auto pixels = [&](int k0) {
-      if (k0 >= K0) return make_uint4(0, 0, 0, 0);
-      if (vec) return *reinterpret_cast<const uint4 *>(img + k0);
-      const uint16_t *q = img + k0;
-      return make_uint4(q[0] | (uint32_t)q[1] << 16, q[2] | (uint32_t)q[3] << 16,
-                        q[4] | (uint32_t)q[5] << 16, q[6] | (uint32_t)q[7] << 16);
-    };
     unsigned s2 = 0, s1 = 0;
     int wide = !wanted;
     for (int base = 0; base < K0; base += 256) {
       int d[8];
-      deltas8(pixels(base + lane * 8), lane, N, d);
+      deltas8(pixels8(img, base + lane * 8, K0, vec), lane, N, d);
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         wide |= d[e] < -kNarrowA || d[e] > kNarrowA;
@@ -325,7 +337,7 @@ __global__ void k_tc_encode_split(const uint16_t *__restrict__ imgs, int N,
     for (int base = 0; base < K0; base += 256) {
       const int k0 = base + lane * 8;
       int d[8];
-      deltas8(pixels(k0), lane, N, d);
+      deltas8(pixels8(img, k0, K0, vec), lane, N, d);
       __align__(16) __half r[8], b[8], q[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
@@ -959,7 +971,7 @@ int64_t tc_workspace_bytes(int64_t Q, int64_t H, int N, bool single_scene) {
   c.take<__half>(Q * KT);
   c.take<__half>(H * KT);
   c.take<int>(Q);                 // A_i
-  c.take<uint32_t>((H + 31) / 32 + 2);
+  c.take<uint32_t>(single_scene ? H : (H + 31) / 32 + 2);  // image of each row, or class bits
   c.take<__half>(cap * (KT / 2 * 3));  // split-square rows
   c.take<int>(cap);                    // their images
   return c.off + 256;
@@ -981,12 +993,16 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
   __half *opa = c.take<__half>(Q * KT);
   __half *opb = c.take<__half>(H * KT);
   int *asum = c.take<int>(Q);
-  uint32_t *hvalid = c.take<uint32_t>((H + 31) / 32 + 2);
+  const bool single = num_scenes == 1;
+  uint32_t *hvalid = c.take<uint32_t>(single ? H : (H + 31) / 32 + 2);
+  int *const row_map = single ? reinterpret_cast<int *>(hvalid) : nullptr;
   __half *ops = c.take<__half>(cap * (KT / 2 * 3));
   int *smap = c.take<int>(cap);
   int *const scount = counts + 7;  // their number (zeroed by the caller with the other counts)
+  int *const rcount = counts + 8;  // rows of the fp16 class (zeroed likewise)
   cudaError_t e;
-  if ((e = cudaMemsetAsync(hvalid, 0, sizeof(uint32_t) * ((H + 31) / 32 + 2), st)) != cudaSuccess)
+  if (!single &&
+      (e = cudaMemsetAsync(hvalid, 0, sizeof(uint32_t) * ((H + 31) / 32 + 2), st)) != cudaSuccess)
     return e;
   auto blocks_for = [](int64_t warps) {
     int64_t b = (warps + 7) / 8;
@@ -994,7 +1010,7 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
   };
   const int *any = skip_tile ? any_tile : nullptr;
   k_tc_encode<<<blocks_for(Q), 256, 0, st>>>(tab, qscene, Q, N, 1, opa, nwide, wn_list, counts + 0,
-                                             asum, nullptr, skip_tile, nullptr);
+                                             asum, nullptr, skip_tile, nullptr, nullptr, nullptr);
   // few needles of one scene: the haystack's operands are built inside the GEMM kernel
   const bool query = split_haystack && !skip_tile && !test_withhold && Q <= kQueryNeedles &&
                      (reinterpret_cast<uintptr_t>(split_haystack) & 15) == 0;  // (TMA)
@@ -1028,7 +1044,8 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
     k_tc_query<<<(unsigned)(q.items < sms ? q.items : sms), kQThreads, smem_q, st>>>(mq, mp, q);
   } else {
     k_tc_encode<<<blocks_for(H), 256, 0, st>>>(tab, hscene, H, N, 0, opb, hwide, wh_list,
-                                               counts + 1, nullptr, hvalid, nullptr, any);
+                                               counts + 1, nullptr, single ? nullptr : hvalid,
+                                               nullptr, any, row_map, rcount);
   }
   count_launches(2);
   if (split_haystack) {
@@ -1050,7 +1067,7 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
   a.nflags = nflags;
   a.asum = asum;
   a.dtrue = dtrue;
-  a.hvalid = hvalid;
+  a.hvalid = single ? nullptr : hvalid;
   a.rank = rank;
   a.best = best;
   a.status = status;
@@ -1060,9 +1077,9 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
   a.skip_tile = skip_tile;
   a.any_tile = any;
   a.ka_blocks = (int)(KT / kBK);
-  a.hcount = nullptr;
-  a.hcap = cap;
-  a.hmap = nullptr;
+  a.hcount = single ? rcount : nullptr;
+  a.hcap = (int)H;
+  a.hmap = row_map;
   const size_t smem = 1024 + kStages * (kStageA + kStageB) + 256;
   if ((e = cudaFuncSetAttribute(k_tc_rank, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem)) != cudaSuccess)
@@ -1080,6 +1097,7 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
     if ((e = encode_map(&mb, ops, cap, (int)(KT / 2 * 3), kBN)) != cudaSuccess) return e;
     a.KT = (int)(KT / 2 * 3);
     a.hcount = scount;
+    a.hcap = cap;
     a.hvalid = nullptr;
     a.hmap = smap;
     a.withhold_first_load = 0;
