@@ -33,7 +33,7 @@ def dev(a):
 
 @pytest.mark.parametrize("Q,H,N", [(1, 1, 2), (3, 7, 12), (5, 9, 8), (40, 40, 64), (9, 64, 64),
                                    (9, 65, 64), (7, 16, 128), (7, 17, 128), (256, 256, 32),
-                                   (257, 256, 32), (30, 257, 16), (100, 200, 33)])
+                                   (200, 257, 32), (30, 257, 16), (100, 200, 33)])
 @pytest.mark.parametrize("mode", [0, 6])
 def test_sizes(rici, oracle_mod, Q, H, N, mode):
     rng = np.random.default_rng(Q + H + N)
