@@ -139,6 +139,9 @@ struct Tuning {
 };
 Tuning current_tuning();
 
+// Scene of a launch-wide needle or haystack image (null: a single scene).
+__device__ __forceinline__ int scene_at(const int *scene, int64_t x) { return scene ? scene[x] : 0; }
+
 struct SearchBatch {
   int num_scenes;
   int64_t Qtot, Htot, Hmax, tiles_total;

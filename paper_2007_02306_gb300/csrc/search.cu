@@ -21,7 +21,7 @@
 //                   first; each broadcast needle word serves all of a thread's images.
 //   k_wide          pairs with a wide side: Listing 1 over the needle's non-zero deltas in
 //                   int64, reading the uint16 images.
-//   k_finalize / k_top1_exact   combine counts and top-1 candidates.
+//   k_finalize      combines counts and top-1 candidates.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -239,18 +239,20 @@ __device__ int64_t warp_crss(const uint16_t *n, const uint16_t *h, int N) {
   return (int64_t)__shfl_sync(0xffffffffu, s, 0);
 }
 
+// Also sets up each needle's rank, minimum and flags.
 __global__ void k_true_distance(const SearchScene *__restrict__ tab, const int *__restrict__ qscene,
                                 int64_t Qtot, int N, int64_t *__restrict__ dtrue,
                                 int *__restrict__ rank, unsigned long long *__restrict__ best,
-                                int *__restrict__ flags, int *status) {
+                                int *__restrict__ flags, int *__restrict__ top1_flag, int *status) {
   const int lane = threadIdx.x & 31;
   const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t K = (int64_t)N * N;
   for (int64_t i = w; i < Qtot; i += nw) {
-    const SearchScene &sc = tab[qscene[i]];
+    const SearchScene &sc = tab[scene_at(qscene, i)];
     const int64_t il = i - sc.qoff;
     const int64_t m = sc.match ? sc.match[il] : il;
+    if (lane == 0) top1_flag[i] = 0;
     if (m < 0 || m >= sc.H) {
       if (lane == 0) {
         set_status(status, RICI_ERR_INDEX_OUT_OF_RANGE);
@@ -296,12 +298,14 @@ __global__ void k_scene_index(const SearchScene *__restrict__ tab, int ns, int64
   }
 }
 
+constexpr int kCounts = 16;  // list lengths of a call, zeroed with its scene table
 constexpr int kFillChunk = 150;
 struct SearchFill {
   SearchScene e[kFillChunk];
   int n;
 };
-__global__ void k_fill_search_table(SearchScene *dst, SearchFill f) {
+__global__ void k_fill_search_table(SearchScene *dst, SearchFill f, int *counts, int ncounts) {
+  if (threadIdx.x < ncounts) counts[threadIdx.x] = 0;
   for (int i = threadIdx.x; i < f.n; i += blockDim.x) dst[i] = f.e[i];
 }
 
@@ -565,7 +569,8 @@ __global__ void __launch_bounds__(kDenseThreads, (N * kImg <= 64 ? 4 : 2) * 256 
 constexpr int kSparseWarps = 8;   // needles per block, one per warp
 constexpr int kSparseImg = 4;     // haystack images per lane
 constexpr int kSparseStepLong = 2;  // needle words per step after the first two (loads of a step are
-                                    // in flight together)
+                                    // in flight together; four spill the sweep's registers: 16,384
+                                    // sparse needles x 262,144 5.4 against 4.3 ms)
 constexpr int64_t kSparseBandMax = 64;  // haystack tiles per band of the sparse work order
 
 __device__ __forceinline__ int sparse_class(int wsq) {  // 0 = heaviest
@@ -635,42 +640,49 @@ __global__ void __launch_bounds__(256) k_sparse_needles(const int8_t *__restrict
 // calls: 7.8 ms with early loads alone, 4.4 ms with the constant distances and the single vote (64
 // registers, four blocks per SM; three 5.2 ms).  Groups held in shared memory instead of gathers
 // were slower (+0.8 ms), as was deciding by one word (+0.65 ms).
-// The images of a tile that the needle's first two words leave: the further entries, kSparseStepLong
+// The images of a tile that the needle's first two words leave: the further entries, 32 at a time
+// through shared memory (`stage`, one per lane; registers would hold a step's four), kSparseStepLong
 // per step with their loads in flight together, then the count and the minimum.  Warp collective;
 // returns the words this lane evaluated.  (Inlined: as a call it spilled the sweep's registers.)
 template <int N, bool kCount>
 __device__ __forceinline__ unsigned long long sparse_rest(const int8_t *tile, const int4 *e, int ne,
-                                                       int4 acc4, unsigned alive, int thr, int j0,
-                                                       int *rank, unsigned long long *best,
-                                                       unsigned long long &lane_slots) {
+                                                          int (&acc)[kSparseImg], unsigned alive,
+                                                          int thr, int j0, int4 *stage, int *rank,
+                                                          unsigned long long *best,
+                                                          unsigned long long &lane_slots) {
   constexpr int kGroup = N * N / 4 * 128;
   const int lane = threadIdx.x & 31;
-  int acc[kSparseImg] = {acc4.x, acc4.y, acc4.z, acc4.w};
   unsigned long long pair_words = 0;
   for (int i = 2; i < ne; i += kSparseStepLong) {
     if (__ballot_sync(0xffffffffu, alive != 0) == 0) return pair_words;
+    if (((i - 2) & 31) == 0) {
+      __syncwarp();
+      stage[lane] = i + lane < ne ? e[i + lane] : make_int4(0, 0, 0, 0);
+      __syncwarp();
+    }
+    const int4 *E = stage + ((i - 2) & 31);
     if (kCount) {
       const int n = ne - i < kSparseStepLong ? ne - i : kSparseStepLong;
       pair_words += (unsigned long long)__popc(alive) * n;
       lane_slots += (unsigned long long)kSparseImg * n;
     }
-    int4 E[kSparseStepLong];
-#pragma unroll
-    for (int u = 0; u < kSparseStepLong; ++u) E[u] = i + u < ne ? e[i + u] : make_int4(0, 0, 0, 0);
     int w[kSparseStepLong][kSparseImg];
 #pragma unroll
-    for (int u = 0; u < kSparseStepLong; ++u)
+    for (int u = 0; u < kSparseStepLong; ++u) {
+      const int8_t *p = tile + E[u].z;
 #pragma unroll
       for (int k = 0; k < kSparseImg; ++k)
-        w[u][k] =
-            (alive >> k) & 1u ? *reinterpret_cast<const int *>(tile + E[u].z + k * kGroup) : 0;
+        w[u][k] = (alive >> k) & 1u ? *reinterpret_cast<const int *>(p + k * kGroup) : 0;
+    }
 #pragma unroll
-    for (int u = 0; u < kSparseStepLong; ++u)
+    for (int u = 0; u < kSparseStepLong; ++u) {
+      const int4 x = E[u];
 #pragma unroll
       for (int k = 0; k < kSparseImg; ++k) {
-        const int bm = w[u][k] & E[u].y;
-        acc[k] = __dp4a(bm, bm, acc[k] + E[u].w) - 2 * __dp4a(E[u].x, w[u][k], 0);
+        const int bm = w[u][k] & x.y;
+        acc[k] = __dp4a(bm, bm, acc[k] + x.w) - 2 * __dp4a(x.x, w[u][k], 0);
       }
+    }
 #pragma unroll
     for (int k = 0; k < kSparseImg; ++k)
       if (acc[k] > 0) alive &= ~(1u << k);  // images that have exited keep stale sums
@@ -705,6 +717,7 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 4) k_sparse(
     int64_t band_h) {
   constexpr int kTile = 32 * kSparseImg;
   static_assert(kSparseImg == 4, "one uint4 of image bits per tile");
+  __shared__ int4 stage[kSparseWarps][32];
   constexpr int KW = N * N / 4;
   constexpr int kGroup = KW * 128;  // bytes of a group of 32 images
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -774,8 +787,8 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 4) k_sparse(
       if (acc[k] <= 0) alive |= ((w >> lane) & 1u) << k;
     }
     const unsigned long long more =
-        sparse_rest<N, kCount>(tile, e, ne, make_int4(acc[0], acc[1], acc[2], acc[3]), alive, thr,
-                               (int)(ht * kTile) + lane, rank + q, best + q, lane_slots);
+        sparse_rest<N, kCount>(tile, e, ne, acc, alive, thr, (int)(ht * kTile) + lane, stage[warp],
+                               rank + q, best + q, lane_slots);
     if (kCount) pair_words += more;
   }
   if (kCount) {  // lane_slots is the same in every lane of the warp
@@ -814,7 +827,7 @@ __global__ void __launch_bounds__(kWideThreads) k_wide(
     const int64_t qi = it / chunks, ch = it - qi * chunks;
     const int64_t i = pass == 0 ? wide_n_list[qi] : qi;
     if (nflags[i] != 0 || (pass == 1 && nwide[i])) continue;  // uniform over the block
-    const int si = qscene[i];
+    const int si = scene_at(qscene, i);
     const SearchScene &sc = tab[si];
     if (pass != 1 && ch * kWideThreads >= sc.H) continue;     // uniform over the block
     const int64_t il = i - sc.qoff;
@@ -867,7 +880,7 @@ __global__ void __launch_bounds__(kWideThreads) k_wide(
     if (pass == 1) {
       if (hj < nh) {
         const int64_t jg = wide_h_list[sub_list ? sub_list[hj] : hj];
-        if (hscene[jg] == si) jl = jg - sc.hoff;
+        if (scene_at(hscene, jg) == si) jl = jg - sc.hoff;
       }
     } else if (hj < sc.H) {
       jl = hj;
@@ -953,36 +966,41 @@ __global__ void k_auto_tiles(const int *__restrict__ excl_dense, int64_t Q, int6
   }
 }
 
-// Scene-local outputs: rank, true distance and top-1 (smallest index among minimal distances).
-__global__ void k_finalize(const SearchScene *__restrict__ tab, const int *__restrict__ qscene,
-                           int64_t Qtot, const int *__restrict__ rank,
-                           const int64_t *__restrict__ dtrue, const unsigned long long *__restrict__ best,
-                           const int *__restrict__ nflags) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Qtot;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const SearchScene &sc = tab[qscene[i]];
-    const int64_t il = i - sc.qoff;
-    sc.rank[il] = rank[i];
-    if (sc.dtrue) sc.dtrue[il] = dtrue[i];
-    if (sc.top1)
-      sc.top1[il] = (nflags[i] != 0 || best[i] == kNoBest)
-                        ? -1 : (int32_t)(uint32_t)(best[i] & 0xffffffffull);
-  }
-}
-
-// Needles whose best distance reached 2^32-1: exact (distance, index) minimum over the scene.
-__global__ void __launch_bounds__(256) k_top1_exact(const SearchScene *__restrict__ tab,
-                                                   const int *__restrict__ qscene, int64_t Qtot,
-                                                   int N, const int *__restrict__ top1_flag,
-                                                   const int *__restrict__ nflags) {
+// Scene-local outputs: rank, true distance and top-1 (smallest index among minimal distances).  A
+// needle whose best distance reached 2^32 - 1 gets its top-1 from the exact (distance, index) minimum
+// over the scene, by its block (one block per 256 needles).
+__global__ void __launch_bounds__(256) k_finalize(const SearchScene *__restrict__ tab,
+                                                  const int *__restrict__ qscene, int64_t Qtot,
+                                                  int N, const int *__restrict__ rank,
+                                                  const int64_t *__restrict__ dtrue,
+                                                  const unsigned long long *__restrict__ best,
+                                                  const int *__restrict__ nflags,
+                                                  const int *__restrict__ top1_flag) {
+  __shared__ int exact_s[256];
+  __shared__ int nexact;
   __shared__ long long bd[8];
   __shared__ long long bj[8];
   const int64_t K = (int64_t)N * N;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int64_t i = blockIdx.x; i < Qtot; i += gridDim.x) {
-    if (!top1_flag[i] || nflags[i]) continue;
-    const SearchScene &sc = tab[qscene[i]];
+  if (threadIdx.x == 0) nexact = 0;
+  __syncthreads();
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < Qtot) {
+    const SearchScene &sc = tab[scene_at(qscene, i)];
     const int64_t il = i - sc.qoff;
+    sc.rank[il] = rank[i];
+    if (sc.dtrue) sc.dtrue[il] = dtrue[i];
+    if (sc.top1) {
+      sc.top1[il] = (nflags[i] != 0 || best[i] == kNoBest)
+                        ? -1 : (int32_t)(uint32_t)(best[i] & 0xffffffffull);
+      if (top1_flag[i] && !nflags[i]) exact_s[atomicAdd(&nexact, 1)] = threadIdx.x;
+    }
+  }
+  __syncthreads();
+  for (int x = 0; x < nexact; ++x) {
+    const int64_t ie = blockIdx.x * (int64_t)blockDim.x + exact_s[x];
+    const SearchScene &sc = tab[scene_at(qscene, ie)];
+    const int64_t il = ie - sc.qoff;
     long long md = 0x7fffffffffffffffll, mj = -1;
     for (int64_t j = warp; j < sc.H; j += 8) {
       long long d = warp_crss(sc.needles + il * K, sc.haystack + j * K, N);
@@ -1003,7 +1021,7 @@ __global__ void __launch_bounds__(256) k_top1_exact(const SearchScene *__restric
           d0 = bd[w];
           j0 = bj[w];
         }
-      if (sc.top1) sc.top1[il] = (int32_t)j0;
+      sc.top1[il] = (int32_t)j0;
     }
     __syncthreads();
   }
@@ -1026,7 +1044,7 @@ __global__ void k_distances(const uint16_t *__restrict__ nimg, int64_t Q,
 
 // A whole small search of one scene in one launch: block i ranks needle i, one warp per pair, every
 // distance exact in int64 (so no classes, lists or fallbacks).
-constexpr int kSmallWarps = 8;
+constexpr int kSmallWarps = 16;
 __global__ void __launch_bounds__(kSmallWarps * 32) k_search_small(SearchScene sc, int N,
                                                                    int64_t *__restrict__ distances,
                                                                    int *status) {
@@ -1187,8 +1205,8 @@ int64_t search_batch_workspace_bytes(int num_scenes, int64_t Q, int64_t H, int N
   const bool mid = tensor && num_scenes == 1 && dense_supported(N);
   Carver c(nullptr);
   c.take<SearchScene>(num_scenes);
-  c.take<int>(Q);                        // scene of each needle
-  c.take<int>(H);                        // scene of each haystack image
+  c.take<int>(num_scenes == 1 ? 0 : Q);  // scene of each needle
+  c.take<int>(num_scenes == 1 ? 0 : H);  // scene of each haystack image
   c.take<int8_t>(packed || mid ? Q * K : 0);  // needle deltas (CUDA-core forms)
   c.take<int8_t>(packed || mid ? Q * K : 0);  // needle masks
   c.take<int>((packed && !sparse) || mid ? Q * N : 0);  // needle row sums of squared deltas
@@ -1197,7 +1215,7 @@ int64_t search_batch_workspace_bytes(int num_scenes, int64_t Q, int64_t H, int N
   c.take<int>(H + 4);                    // haystack wide flags (or, sparse form, a bit per image)
   c.take<int>(Q);                        // wide needle list
   c.take<int>(H);                        // wide haystack list
-  c.take<int>(16);                       // list lengths
+  c.take<int>(kCounts);                  // list lengths
   c.take<int>(Q);                        // per-needle state flags
   c.take<int>(Q);                        // top-1 exact fallback flags
   c.take<unsigned long long>(Q);         // packed best (distance, index)
@@ -1253,8 +1271,9 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   const bool mid = tensor && b.num_scenes == 1 && dense_supported(N);
   Carver c(ws);
   SearchScene *tab = c.take<SearchScene>(b.num_scenes);
-  int *qscene = c.take<int>(Q);
-  int *hscene = c.take<int>(H);
+  const bool single = b.num_scenes == 1;  // every image is of scene 0: no index arrays
+  int *qscene = single ? nullptr : c.take<int>(Q);
+  int *hscene = single ? nullptr : c.take<int>(H);
   int8_t *nd = c.take<int8_t>(packed || mid ? Q * K : 0);
   int8_t *nm = c.take<int8_t>(packed || mid ? Q * K : 0);
   int *nrs = c.take<int>(dense || mid ? Q * N : 0);
@@ -1263,7 +1282,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   int *hwide = c.take<int>(H + 4);
   int *wn_list = c.take<int>(Q);
   int *wh_list = c.take<int>(H);
-  int *counts = c.take<int>(16);
+  int *counts = c.take<int>(kCounts);
   int *nflags = c.take<int>(Q);
   int *t1flag = c.take<int>(Q);
   unsigned long long *best = c.take<unsigned long long>(Q);
@@ -1291,21 +1310,22 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
     SearchFill f;
     f.n = b.num_scenes - s0 < kFillChunk ? b.num_scenes - s0 : kFillChunk;
     for (int i = 0; i < f.n; ++i) f.e[i] = scenes[s0 + i];
-    k_fill_search_table<<<1, 256, 0, st>>>(tab + s0, f);
+    k_fill_search_table<<<1, 256, 0, st>>>(tab + s0, f, counts, kCounts);
     count_launches(1);
   }
-  if ((e = cudaMemsetAsync(counts, 0, sizeof(int) * 16, st)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(t1flag, 0, sizeof(int) * Q, st)) != cudaSuccess) return e;
   const int wpb = 8;
   auto blocks_for = [&](int64_t items) {
     int64_t nb = (items + wpb - 1) / wpb;
     return (int)(nb < 152 * 64 ? (nb > 0 ? nb : 1) : 152 * 64);
   };
-  k_scene_index<<<blocks_for((Q > H ? Q : H) / 32 + 1), 256, 0, st>>>(tab, b.num_scenes, Q, H,
-                                                                      qscene, hscene);
+  if (!single) {
+    k_scene_index<<<blocks_for((Q > H ? Q : H) / 32 + 1), 256, 0, st>>>(tab, b.num_scenes, Q, H,
+                                                                        qscene, hscene);
+    count_launches(1);
+  }
   k_true_distance<<<blocks_for(Q), 32 * wpb, 0, st>>>(tab, qscene, Q, N, dt, rank, best, nflags,
-                                                       b.status);
-  count_launches(2);
+                                                       t1flag, b.status);
+  count_launches(1);
   unsigned long long *cnt = reinterpret_cast<unsigned long long *>(b.counters);
   const size_t wide_smem = sizeof(int2) * (size_t)K;
   if ((e = cudaFuncSetAttribute(k_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1430,10 +1450,9 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
     if ((e = cudaMemsetAsync(nwide, 0, sizeof(int) * Q, st)) != cudaSuccess) return e;
     wide(2);
   }
-  k_finalize<<<blocks_for(Q * wpb), 256, 0, st>>>(tab, qscene, Q, rank, dt, best, nflags);
-  k_top1_exact<<<(int)(Q < 152 * 8 ? Q : 152 * 8), 256, 0, st>>>(tab, qscene, Q, N, t1flag,
-                                                                 nflags);
-  count_launches(2);
+  k_finalize<<<(unsigned)((Q + 255) / 256), 256, 0, st>>>(tab, qscene, Q, N, rank, dt, best, nflags,
+                                                          t1flag);
+  count_launches(1);
   if (out_distances && b.num_scenes == 1) {
     k_distances<<<blocks_for(Q * H), 32 * wpb, 0, st>>>(scenes[0].needles, Q, scenes[0].haystack,
                                                          H, N, out_distances);

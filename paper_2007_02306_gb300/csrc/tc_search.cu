@@ -216,7 +216,7 @@ __global__ void k_tc_encode(const SearchScene *__restrict__ tab, const int *__re
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int K0 = N * N;
   for (int64_t i = w; i < n; i += nw) {
-    const SearchScene &sc = tab[scene_of[i]];
+    const SearchScene &sc = tab[scene_at(scene_of, i)];
     const uint16_t *img = needle_side ? sc.needles + (i - sc.qoff) * K0
                                       : sc.haystack + (i - sc.hoff) * K0;
     const int lim = needle_side ? kNarrowA : kNarrowB;
