@@ -7,6 +7,7 @@ is no CPU fallback: if the library is missing or cannot be loaded the calls rais
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 import threading
@@ -79,6 +80,8 @@ def library_path() -> str:
 def load_library(path: str | None = None):
     """Load librici.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -157,13 +160,23 @@ def _check(rc: int):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream_handle(stream):
     if stream is None:
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
+
+
+_SAME_DEVICE = contextlib.nullcontext()
+
+
+def _on(device):
+    """The device of a call as the current one; nothing to do (and undo) where it is already."""
+    if device.index is None or device.index == torch.cuda.current_device():
+        return _SAME_DEVICE
+    return torch.cuda.device(device)
 
 
 def _need(t, dtype, name, shape_tail=None):
@@ -182,15 +195,15 @@ def _need(t, dtype, name, shape_tail=None):
 
 def workspace(device, nbytes: int) -> torch.Tensor:
     """Cached per-device scratch buffer (uint8, 256-byte aligned), grown on demand."""
-    dev = torch.device(device)
+    dev = device if isinstance(device, torch.device) else torch.device(device)
     key = dev.index if dev.index is not None else torch.cuda.current_device()
-    buf = _workspaces.get(key)
+    buf = _workspaces.get(key)  # the aligned part of the allocation, which it keeps alive
     if buf is None or buf.numel() < nbytes:
         _workspaces.pop(key, None)
         buf = torch.empty(max(int(nbytes), 256) + 256, dtype=torch.uint8, device=dev)
+        buf = buf[(-buf.data_ptr()) % 256:]
         _workspaces[key] = buf
-    off = (-buf.data_ptr()) % 256
-    return buf[off:]
+    return buf
 
 
 def release_workspaces() -> None:
@@ -224,7 +237,7 @@ def rici_generate(vertices, normals, triangles, origins, support_radius: float, 
     if nb < 0:
         raise ValueError("invalid sizes")
     ws = workspace(v.device, nb)
-    with torch.cuda.device(v.device):
+    with _on(v.device):
         _check(lib.rici_generate_ex(_ptr(v), _ptr(n), v.shape[0], _ptr(t), t.shape[0], _ptr(o),
                                     o.numel(), float(support_radius), N, _ptr(out), int(mode),
                                     _ptr(counters), _ptr(ws), ws.numel(), _stream_handle(stream)))
@@ -251,7 +264,7 @@ def clutter_areas(vertices, normals, triangles, origins, support_radius: float,
     if nb < 0:
         raise ValueError("invalid sizes")
     ws = workspace(v.device, nb)
-    with torch.cuda.device(v.device):
+    with _on(v.device):
         _check(lib.rici_clutter(_ptr(v), _ptr(n), v.shape[0], _ptr(t), t.shape[0], _ptr(o),
                                 o.numel(), float(support_radius), int(object_vertices),
                                 _ptr(a_all), _ptr(a_obj), _ptr(clu), _ptr(ws), ws.numel(),
@@ -281,7 +294,7 @@ def spin_images(vertices, normals, triangles, origins, support_radius: float, re
     if nb < 0:
         raise ValueError("invalid sizes")
     ws = workspace(v.device, nb)
-    with torch.cuda.device(v.device):
+    with _on(v.device):
         _check(lib.rici_spin_images(_ptr(v), _ptr(n), v.shape[0], _ptr(t), t.shape[0], _ptr(o),
                                     o.numel(), float(support_radius), N, int(samples_side),
                                     _ptr(out), _ptr(ws), ws.numel(), _stream_handle(stream)))
@@ -316,7 +329,7 @@ def crss_search(needles, haystack, true_match=None, *, mode: int = SEARCH_DEFAUL
     if nb < 0:
         raise ValueError("invalid sizes")
     ws = workspace(dev, nb)
-    with torch.cuda.device(dev):
+    with _on(dev):
         _check(lib.crss_search_ex(_ptr(q), Q, _ptr(h), H, N, _ptr(m), _ptr(rank), _ptr(dt),
                                   _ptr(top1), _ptr(dist), int(mode), _ptr(counters), _ptr(ws),
                                   ws.numel(), _stream_handle(stream)))
@@ -349,7 +362,7 @@ def rici_generate_batch(scenes, support_radius: float, resolution: int, *, works
     ws = workspace_tensor if workspace_tensor is not None else workspace(dev, nb)
     if ws.numel() < nb:
         raise ValueError(f"workspace_tensor needs {nb} bytes")
-    with torch.cuda.device(dev):
+    with _on(dev):
         _check(lib.rici_generate_batch(arr, len(scenes), float(support_radius), N, _ptr(ws),
                                        ws.numel(), _stream_handle(stream)))
     return outs
@@ -432,7 +445,7 @@ def batch_run(scenes, support_radius: float, resolution: int, *, mode: int = SEA
     tun = None
     if tuning is not None:
         tun = _Tuning(**{k: tuning[k] for k in TUNING_FIELDS})
-    with torch.cuda.device(dev):
+    with _on(dev):
         _check(lib.rici_batch_run_ex(arr, len(scenes), float(support_radius), N, int(mode),
                                      None if tun is None else ctypes.byref(tun), _ptr(ws),
                                      ws.numel(), _stream_handle(stream)))
@@ -477,7 +490,7 @@ def crss_search_batch(scenes, resolution: int, *, mode: int = SEARCH_TENSOR, wor
     ws = workspace_tensor if workspace_tensor is not None else workspace(dev, nb)
     if ws.numel() < nb:
         raise ValueError(f"workspace_tensor needs {nb} bytes")
-    with torch.cuda.device(dev):
+    with _on(dev):
         _check(lib.crss_search_batch(arr, len(scenes), N, int(mode), _ptr(ws), ws.numel(),
                                      _stream_handle(stream)))
     return res
@@ -593,7 +606,7 @@ def autotune_generate_batch(scenes, support_radius: float, resolution: int, *, r
     dev = outs[0].device if outs else torch.device("cuda")
     ws = workspace(dev, nb)
     best, ms = _Tuning(), ctypes.c_float(0.0)
-    with torch.cuda.device(dev):
+    with _on(dev):
         _check(lib.rici_autotune_generate_batch(arr, len(scenes), float(support_radius), N, _ptr(ws),
                                                 ws.numel(), _stream_handle(stream), int(repeats),
                                                 ctypes.byref(best), ctypes.byref(ms)))
@@ -611,7 +624,7 @@ def autotune_search_batch(scenes, resolution: int, *, repeats: int = 1, stream=N
     dev = scenes[0]["needles"].device if scenes else torch.device("cuda")
     ws = workspace(dev, nb)
     best, ms = _Tuning(), ctypes.c_float(0.0)
-    with torch.cuda.device(dev):
+    with _on(dev):
         _check(lib.rici_autotune_search_batch(arr, len(scenes), N, _ptr(ws), ws.numel(),
                                               _stream_handle(stream), int(repeats),
                                               ctypes.byref(best), ctypes.byref(ms)))
@@ -627,7 +640,7 @@ def project_fp32(points, spin_vertex, spin_normal, stream=None):
     if pts.dim() != 2 or pts.shape[1] != 3 or sv.numel() != 3 or sn.numel() != 3:
         raise ValueError("points must be [n, 3]; spin_vertex and spin_normal 3 floats")
     out = torch.empty_like(pts)
-    with torch.cuda.device(pts.device):
+    with _on(pts.device):
         _check(lib.rici_project_fp32(_ptr(pts), pts.shape[0], _ptr(sv), _ptr(sn), _ptr(out),
                                      _stream_handle(stream)))
     return out
