@@ -1042,6 +1042,41 @@ __global__ void k_distances(const uint16_t *__restrict__ nimg, int64_t Q,
   }
 }
 
+// Distances of one needle to kMany images, one warp: the needle's deltas once for all, sums in 32 bits
+// (all images 16-byte aligned with rows_of_8(N)).  Returns false where a sum could pass 2^31: K
+// (largest difference)^2 bounds it.
+constexpr int kMany = 4;
+__device__ __forceinline__ bool warp_crss_many(const uint16_t *n, const uint16_t *const (&h)[kMany],
+                                               int N, int64_t (&out)[kMany]) {
+  const int lane = threadIdx.x & 31, K = N * N;
+  unsigned s[kMany] = {}, bits = 0;
+  for (int base = 0; base < K; base += 256) {
+    const int k0 = base + lane * 8;
+    const bool in = k0 < K;
+    uint4 px[kMany];
+#pragma unroll
+    for (int m = 0; m < kMany; ++m)
+      px[m] = in ? load_pixels8(h[m], k0, true) : make_uint4(0, 0, 0, 0);
+    int a[8];
+    deltas8(in ? load_pixels8(n, k0, true) : make_uint4(0, 0, 0, 0), lane, N, a);
+#pragma unroll
+    for (int m = 0; m < kMany; ++m) {
+      int b[8];
+      deltas8(px[m], lane, N, b);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const unsigned x = a[e] != 0 ? (unsigned)abs(a[e] - b[e]) : 0u;
+        s[m] += x * x;
+        bits |= x;
+      }
+    }
+  }
+  bits = __reduce_or_sync(0xffffffffu, bits);
+#pragma unroll
+  for (int m = 0; m < kMany; ++m) out[m] = (int64_t)__reduce_add_sync(0xffffffffu, s[m]);
+  return (unsigned long long)bits * bits * (unsigned)K < (1ull << 31);
+}
+
 // A whole small search of one scene in one launch: block i ranks needle i, one warp per pair, every
 // distance exact in int64 (so no classes, lists or fallbacks).
 constexpr int kSmallWarps = 16;
@@ -1068,14 +1103,36 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_search_small(SearchScene s
   int cnt = 0;
   int64_t bd = INT64_MAX, bj = -1;
   if (valid || distances) {
-    for (int64_t j = warp; j < sc.H; j += kSmallWarps) {
-      const int64_t d = warp_crss(needle, sc.haystack + j * K, N);
-      cnt += d < dt;
-      if (d < bd) {  // j ascends: the smallest index of a minimum stays
-        bd = d;
-        bj = j;
+    const bool many = rows_of_8(N) && aligned16(needle) && aligned16(sc.haystack);
+    for (int64_t j0 = warp; j0 < sc.H; j0 += kMany * kSmallWarps) {
+      int64_t d[kMany];
+      const uint16_t *h[kMany];
+#pragma unroll
+      for (int m = 0; m < kMany; ++m) {  // (past the end: the last image again)
+        const int64_t j = j0 + m * kSmallWarps;
+        h[m] = sc.haystack + (j < sc.H ? j : sc.H - 1) * K;
       }
-      if (distances && lane == 0) distances[i * sc.H + j] = d;
+      if (!many || !warp_crss_many(needle, h, N, d)) {
+#pragma unroll 1
+        for (int m = 0; m < kMany; ++m) {
+          const int64_t j = j0 + m * kSmallWarps;
+          const int64_t x = warp_crss(needle, sc.haystack + (j < sc.H ? j : sc.H - 1) * K, N);
+#pragma unroll
+          for (int o = 0; o < kMany; ++o)
+            if (o == m) d[o] = x;
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < kMany; ++m) {
+        const int64_t j = j0 + m * kSmallWarps;
+        if (j >= sc.H) continue;
+        cnt += d[m] < dt;
+        if (d[m] < bd) {  // j ascends: the smallest index of a minimum stays
+          bd = d[m];
+          bj = j;
+        }
+        if (distances && lane == 0) distances[i * sc.H + j] = d[m];
+      }
     }
   }
   if (lane == 0) {
@@ -1102,8 +1159,8 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_search_small(SearchScene s
 // AUTO), no work counters, and so little work that launches decide.  A pair costs a warp about
 // 0.45 us and 0.11 us per 256 pixels, one after another, so the haystack is limited (256 images of up
 // to 32 x 32, 64 of 64 x 64, 16 of 128 x 128), and with it the work in all.  162 x 162 images of 32 x
-// 32 with the distance matrix: 114 us in the general sequence of 19 launches, 35 us here (most of
-// it the call's host side).  Past the limits it loses: 64 x 512 images of 32 x 32 80 against 93 us,
+// 32 with the distance matrix: 114 us in the general sequence of 19 launches, 29 us here.  With one
+// pair at a time per warp and 8 warps it lost past the limits: 64 x 512 images of 32 x 32 80 against 93 us,
 // 512 x 512 190 against 95 us, 16 x 2,048 of 16 x 16 146 against 85 us.
 bool small_search(const SearchBatch &b) {
   const int64_t K = (int64_t)b.N * b.N < 1024 ? 1024 : (int64_t)b.N * b.N;
