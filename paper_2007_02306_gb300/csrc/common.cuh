@@ -194,7 +194,8 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
 
 // Tensor-core search (tc_search.cu): operand encoding + persistent tcgen05 GEMM with the rank /
 // top-1 epilogue for narrow x narrow pairs of every scene.  Fills nwide/hwide and the wide
-// lists/counts (launch-wide indices).  With split_haystack (single scene): the haystack images outside
+// lists/counts (launch-wide indices).  With haystack (single scene) few needles take a kernel that reads its pixels
+// itself, and with split the haystack images outside
 // the fp16 class that only exceed its limit on one delta are ranked too, by a second GEMM with a
 // split square, and left_list / *left_count (zeroed before) receive the other ones.
 bool tc_supported(int N);
@@ -208,7 +209,7 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
                                       cudaStream_t st, const int *skip_needle = nullptr,
                                       const int *skip_tile = nullptr,
                                       const int *any_tile = nullptr,
-                                      const uint16_t *split_haystack = nullptr,
+                                      const uint16_t *haystack = nullptr, bool split = false,
                                       int *left_list = nullptr, int *left_count = nullptr);
 
 // Integer tensor-core search (i8_search.cu): int8 operand encoding + mma.sync s8 GEMM with the

@@ -804,9 +804,10 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 4) k_sparse(
 //   pass 0: needles = wide needle list, haystack = the needle's whole scene.
 //   pass 1: needles = all needles that are not wide, haystack = wide images of the same scene.
 //   pass 2: needles = all needles, haystack = the whole scene (reference path).
+// mode 0 runs passes 0 and 1 (in one launch), mode 2 pass 2.
 __global__ void __launch_bounds__(kWideThreads) k_wide(
     const SearchScene *__restrict__ tab, const int *__restrict__ qscene,
-    const int *__restrict__ hscene, int64_t Qtot, int64_t Hmax, int N, int pass,
+    const int *__restrict__ hscene, int64_t Qtot, int64_t Hmax, int N, int mode,
     const int *__restrict__ nwide, const int *__restrict__ wide_n_list,
     const int *__restrict__ wide_n_count, const int *__restrict__ wide_h_list,
     const int *__restrict__ wide_h_count, const int64_t *__restrict__ dtrue,
@@ -819,11 +820,14 @@ __global__ void __launch_bounds__(kWideThreads) k_wide(
   __shared__ int nnz_s;
   const int tid = threadIdx.x, lane = tid & 31;
   const int64_t K = (int64_t)N * N;
-  const int64_t nq = pass == 0 ? *wide_n_count : Qtot;
-  const int64_t nh = pass == 1 ? (sub_list ? *sub_count : *wide_h_count) : Hmax;
-  const int64_t chunks = (nh + kWideThreads - 1) / kWideThreads;
-  const int64_t items = nq * chunks;
-  for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+  const int64_t chunks_all = (Hmax + kWideThreads - 1) / kWideThreads;
+  const int64_t nh = mode == 0 ? (sub_list ? *sub_count : *wide_h_count) : 0;  // pass 1
+  const int64_t chunks_list = (nh + kWideThreads - 1) / kWideThreads;
+  const int64_t items0 = (mode == 0 ? *wide_n_count : Qtot) * chunks_all;
+  const int64_t items = items0 + (mode == 0 ? Qtot * chunks_list : 0);
+  for (int64_t it0 = blockIdx.x; it0 < items; it0 += gridDim.x) {
+    const int pass = mode == 2 ? 2 : (it0 < items0 ? 0 : 1);
+    const int64_t it = pass == 1 ? it0 - items0 : it0, chunks = pass == 1 ? chunks_list : chunks_all;
     const int64_t qi = it / chunks, ch = it - qi * chunks;
     const int64_t i = pass == 0 ? wide_n_list[qi] : qi;
     if (nflags[i] != 0 || (pass == 1 && nwide[i])) continue;  // uniform over the block
@@ -1352,7 +1356,13 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   int *mid_nflag = c.take<int>(mid ? Q : 0);
   int *mid_hflag = c.take<int>(mid ? H : 0);
   int *mid_list = c.take<int>(mid ? Q + H : 0);
+  // the images of neither tensor-core class; at 8 x 8 all outside the fp16 class: the second GEMM's
+  // two launches cost as much as the CUDA cores take for them (600 x 20,000: 133 us with them, 112
+  // without; 2,000 x 60,000: 508 us both)
+  const bool split = mid && N >= 16;
   int *left_list = c.take<int>(mid ? H : 0);
+  if (!split) left_list = wh_list;
+  int *const left_count = counts + (split ? 6 : 1);
   int8_t *hword = c.take<int8_t>(autom ? (H + 127) / 128 * 128 * K : 0);
   uint32_t *auto_narrow = c.take<uint32_t>(autom ? (H + 127) / 128 * 4 : 0);
   int *auto_list = c.take<int>(autom ? H : 0);
@@ -1388,13 +1398,15 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   if ((e = cudaFuncSetAttribute(k_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)wide_smem)) != cudaSuccess)
     return e;
-  auto wide = [&](int pass, const int *sub_list = nullptr, const int *sub_count = nullptr,
+  // int64 pairs: needles outside the class against everything and the others against the images
+  // outside it (mode 0), or every pair (mode 2)
+  auto wide = [&](int mode, const int *sub_list = nullptr, const int *sub_count = nullptr,
                   const int *list = nullptr, const int *list_count = nullptr) {
-    k_wide<<<152 * 8, kWideThreads, wide_smem, st>>>(tab, qscene, hscene, Q, b.Hmax, N, pass,
+    k_wide<<<152 * 8, kWideThreads, wide_smem, st>>>(tab, qscene, hscene, Q, b.Hmax, N, mode,
                                                    nwide, wn_list, counts + 0,
                                                    list ? list : wh_list,
-                                                   list_count ? list_count : counts + 1, dt, nflags, rank, best, t1flag, cnt,
-                                                   sub_list, sub_count);
+                                                   list_count ? list_count : counts + 1, dt, nflags,
+                                                   rank, best, t1flag, cnt, sub_list, sub_count);
     count_launches(1);
   };
   auto run_dense = [&](const int *nexcl, const int *hexcl, const int *hcount, const int *hmap,
@@ -1447,25 +1459,24 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
                                        tc_ws, nwide, hwide, wn_list, wh_list, counts, nflags, dt,
                                        rank, best, b.status, withhold, st, sparse_of,
                                        autom ? skip_tile : nullptr, counts + 5,
-                                       mid ? s0.haystack : nullptr, left_list, counts + 6)) !=
+                                       mid ? s0.haystack : nullptr, split, left_list, left_count)) !=
         cudaSuccess)
       return e;
-    wide(0);  // needles outside the fp16 class against the whole haystack (int64)
     if (mid) {
       // the haystack images of neither tensor-core class, compacted in list order (list and
       // count from the tensor-core encodes); narrow needles x those images on CUDA cores, and the
       // int64 kernel only for the compacted images outside the int8 class
-      encode_rows(hd, mid_hflag, mid_list + Q, counts + 3, left_list, counts + 6);
+      encode_rows(hd, mid_hflag, mid_list + Q, counts + 3, left_list, left_count);
       // (AUTO: counts[5] = 0 when no needle is left for the tensor-core side)
-      if ((e = run_dense(autom ? excl_dense : nwide, mid_hflag, counts + 6, left_list,
+      if ((e = run_dense(autom ? excl_dense : nwide, mid_hflag, left_count, left_list,
                          autom ? counts + 5 : nullptr)) != cudaSuccess)
         return e;
-      // images outside the int8 class: AUTO's word encode has listed them, the compacted encode (as
-      // compact indices) those of its images
-      if (autom) wide(1, nullptr, nullptr, auto_list, counts + 4);
-      else wide(1, mid_list + Q, counts + 3, left_list);
+      // needles outside the class, and images outside the int8 class: AUTO's word encode has listed
+      // these, the compacted encode (as compact indices) those of its images
+      if (autom) wide(0, nullptr, nullptr, auto_list, counts + 4);
+      else wide(0, mid_list + Q, counts + 3, left_list);
     } else {
-      wide(1);
+      wide(0);
     }
     if (autom) {
       // the sparse-needle form for its needles against every int8-class image
@@ -1479,7 +1490,6 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
                                        rank, best, st)) != cudaSuccess)
       return e;
     wide(0);
-    wide(1);
   } else if (dense) {
     // single scene: launch-wide indices are the scene's own
     const SearchScene &s0 = scenes[0];
@@ -1489,7 +1499,6 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
     encode_rows(hd, hwide, wh_list, counts + 1, nullptr, nullptr);
     if ((e = run_dense(nwide, hwide, nullptr, nullptr)) != cudaSuccess) return e;
     wide(0);
-    wide(1);
   } else if (sparse) {
     const SearchScene &s0 = scenes[0];
     k_encode_needles<<<blocks_for(Q), 32 * wpb, 0, st>>>(s0.needles, Q, N, nd, nm, nwide, wn_list,
@@ -1502,7 +1511,6 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
                            st)) != cudaSuccess)
       return e;
     wide(0);
-    wide(1);
   } else {
     if ((e = cudaMemsetAsync(nwide, 0, sizeof(int) * Q, st)) != cudaSuccess) return e;
     wide(2);

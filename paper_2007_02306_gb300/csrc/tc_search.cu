@@ -985,7 +985,7 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
                                       unsigned long long *best, int *status, int test_withhold,
                                       cudaStream_t st, const int *skip_needle,
                                       const int *skip_tile, const int *any_tile,
-                                      const uint16_t *split_haystack, int *left_list,
+                                      const uint16_t *haystack, bool split, int *left_list,
                                       int *left_count) {
   const int64_t KT = 2ll * N * N;
   const int cap = num_scenes == 1 ? split_capacity(H) : 0;
@@ -1012,12 +1012,12 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
   k_tc_encode<<<blocks_for(Q), 256, 0, st>>>(tab, qscene, Q, N, 1, opa, nwide, wn_list, counts + 0,
                                              asum, nullptr, skip_tile, nullptr, nullptr, nullptr);
   // few needles of one scene: the haystack's operands are built inside the GEMM kernel
-  const bool query = split_haystack && !skip_tile && !test_withhold && Q <= kQueryNeedles &&
-                     (reinterpret_cast<uintptr_t>(split_haystack) & 15) == 0;  // (TMA)
+  const bool query = haystack && !skip_tile && !test_withhold && Q <= kQueryNeedles &&
+                     (reinterpret_cast<uintptr_t>(haystack) & 15) == 0;  // (TMA)
   if (query) {
     CUtensorMap mq, mp;
     if ((e = encode_map(&mq, opa, Q, (int)KT, kBM)) != cudaSuccess) return e;
-    if ((e = encode_map(&mp, split_haystack, H, (int)(KT / 2), kQN, false)) != cudaSuccess) return e;
+    if ((e = encode_map(&mp, haystack, H, (int)(KT / 2), kQN, false)) != cudaSuccess) return e;
     QueryArgs q;
     q.Q = Q;
     q.H = H;
@@ -1048,8 +1048,8 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
                                                nullptr, any, row_map, rcount);
   }
   count_launches(2);
-  if (split_haystack) {
-    k_tc_encode_split<<<blocks_for(cap), 256, 0, st>>>(split_haystack, N, wh_list, counts + 1, cap,
+  if (split) {
+    k_tc_encode_split<<<blocks_for(cap), 256, 0, st>>>(haystack, N, wh_list, counts + 1, cap,
                                                        ops, smap, scount, left_list, left_count,
                                                        any);
     count_launches(1);
@@ -1092,7 +1092,7 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
     k_tc_rank<<<grid, kTcThreads, smem, st>>>(ma, mb, a);
     count_launches(1);
   }
-  if (split_haystack) {
+  if (split) {
     // the needles' tiles against the compacted split-square images (count on the device)
     if ((e = encode_map(&mb, ops, cap, (int)(KT / 2 * 3), kBN)) != cudaSuccess) return e;
     a.KT = (int)(KT / 2 * 3);
