@@ -50,7 +50,6 @@ constexpr uint32_t kStageB = kBN * kBK * 2;  // 32 KB
 constexpr int kNarrowA = 127;     // |delta| limit of fp16-class needles (int8)
 constexpr int kNarrowB = 45;      // |delta| limit of fp16-class haystack images (b^2 < 2^11)
 constexpr int64_t kExactSum = 1ll << 24;  // bound on every partial sum (exact FP32 integers)
-constexpr unsigned long long kNoBestTc = ~0ull;
 constexpr unsigned long long kWaitBudgetNs = 2000000000ull;
 constexpr unsigned long long kDrainBudgetNs = 200000000ull;
 
@@ -89,9 +88,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait for the phase with the given parity; false (and RICI_ERR_TIMEOUT) on timeout.
+// Bounded wait for the phase with the given parity; false (and RICI_ERR_TIMEOUT) on timeout.  The
+// waits between loads and MMAs poll without a pause: a stage is due every 300 ns, and waking up late
+// idles the tensor cores (8,192 x 262,144 images of 64 x 64: 22.9 -> 22.0 ms;
+// 100 x 90,001 in k_tc_query 321.8 -> 318.9 us).
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *status,
-                                          int *abort_flag) {
+                                          int *abort_flag, unsigned pause_ns = 32) {
   if (mbar_try_wait(bar, parity)) return true;
   const unsigned long long t0 = globaltimer();
   while (true) {
@@ -102,7 +104,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *s
       *(volatile int *)abort_flag = 1;
       return false;
     }
-    __nanosleep(32);
+    if (pause_ns) __nanosleep(pause_ns);
   }
 }
 
@@ -180,6 +182,77 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
         "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
       : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// ---------------------------------------------------------------- epilogue
+
+// One needle's row of an accumulator tile: S values are integers with |S| < 2^24 for images of the
+// class.  Counts S < thr, and keeps the smallest S up to lim with its smallest image index.
+//
+// lim starts from the best distance any tile has reported so far (or thr), so that after the first
+// tiles hardly a column passes it: 32 columns cost a minimum, a comparison and an addition each, and
+// are only looked at one by one when their minimum reaches lim in some lane.  With a 64-bit key per
+// column up to thr, some lane passed in nearly every column, and the four epilogue warps took 16,000
+// cycles per tile of 128 x 256 and bound the kernel below 32 x 32 pixels: 8,000 x 200,000 images of
+// 8 x 8 2.63 -> 0.68 ms, of 16 x 16 2.60 -> 0.66 ms (start of the best distance at thr: 1.25, 1.16).
+struct RowRank {
+  float thr, lim;
+  uint32_t j;  // image of the smallest S so far, ~0 if none
+  int count;
+};
+
+__device__ __forceinline__ float clamp_s(int64_t s) {  // exact below 2^24, beyond every S above
+  return (float)(s > (1ll << 25) ? (1ll << 25) : (s < -(1ll << 25) ? -(1ll << 25) : s));
+}
+
+// Rows that are not ranked get thr = lim = -infinity.
+__device__ __forceinline__ RowRank row_rank(bool row_ok, int64_t asum, const int64_t *dtrue,
+                                            const unsigned long long *best) {
+  RowRank r;
+  r.thr = r.lim = -__int_as_float(0x7f800000);
+  r.j = ~0u;
+  r.count = 0;
+  if (row_ok) {
+    r.thr = clamp_s(*dtrue - asum);
+    // (other blocks lower it meanwhile; any earlier value will do)
+    r.lim = fminf(r.thr, clamp_s((int64_t)(__ldcg(best) >> 32) - asum));
+  }
+  return r;
+}
+
+// Columns 0..31 of v, bit e of valid: column e is an image of the class; index(e) is its number.
+template <typename F>
+__device__ __forceinline__ void rank_columns(RowRank &r, uint32_t (&v)[32], uint32_t valid,
+                                             F index) {
+  if (valid != 0xffffffffu) {  // uniform over the warp
+#pragma unroll
+    for (int e = 0; e < 32; ++e)
+      if (!((valid >> e) & 1u)) v[e] = 0x7f800000u;  // +infinity
+  }
+  float m = __uint_as_float(v[0]);
+#pragma unroll
+  for (int e = 0; e < 32; ++e) {
+    m = fminf(m, __uint_as_float(v[e]));
+    r.count += __uint_as_float(v[e]) < r.thr;
+  }
+  if (m <= r.lim) {
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+      if (__uint_as_float(v[e]) == m) {
+        const uint32_t j = index(e);
+        if (m < r.lim || j < r.j) r.j = j;
+        r.lim = m;
+      }
+    }
+  }
+}
+
+// The row's results: count of smaller distances, smallest (distance, image).
+__device__ __forceinline__ void row_report(const RowRank &r, int64_t asum, int *rank,
+                                           unsigned long long *best) {
+  if (r.count) atomicAdd(rank, r.count);
+  if (r.j != ~0u)
+    atomicMin(best, ((unsigned long long)(asum + (int64_t)r.lim) << 32) | (unsigned long long)r.j);
 }
 
 // ---------------------------------------------------------------- operand encoding (S2)
@@ -462,7 +535,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const int ya = (int)(tt.qbeg + tt.m * kBM), yb = (int)(tt.hbeg + tt.n * kBN);
         for (int kb = 0; kb < kblocks; ++kb, ++it) {
           const uint32_t s = it % kStages, round = it / kStages;
-          if (!mbar_wait(&empty[s], (round & 1) ^ 1, a.status, abort_flag)) {
+          if (!mbar_wait(&empty[s], (round & 1) ^ 1, a.status, abort_flag, 0)) {
             ok = false;
             break;
           }
@@ -490,12 +563,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         if (a.skip_tile && a.skip_tile[tile_of(tab, a.num_scenes, t, a.group_m).m]) continue;
         const uint32_t buf = lt & 1, use = lt >> 1;
         ++lt;  // local count of processed tiles (selects the accumulator buffer)
-        if (!mbar_wait(&tempty[buf], (use & 1) ^ 1, a.status, abort_flag)) break;
+        if (!mbar_wait(&tempty[buf], (use & 1) ^ 1, a.status, abort_flag, 0)) break;
         tc_fence_after();
         const uint32_t tacc = tmem + buf * kBN;
         for (int kb = 0; kb < kblocks; ++kb, ++it) {
           const uint32_t s = it % kStages, round = it / kStages;
-          if (!mbar_wait(&full[s], round & 1, a.status, abort_flag)) {
+          if (!mbar_wait(&full[s], round & 1, a.status, abort_flag, 0)) {
             ok = false;
             break;
           }
@@ -533,54 +606,32 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       const int64_t i = tt.qbeg + il;         // launch-wide needle
       const bool row_ok = il < tt.Q && a.nflags[i] == 0 && !a.nwide[i] &&
                           !(a.skip_needle && a.skip_needle[i]);
-      float thr = 0.0f;
-      int64_t asum = 0, thr_i = 0;
-      if (row_ok) {
-        asum = a.asum[i];
-        thr_i = a.dtrue[i] - asum;
-        // fp16-class S values are integers with |S| < 2^24; clamping keeps S < thr exact
-        thr = (float)(thr_i > (1ll << 25) ? (1ll << 25) : (thr_i < -(1ll << 25) ? -(1ll << 25) : thr_i));
-      }
-      int cnt = 0;
-      unsigned long long bestk = kNoBestTc;
+      const int64_t asum = row_ok ? a.asum[i] : 0;
+      RowRank r = row_rank(row_ok, asum, a.dtrue + i, a.best + i);
       const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + buf * kBN;
 #pragma unroll 1
       for (int c0 = 0; c0 < kBN; c0 += 32) {
+        const int64_t j0 = tt.n * kBN + c0;  // scene-local haystack column
+        if (j0 >= tt.H) break;               // (uniform over the block)
         uint32_t v[32];
         tmem_ld32(taddr + c0, v);
-        const int64_t j0 = tt.n * kBN + c0;  // scene-local haystack column
-        uint32_t vm = 0;  // bit e: column j0 + e is a narrow haystack image of this scene
-        if (row_ok && j0 < tt.H) {
+        uint32_t vm = 0xffffffffu;  // bit e: column j0 + e is a narrow haystack image of this scene
+        if (a.hvalid) {
           const int64_t g0 = tt.hbeg + j0;   // launch-wide index (any alignment)
-          vm = 0xffffffffu;
-          if (a.hvalid) {
-            const uint32_t lo = a.hvalid[g0 >> 5], hi = a.hvalid[(g0 >> 5) + 1];
-            const int sh = (int)(g0 & 31);
-            vm = sh ? (lo >> sh) | (hi << (32 - sh)) : lo;
-          }
-          const int64_t rem = tt.H - j0;
-          if (rem < 32) vm &= (1u << rem) - 1u;
+          const uint32_t lo = a.hvalid[g0 >> 5], hi = a.hvalid[(g0 >> 5) + 1];
+          const int sh = (int)(g0 & 31);
+          vm = sh ? (lo >> sh) | (hi << (32 - sh)) : lo;
         }
-#pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          const float sv = __uint_as_float(v[e]);
-          const bool ok = (vm >> e) & 1u;
-          cnt += (ok && sv < thr);
-          if (ok && sv <= thr) {
-            const unsigned long long dist = (unsigned long long)(asum + (int64_t)sv);
-            const uint32_t j = a.hmap ? (uint32_t)a.hmap[j0 + e] : (uint32_t)(j0 + e);
-            const unsigned long long key = (dist << 32) | (unsigned long long)j;
-            bestk = key < bestk ? key : bestk;
-          }
-        }
+        const int64_t rem = tt.H - j0;
+        if (rem < 32) vm &= (1u << rem) - 1u;
+        rank_columns(r, v, vm, [&](int e) {
+          return a.hmap ? (uint32_t)a.hmap[j0 + e] : (uint32_t)(j0 + e);
+        });
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[buf]);
-      if (row_ok) {
-        if (cnt) atomicAdd(&a.rank[i], cnt);
-        if (bestk != kNoBestTc) atomicMin(&a.best[i], bestk);
-      }
+      if (row_ok) row_report(r, asum, a.rank + i, a.best + i);
     }
   }
 
@@ -611,7 +662,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // MMAs read 64 KB, 1,250 cycles at 128 bytes each against 1,376 measured (0.2 ms for 90,001 images of
 // 64 x 64 and a needle tile; their pixels alone take 0.11 ms of HBM).  Whole calls, operand rows
 // written by an encode and read by k_tc_rank against this kernel: 100 needles 715 -> 355 us, 256
-// 754 -> 554 us, 512 959 -> 916 us, 1,024 1,357 -> 1,712 us; 90,001 images of 32 x 32: 128 needles 262 ->
+// 754 -> 554 us, 512 959 -> 916 us, 1,024 1,357 -> 1,712 us (100 needles since, whole call: 319 us); 90,001 images of 32 x 32: 128 needles 262 ->
 // 147 us, 512 352 -> 305 us; so up to 512 needles take it.
 constexpr int kQN = 128;          // haystack images per tile
 constexpr int kQRaw = 3;          // pixel stages (16 KB)
@@ -697,7 +748,7 @@ __global__ void __launch_bounds__(kQThreads, 1)
         const int y = (int)(t / a.tiles_m * kQN);
         for (int c = 0; c < chunks; ++c, ++it) {
           const uint32_t s = it % kQRaw, round = it / kQRaw;
-          if (!mbar_wait(&px_empty[s], (round & 1) ^ 1, a.status, abort_flag)) {
+          if (!mbar_wait(&px_empty[s], (round & 1) ^ 1, a.status, abort_flag, 0)) {
             ok = false;
             break;
           }
@@ -717,7 +768,7 @@ __global__ void __launch_bounds__(kQThreads, 1)
         const int y = (int)(t % a.tiles_m * kBM);
         for (int c = 0; c < chunks; ++c, ++it) {
           const uint32_t s = it % kQOps, round = it / kQOps;
-          if (!mbar_wait(&op_empty[s], (round & 1) ^ 1, a.status, abort_flag)) {
+          if (!mbar_wait(&op_empty[s], (round & 1) ^ 1, a.status, abort_flag, 0)) {
             ok = false;
             break;
           }
@@ -737,13 +788,13 @@ __global__ void __launch_bounds__(kQThreads, 1)
       for (int64_t t = blockIdx.x; t < a.items && ok; t += gridDim.x) {
         const uint32_t buf = lt & 1, use = lt >> 1;
         ++lt;
-        if (!mbar_wait(&tempty[buf], (use & 1) ^ 1, a.status, abort_flag)) break;
+        if (!mbar_wait(&tempty[buf], (use & 1) ^ 1, a.status, abort_flag, 0)) break;
         tc_fence_after();
         const uint32_t tacc = tmem + buf * kQN;
         for (int c = 0; c < chunks; ++c, ++it) {
           const uint32_t s = it % kQOps, round = it / kQOps;
-          if (!mbar_wait(&a_full[s], round & 1, a.status, abort_flag) ||
-              !mbar_wait(&b_full[s], round & 1, a.status, abort_flag)) {
+          if (!mbar_wait(&a_full[s], round & 1, a.status, abort_flag, 0) ||
+              !mbar_wait(&b_full[s], round & 1, a.status, abort_flag, 0)) {
             ok = false;
             break;
           }
@@ -882,43 +933,21 @@ __global__ void __launch_bounds__(kQThreads, 1)
       tc_fence_after();
       const int64_t i = t % a.tiles_m * kBM + row;
       const bool row_ok = i < a.Q && a.nflags[i] == 0 && !a.nwide[i];
-      float thr = 0.0f;
-      int64_t asum = 0;
-      if (row_ok) {
-        asum = a.asum[i];
-        const int64_t thr_i = a.dtrue[i] - asum;
-        // fp16-class S values are integers with |S| < 2^24; clamping keeps S < thr exact
-        thr = (float)(thr_i > (1ll << 25) ? (1ll << 25) : (thr_i < -(1ll << 25) ? -(1ll << 25) : thr_i));
-      }
-      int cnt = 0;
-      unsigned long long bestk = kNoBestTc;
+      const int64_t asum = row_ok ? a.asum[i] : 0;
+      RowRank r = row_rank(row_ok, asum, a.dtrue + i, a.best + i);
       const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + buf * kQN;
 #pragma unroll 1
       for (int c0 = 0; c0 < kQN; c0 += 32) {
         uint32_t v[32];
         tmem_ld32(taddr + c0, v);
         const uint32_t in = __ballot_sync(0xffffffffu, cls[buf * kQN + c0 + lane] != 0);
-        const uint32_t vm = row_ok ? in : 0;
-        const int64_t j0 = t / a.tiles_m * kQN + c0;
-#pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          const float sv = __uint_as_float(v[e]);
-          const bool in_e = (vm >> e) & 1u;
-          cnt += (in_e && sv < thr);
-          if (in_e && sv <= thr) {
-            const unsigned long long dist = (unsigned long long)(asum + (int64_t)sv);
-            const unsigned long long key = (dist << 32) | (unsigned long long)(uint32_t)(j0 + e);
-            bestk = key < bestk ? key : bestk;
-          }
-        }
+        const uint32_t j0 = (uint32_t)(t / a.tiles_m * kQN + c0);
+        rank_columns(r, v, in, [&](int e) { return j0 + e; });
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[buf]);
-      if (row_ok) {
-        if (cnt) atomicAdd(&a.rank[i], cnt);
-        if (bestk != kNoBestTc) atomicMin(&a.best[i], bestk);
-      }
+      if (row_ok) row_report(r, asum, a.rank + i, a.best + i);
     }
   }
 
