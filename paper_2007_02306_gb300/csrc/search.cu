@@ -1356,10 +1356,11 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   int *mid_nflag = c.take<int>(mid ? Q : 0);
   int *mid_hflag = c.take<int>(mid ? H : 0);
   int *mid_list = c.take<int>(mid ? Q + H : 0);
-  // the images of neither tensor-core class; at 8 x 8 all outside the fp16 class: the second GEMM's
-  // two launches cost as much as the CUDA cores take for them (600 x 20,000: 133 us with them, 112
-  // without; 2,000 x 60,000: 508 us both)
-  const bool split = mid && N >= 16;
+  // the images of neither tensor-core class; in small searches of images below 32 x 32 all outside
+  // the fp16 class: the second GEMM's two launches cost more than the CUDA cores take for them there.
+  // With it against without, 8 x 8: 600 x 20,000 84 against 77 us, 2,000 x 60,000 182 against 196,
+  // 8,000 x 200,000 614 against 683; 16 x 16: 83 against 75, 193 against 184, 652 against 645
+  const bool split = mid && (N >= 32 || Q * H >= (1ll << 26));
   int *left_list = c.take<int>(mid ? H : 0);
   if (!split) left_list = wh_list;
   int *const left_count = counts + (split ? 6 : 1);

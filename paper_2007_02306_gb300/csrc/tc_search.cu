@@ -599,7 +599,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       const uint32_t buf = lt & 1, use = lt >> 1;
       ++lt;
       // warp-uniform outcome before the .sync.aligned TMEM loads
-      const bool ready = __all_sync(0xffffffffu, mbar_wait(&tfull[buf], use & 1, a.status, abort_flag));
+      const bool ready =
+          __all_sync(0xffffffffu, mbar_wait(&tfull[buf], use & 1, a.status, abort_flag));
       if (!ready) break;
       tc_fence_after();
       const int64_t il = tt.m * kBM + row;  // scene-local needle
@@ -662,8 +663,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // MMAs read 64 KB, 1,250 cycles at 128 bytes each against 1,376 measured (0.2 ms for 90,001 images of
 // 64 x 64 and a needle tile; their pixels alone take 0.11 ms of HBM).  Whole calls, operand rows
 // written by an encode and read by k_tc_rank against this kernel: 100 needles 715 -> 355 us, 256
-// 754 -> 554 us, 512 959 -> 916 us, 1,024 1,357 -> 1,712 us (100 needles since, whole call: 319 us); 90,001 images of 32 x 32: 128 needles 262 ->
-// 147 us, 512 352 -> 305 us; so up to 512 needles take it.
+// 754 -> 554 us, 512 959 -> 916 us, 1,024 1,357 -> 1,712 us; 90,001 images of 32 x 32: 128 needles
+// 262 -> 147 us, 512 352 -> 305 us; so up to 512 needles take it.  (100 needles since then: 319 us.)
 constexpr int kQN = 128;          // haystack images per tile
 constexpr int kQRaw = 3;          // pixel stages (16 KB)
 constexpr int kQOps = 2;          // operand stages (needles 32 KB, haystack 32 KB)
@@ -980,7 +981,8 @@ cudaError_t encode_map(CUtensorMap *map, const void *base, int64_t rows, int KT,
   cuuint64_t strides[1] = {(cuuint64_t)KT * 2};
   cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
-  CUresult r = fn(map, half ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, const_cast<void *>(base), dims, strides,
+  CUresult r = fn(map, half ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT16, 2,
+                  const_cast<void *>(base), dims, strides,
                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;

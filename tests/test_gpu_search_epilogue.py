@@ -32,3 +32,29 @@ def test_ties(oracle_mod, Q, H, N, kinds):
     assert rici.sync_status() == 0
     for k in ("rank", "true_distance", "top1"):
         assert np.array_equal(got[k].cpu().numpy(), ref[k]), k
+
+
+@pytest.mark.parametrize("N", [8, 16])
+@pytest.mark.parametrize("H", [(1 << 17) - 1, 1 << 17])
+@pytest.mark.parametrize("mode", [3, 6])
+def test_second_gemm_of_small_images(N, H, mode):
+    """Either side of 2^26 pairs, where images with wider deltas move from the CUDA cores to a second
+    GEMM; equal to the int64 form."""
+    import torch
+
+    import paper_2007_02306_gb300 as rici
+
+    Q = 512
+    g = torch.Generator().manual_seed(N + H)
+    hay = torch.randint(0, 12, (H, N, N), generator=g).to(torch.int32)
+    hay[::9, 1, N // 2:] += 60     # the split-square class
+    hay[5::4001, 2, 3] += 500      # outside int8
+    nd = hay[torch.randperm(H, generator=g)[:Q]].clone()
+    nd[::2, 0, 1] += 3
+    m = torch.randint(0, H, (Q,), generator=g)
+    nd, hay = nd.to(torch.uint16).cuda(), hay.to(torch.uint16).cuda()
+    a = rici.crss_search(nd, hay, m.cuda(), mode=mode)
+    b = rici.crss_search(nd, hay, m.cuda(), mode=rici.SEARCH_EXACT_SLOW)
+    assert rici.sync_status() == 0
+    for k in ("rank", "true_distance", "top1"):
+        assert torch.equal(a[k], b[k]), k
