@@ -73,7 +73,9 @@ MACS_PER_TERM = 2
 DP4A_PER_SM_CLK = 64
 # DRAM bytes (read + write) per full-size launch from one-pass ncu captures (commands in
 # profiles/); None where the kernel changed since it was captured
-TRAFFIC = {"k_generate_R0.6": None,
+# (k_generate at R = 0.6: 394.3 GB read + 6.6 GB written on the first 131,072 origins, scaled to the
+# full launch by 2,509,797 / 131,072 origins)
+TRAFFIC = {"k_generate_R0.6": (394.34e9 + 6.62e9) * 2509797 / 131072,
            "k_tc_rank_clutter": None, "k_dense_clutter": 1.895e9 + 5.57e6}
 
 
