@@ -1738,19 +1738,20 @@ __global__ void k_tri_area(const float4 *__restrict__ rec, int64_t rs, const int
   }
 }
 
-// Share of a triangle's area at heights in [-H, H], from its vertices' heights.
+// Share of a triangle's area at heights in [-H, H], from its vertices' heights.  The slab is closed: a
+// triangle that lies in an end plane is inside.
 __device__ double slab_share(double z0, double z1, double z2, double H) {
   const double lo = fmin(z0, fmin(z1, z2)), hi = fmax(z0, fmax(z1, z2));
   const double mid = fmax(fmin(z0, z1), fmin(fmax(z0, z1), z2));
-  // share below a height: quadratic on either side of the middle vertex
+  // share below a height between lo and hi: quadratic on either side of the middle vertex
   auto below = [&](double h) -> double {
-    if (h <= lo) return 0.0;
-    if (h >= hi) return 1.0;
     const double d = h <= mid ? h - lo : hi - h;
     const double f = d * d / ((h <= mid ? mid - lo : hi - mid) * (hi - lo));
     return h <= mid ? f : 1.0 - f;
   };
-  return below(H) - below(-H);
+  const double upper = H >= hi ? 1.0 : (H <= lo ? 0.0 : below(H));
+  const double lower = -H <= lo ? 0.0 : (-H >= hi ? 1.0 : below(-H));
+  return upper - lower;
 }
 
 // Area within the disk |x| <= R of the projection (onto (Tx, Ty)) of a triangle inside the slab,
