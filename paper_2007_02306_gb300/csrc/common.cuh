@@ -279,7 +279,7 @@ __device__ __forceinline__ void set_status(int *status, int bits) { atomicOr(sta
 __host__ __device__ constexpr bool rows_of_8(int N) {
   return N == 8 || N == 16 || N == 32 || N == 64 || N == 128;
 }
-__device__ __forceinline__ bool aligned16(const void *p) {
+__host__ __device__ __forceinline__ bool aligned16(const void *p) {
   return (reinterpret_cast<uintptr_t>(p) & 15) == 0;
 }
 

@@ -203,13 +203,16 @@ __global__ void __launch_bounds__(kGroupWarps * 32) k_encode_groups(
   }
 }
 
-// Exact int64 distance of one pair, one warp: 256 pixels per pass where both images can be read 8
-// at a time, else 32.
+// Exact int64 distance of one pair, one warp.  kRows (rows_of_8(N), both images 16-byte aligned): 256
+// pixels per pass, else 32.  Two instantiations, so that the kernels of the second form keep the few
+// registers of its loop (k_distances 31 against 42: 2,000 x 3,000 distances of 33 x 33 11.1 against
+// 14.8 ms with both in one).
+template <bool kRows>
 __device__ int64_t warp_crss(const uint16_t *n, const uint16_t *h, int N) {
   const int lane = threadIdx.x & 31;
   const int K = N * N;
   unsigned long long s = 0;
-  if (rows_of_8(N) && aligned16(n) && aligned16(h)) {
+  if constexpr (kRows) {
 #pragma unroll 4
     for (int base = 0; base < K; base += 256) {
       const int k0 = base + lane * 8;
@@ -240,6 +243,7 @@ __device__ int64_t warp_crss(const uint16_t *n, const uint16_t *h, int N) {
 }
 
 // Also sets up each needle's rank, minimum and flags.
+template <bool kRows>
 __global__ void k_true_distance(const SearchScene *__restrict__ tab, const int *__restrict__ qscene,
                                 int64_t Qtot, int N, int64_t *__restrict__ dtrue,
                                 int *__restrict__ rank, unsigned long long *__restrict__ best,
@@ -263,7 +267,7 @@ __global__ void k_true_distance(const SearchScene *__restrict__ tab, const int *
       }
       continue;
     }
-    int64_t d = warp_crss(sc.needles + il * K, sc.haystack + m * K, N);
+    int64_t d = warp_crss<kRows>(sc.needles + il * K, sc.haystack + m * K, N);
     if (lane == 0) {
       dtrue[i] = d;
       rank[i] = 0;
@@ -804,8 +808,11 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 4) k_sparse(
 //   pass 0: needles = wide needle list, haystack = the needle's whole scene.
 //   pass 1: needles = all needles that are not wide, haystack = wide images of the same scene.
 //   pass 2: needles = all needles, haystack = the whole scene (reference path).
-// mode 0 runs passes 0 and 1 (in one launch), mode 2 pass 2.
-__global__ void __launch_bounds__(kWideThreads) k_wide(
+// mode 0 runs passes 0 and 1 (in one launch), mode 2 pass 2.  kRows: rows_of_8(N).  Eight blocks per SM:
+// with 40 registers and six of them the rest of the grid came as a second wave (1,000 x 2,000 images
+// of 48 x 48 187 -> 158 us, of noise of 32 x 32 18.8 -> 14.6 ms with the exact top-1).
+template <bool kRows>
+__global__ void __launch_bounds__(kWideThreads, 8) k_wide(
     const SearchScene *__restrict__ tab, const int *__restrict__ qscene,
     const int *__restrict__ hscene, int64_t Qtot, int64_t Hmax, int N, int mode,
     const int *__restrict__ nwide, const int *__restrict__ wide_n_list,
@@ -840,7 +847,7 @@ __global__ void __launch_bounds__(kWideThreads) k_wide(
     __syncthreads();
     if (tid == 0) nnz_s = 0;
     __syncthreads();
-    if (rows_of_8(N)) {  // 256 pixels per warp and pass
+    if constexpr (kRows) {  // 256 pixels per warp and pass
       const bool vec = aligned16(n);
       for (int base = (tid >> 5) * 256; base < K; base += kWideThreads * 8) {
         const int k0 = base + lane * 8;
@@ -863,7 +870,7 @@ __global__ void __launch_bounds__(kWideThreads) k_wide(
           if (d[e] != 0) nz[at++] = make_int2(k0 + e, d[e]);
       }
     }
-    for (int64_t base = rows_of_8(N) ? K : 0; base < K; base += kWideThreads) {
+    for (int64_t base = kRows ? K : 0; base < K; base += kWideThreads) {
       int k = (int)(base + tid);
       int a = 0;
       if (k < K) {
@@ -974,10 +981,11 @@ __global__ void k_auto_tiles(const int *__restrict__ excl_dense, int64_t Q, int6
 // packed minimum holds distances below 2^32 - 1 exactly; where it is at that limit (top1_flag: some
 // pair's distance reached it) the top-1 is the exact (distance, index) minimum over the scene instead.
 // Each such needle takes a pass over its haystack by one block, so the needles are dealt out to all
-// blocks of the grid one by one (kFinalizeBlocks): 300 such needles x 3,000 images of 32 x 32 take
-// 9.1 ms, and 96.7 ms with 256 consecutive needles to a block.
+// blocks of the grid one by one, all eight blocks of an SM at once (kFinalizeBlocks): 300 such needles x
+// 3,000 images of 32 x 32 take 6.7 ms, and 96.7 ms with 256 consecutive needles to a block.
 constexpr int kFinalizeBlocks = 152 * 8;
-__global__ void __launch_bounds__(256) k_finalize(const SearchScene *__restrict__ tab,
+template <bool kRows>
+__global__ void __launch_bounds__(256, 8) k_finalize(const SearchScene *__restrict__ tab,
                                                   const int *__restrict__ qscene, int64_t Qtot,
                                                   int N, const int *__restrict__ rank,
                                                   const int64_t *__restrict__ dtrue,
@@ -1018,7 +1026,7 @@ __global__ void __launch_bounds__(256) k_finalize(const SearchScene *__restrict_
       const int64_t il = ie - sc.qoff;
       long long md = 0x7fffffffffffffffll, mj = -1;
       for (int64_t j = warp; j < sc.H; j += 8) {
-        long long d = warp_crss(sc.needles + il * K, sc.haystack + j * K, N);
+        long long d = warp_crss<kRows>(sc.needles + il * K, sc.haystack + j * K, N);
         if (d < md) {
           md = d;
           mj = j;
@@ -1044,6 +1052,7 @@ __global__ void __launch_bounds__(256) k_finalize(const SearchScene *__restrict_
 }
 
 // Full distance matrix (exact int64), one warp per pair.
+template <bool kRows>
 __global__ void k_distances(const uint16_t *__restrict__ nimg, int64_t Q,
                             const uint16_t *__restrict__ himg, int64_t H, int N,
                             int64_t *__restrict__ out) {
@@ -1053,7 +1062,7 @@ __global__ void k_distances(const uint16_t *__restrict__ nimg, int64_t Q,
   const int64_t K = (int64_t)N * N;
   for (int64_t p = w; p < Q * H; p += nw) {
     const int64_t i = p / H, j = p - i * H;
-    int64_t d = warp_crss(nimg + i * K, himg + j * K, N);
+    int64_t d = warp_crss<kRows>(nimg + i * K, himg + j * K, N);
     if (lane == 0) out[p] = d;
   }
 }
@@ -1096,6 +1105,7 @@ __device__ __forceinline__ bool warp_crss_many(const uint16_t *n, const uint16_t
 // A whole small search of one scene in one launch: block i ranks needle i, one warp per pair, every
 // distance exact in int64 (so no classes, lists or fallbacks).
 constexpr int kSmallWarps = 16;
+template <bool kRows>
 __global__ void __launch_bounds__(kSmallWarps * 32) k_search_small(SearchScene sc, int N,
                                                                    int64_t *__restrict__ distances,
                                                                    int *status) {
@@ -1108,7 +1118,7 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_search_small(SearchScene s
   const int64_t m = sc.match ? sc.match[i] : i;
   const bool valid = m >= 0 && m < sc.H;
   if (warp == 0) {
-    const int64_t d = valid ? warp_crss(needle, sc.haystack + m * K, N) : -1;
+    const int64_t d = valid ? warp_crss<kRows>(needle, sc.haystack + m * K, N) : -1;
     if (lane == 0) {
       dt_s = d;
       if (!valid) set_status(status, RICI_ERR_INDEX_OUT_OF_RANGE);
@@ -1119,7 +1129,6 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_search_small(SearchScene s
   int cnt = 0;
   int64_t bd = INT64_MAX, bj = -1;
   if (valid || distances) {
-    const bool many = rows_of_8(N) && aligned16(needle) && aligned16(sc.haystack);
     for (int64_t j0 = warp; j0 < sc.H; j0 += kMany * kSmallWarps) {
       int64_t d[kMany];
       const uint16_t *h[kMany];
@@ -1128,11 +1137,11 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_search_small(SearchScene s
         const int64_t j = j0 + m * kSmallWarps;
         h[m] = sc.haystack + (j < sc.H ? j : sc.H - 1) * K;
       }
-      if (!many || !warp_crss_many(needle, h, N, d)) {
+      if (!kRows || !warp_crss_many(needle, h, N, d)) {
 #pragma unroll 1
         for (int m = 0; m < kMany; ++m) {
           const int64_t j = j0 + m * kSmallWarps;
-          const int64_t x = warp_crss(needle, sc.haystack + (j < sc.H ? j : sc.H - 1) * K, N);
+          const int64_t x = warp_crss<kRows>(needle, sc.haystack + (j < sc.H ? j : sc.H - 1) * K, N);
 #pragma unroll
           for (int o = 0; o < kMany; ++o)
             if (o == m) d[o] = x;
@@ -1320,8 +1329,15 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   const int N = b.N;
   const int64_t K = (int64_t)N * N;
   if (Q == 0) return cudaSuccess;
+  // rows: images that a warp reads 8 pixels at a time; pairs: and that fill its 256 pixels (8 x 8 ones
+  // leave three lanes of four idle: 1,000 x 20,000 distances 4.38 ms so, 4.06 ms 32 pixels at a time)
+  bool rows = rows_of_8(N);
+  for (int i = 0; i < b.num_scenes; ++i)
+    rows = rows && aligned16(scenes[i].needles) && aligned16(scenes[i].haystack);
+  const bool pairs = rows && K >= 256;
   if (small_search(b)) {
-    k_search_small<<<(unsigned)Q, kSmallWarps * 32, 0, st>>>(scenes[0], N, out_distances, b.status);
+    const auto small_kernel = rows ? k_search_small<true> : k_search_small<false>;
+    small_kernel<<<(unsigned)Q, kSmallWarps * 32, 0, st>>>(scenes[0], N, out_distances, b.status);
     count_launches(1);
     return cudaGetLastError();
   }
@@ -1403,23 +1419,24 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
                                                                         qscene, hscene);
     count_launches(1);
   }
-  k_true_distance<<<blocks_for(Q), 32 * wpb, 0, st>>>(tab, qscene, Q, N, dt, rank, best, nflags,
-                                                       t1flag, b.status);
+  const auto true_kernel = pairs ? k_true_distance<true> : k_true_distance<false>;
+  true_kernel<<<blocks_for(Q), 32 * wpb, 0, st>>>(tab, qscene, Q, N, dt, rank, best, nflags, t1flag,
+                                                  b.status);
   count_launches(1);
   unsigned long long *cnt = reinterpret_cast<unsigned long long *>(b.counters);
   const size_t wide_smem = sizeof(int2) * (size_t)K;
-  if ((e = cudaFuncSetAttribute(k_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const auto wide_kernel = rows_of_8(N) ? k_wide<true> : k_wide<false>;
+  if ((e = cudaFuncSetAttribute(wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)wide_smem)) != cudaSuccess)
     return e;
   // int64 pairs: needles outside the class against everything and the others against the images
   // outside it (mode 0), or every pair (mode 2)
   auto wide = [&](int mode, const int *sub_list = nullptr, const int *sub_count = nullptr,
                   const int *list = nullptr, const int *list_count = nullptr) {
-    k_wide<<<152 * 8, kWideThreads, wide_smem, st>>>(tab, qscene, hscene, Q, b.Hmax, N, mode,
-                                                   nwide, wn_list, counts + 0,
-                                                   list ? list : wh_list,
-                                                   list_count ? list_count : counts + 1, dt, nflags,
-                                                   rank, best, t1flag, cnt, sub_list, sub_count);
+    wide_kernel<<<152 * 8, kWideThreads, wide_smem, st>>>(
+        tab, qscene, hscene, Q, b.Hmax, N, mode, nwide, wn_list, counts + 0, list ? list : wh_list,
+        list_count ? list_count : counts + 1, dt, nflags, rank, best, t1flag, cnt, sub_list,
+        sub_count);
     count_launches(1);
   };
   auto run_dense = [&](const int *nexcl, const int *hexcl, const int *hcount, const int *hmap,
@@ -1528,12 +1545,15 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
     if ((e = cudaMemsetAsync(nwide, 0, sizeof(int) * Q, st)) != cudaSuccess) return e;
     wide(2);
   }
-  k_finalize<<<(unsigned)(Q < kFinalizeBlocks ? Q : kFinalizeBlocks), 256, 0, st>>>(
+  const auto finalize_kernel = pairs ? k_finalize<true> : k_finalize<false>;
+  finalize_kernel<<<(unsigned)(Q < kFinalizeBlocks ? Q : kFinalizeBlocks), 256, 0, st>>>(
       tab, qscene, Q, N, rank, dt, best, nflags, t1flag);
   count_launches(1);
   if (out_distances && b.num_scenes == 1) {
-    k_distances<<<blocks_for(Q * H), 32 * wpb, 0, st>>>(scenes[0].needles, Q, scenes[0].haystack,
-                                                         H, N, out_distances);
+    const auto distances_kernel = pairs ? k_distances<true> : k_distances<false>;
+    distances_kernel<<<blocks_for(Q * H), 32 * wpb, 0, st>>>(scenes[0].needles, Q,
+                                                             scenes[0].haystack, H, N,
+                                                             out_distances);
     count_launches(1);
   }
   return cudaGetLastError();
