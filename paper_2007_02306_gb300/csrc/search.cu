@@ -1180,17 +1180,34 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_search_small(SearchScene s
   }
 }
 
-// Whether a call takes k_search_small: the forms that leave the choice to the library (DEFAULT,
-// AUTO), no work counters, and so little work that launches decide.  A pair costs a warp about
-// 0.45 us and 0.11 us per 256 pixels, one after another, so the haystack is limited (256 images of up
-// to 32 x 32, 64 of 64 x 64, 16 of 128 x 128), and with it the work in all.  162 x 162 images of 32 x
-// 32 with the distance matrix: 114 us in the general sequence of 19 launches, 29 us here.  With one
-// pair at a time per warp and 8 warps it lost past the limits: 64 x 512 images of 32 x 32 80 against 93 us,
-// 512 x 512 190 against 95 us, 16 x 2,048 of 16 x 16 146 against 85 us.
-bool small_search(const SearchBatch &b) {
-  const int64_t K = (int64_t)b.N * b.N < 1024 ? 1024 : (int64_t)b.N * b.N;
-  return (b.mode == RICI_SEARCH_DEFAULT || b.mode == RICI_SEARCH_AUTO) && b.num_scenes == 1 &&
-         !b.counters && b.Htot * K <= (1 << 18) && b.Qtot * b.Htot * K <= (1 << 26);
+// Whether a call takes k_search_small: the forms that leave the choice to the library (DEFAULT, AUTO),
+// no work counters, and so little work that launches decide.  The haystack is limited (256 images of
+// up to 32 x 32, 64 of 64 x 64, 16 of 128 x 128), and with it the work in all: past that the general
+// sequence wins (64 x 512 images of 32 x 32 80 against 93 us, 512 x 512 95 against 190 us).  Within:
+//   8 pixels per lane (rows): on top of what both sides pay, the blocks (one per needle) take about 5 ns
+//     each, and 0.35 ns per 256 pixels of a pair, where a warp takes four pairs at a time, there or not;
+//     the general sequence's further launches take 25 us and 4.5 us per 256 pixels.  162 x 162 images
+//     of 32 x 32 114 us in 19 launches, 23 us here; 4,000 x 4 75 and 54 us, 4,000 x 16 75 and 126 us;
+//     16,000 x 1 of 8 x 8 61 and 109 us; 600 x 16 of 64 x 64 109 and 64 us, 1,000 x 16 108 and 111 us.
+//   1 pixel per lane (other resolutions, unaligned images): `serial` steps one after another in a warp,
+//     0.3 us each, so it wins up to 72 of them (1 x 64 images of 20 x 20 32 and 27 us, 1 x 32 of 33 x 33 50
+//     and 54 us, 64 x 240 52 and 186 us) while the needles' blocks are resident together (300 x 4 of
+//     33 x 33 52 and 47 us, 1,000 x 1 of 24 x 24 35 and 60 us).  Unaligned images that the general
+//     sequence would take on tensor cores up to 256 steps (64 x 64 of 32 x 32 78 and 60 us, 64 x 256
+//     89 and 179 us; 1 x 16 of 64 x 64 156 and 148 us).
+bool small_search(const SearchBatch &b, bool rows) {
+  const int64_t Q = b.Qtot, H = b.Htot, K = (int64_t)b.N * b.N, K1 = K < 1024 ? 1024 : K;
+  if (!((b.mode == RICI_SEARCH_DEFAULT || b.mode == RICI_SEARCH_AUTO) && b.num_scenes == 1 &&
+        !b.counters && H * K1 <= (1 << 18) && Q * H * K1 <= (1 << 26)))
+    return false;
+  if (rows) {
+    const int64_t passes = (K + 255) / 256;
+    const int64_t work = Q * (H < 16 ? H : 16) * ((H + 63) / 64) * passes;
+    return 7 * work + 100 * Q <= 500000 + 90000 * passes;
+  }
+  const int64_t serial = (K + 31) / 32 * (1 + (H + 15) / 16);
+  return rows_of_8(b.N) ? serial <= 256 && Q * (serial + 16) <= (1 << 16)
+                        : serial <= 72 && Q * (serial + 16) <= (1 << 15);
 }
 
 bool dense_supported(int N) { return N == 8 || N == 16 || N == 32 || N == 64 || N == 128; }
@@ -1335,7 +1352,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   for (int i = 0; i < b.num_scenes; ++i)
     rows = rows && aligned16(scenes[i].needles) && aligned16(scenes[i].haystack);
   const bool pairs = rows && K >= 256;
-  if (small_search(b)) {
+  if (small_search(b, rows)) {
     const auto small_kernel = rows ? k_search_small<true> : k_search_small<false>;
     small_kernel<<<(unsigned)Q, kSmallWarps * 32, 0, st>>>(scenes[0], N, out_distances, b.status);
     count_launches(1);
