@@ -449,8 +449,10 @@ __global__ void k_scan_final(const int *__restrict__ in, int64_t n, const int *_
 // scan, sorted records, bounding spheres (the steps of k_tri_bbox .. k_chunk_spheres, with the
 // bins in shared memory).  Nine dependent launches of a few microseconds each cost more than the
 // work of up to kSmallTris triangles: 162 images of a 320-triangle mesh 62 us with them, 37 us
-// with this launch and the generation's (most of it the call's host side).
-constexpr int kSmallTris = 8192;
+// with this launch and the generation's (most of it the call's host side).  One block takes 5 us per
+// 1,000 triangles, so the sides meet between 5,000 (one image 60 us here, 63 us in nine launches) and
+// 6,000 (66 and 63 us; 8,192: 83 and 67 us).
+constexpr int kSmallTris = 5120;
 constexpr int kSmallBins = 4096;  // 8^L bins in use: L <= 4 for up to 2^14 buckets
 __global__ void __launch_bounds__(1024) k_sort_small(GenScene sc, GenScene *__restrict__ tab,
                                                      uint32_t *__restrict__ tb,
