@@ -683,6 +683,7 @@ struct QueryArgs {
   unsigned long long *best;
   int *hwide, *wh_list, *wh_count;
   int *status;
+  int withhold_first_load;  // test hook: block 0 skips the load of its first pixels
 };
 
 __global__ void __launch_bounds__(kQThreads, 1)
@@ -753,12 +754,15 @@ __global__ void __launch_bounds__(kQThreads, 1)
             ok = false;
             break;
           }
+          if (a.withhold_first_load && blockIdx.x == 0 && it == 0) continue;
           mbar_arrive_expect_tx(&px_full[s], kQTile);
           tma_load_2d(s_px + s * kQTile, &map_px, &px_full[s], c * 64, y);
         }
       }
-      for (uint32_t j = 1; j <= (uint32_t)kQRaw && j <= it; ++j)
+      for (uint32_t j = 1; j <= (uint32_t)kQRaw && j <= it; ++j) {
+        if (a.withhold_first_load && blockIdx.x == 0 && it == j) continue;
         mbar_drain(&px_full[(it - j) % kQRaw], ((it - j) / kQRaw) & 1, a.status);
+      }
     }
   } else if (warp == 6 + kQConvWarps) {
     // ---------------- needle operands
@@ -1043,7 +1047,7 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
   k_tc_encode<<<blocks_for(Q), 256, 0, st>>>(tab, qscene, Q, N, 1, opa, nwide, wn_list, counts + 0,
                                              asum, nullptr, skip_tile, nullptr, nullptr, nullptr);
   // few needles of one scene: the haystack's operands are built inside the GEMM kernel
-  const bool query = haystack && !skip_tile && !test_withhold && Q <= kQueryNeedles &&
+  const bool query = haystack && !skip_tile && Q <= kQueryNeedles &&
                      (reinterpret_cast<uintptr_t>(haystack) & 15) == 0;  // (TMA)
   if (query) {
     CUtensorMap mq, mp;
@@ -1065,6 +1069,7 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
     q.wh_list = wh_list;
     q.wh_count = counts + 1;
     q.status = status;
+    q.withhold_first_load = test_withhold;
     const size_t smem_q = 1024 + (kQRaw + 4 * kQOps) * kQTile + 512;
     if ((e = cudaFuncSetAttribute(k_tc_query, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)smem_q)) != cudaSuccess)
