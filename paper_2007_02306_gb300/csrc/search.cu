@@ -808,11 +808,13 @@ __global__ void __launch_bounds__(kSparseWarps * 32, 4) k_sparse(
 //   pass 0: needles = wide needle list, haystack = the needle's whole scene.
 //   pass 1: needles = all needles that are not wide, haystack = wide images of the same scene.
 //   pass 2: needles = all needles, haystack = the whole scene (reference path).
-// mode 0 runs passes 0 and 1 (in one launch), mode 2 pass 2.  kRows: rows_of_8(N).  Eight blocks per SM:
-// with 40 registers and six of them the rest of the grid came as a second wave (1,000 x 2,000 images
-// of 48 x 48 187 -> 158 us, of noise of 32 x 32 18.8 -> 14.6 ms with the exact top-1).
+// mode 0 runs passes 0 and 1 (in one launch), mode 2 pass 2.  kRows: rows_of_8(N), 40 registers and six
+// blocks per SM (at 32 they spill); else eight.  The items' costs differ widely, so the first form's
+// grid is twice what is resident: 1,000 x 2,000 images of noise of 32 x 32 17.9 ms with one and a third
+// times as many blocks, 13.3 ms with just as many, 13.2 ms so; 300 x 3,000 of 64 x 64 39.3, 28.5,
+// 27.5 ms; the images outside int8 of 16,384 x 262,144 sparse ones 122, 120, 111 us.
 template <bool kRows>
-__global__ void __launch_bounds__(kWideThreads, 8) k_wide(
+__global__ void __launch_bounds__(kWideThreads, kRows ? 6 : 8) k_wide(
     const SearchScene *__restrict__ tab, const int *__restrict__ qscene,
     const int *__restrict__ hscene, int64_t Qtot, int64_t Hmax, int N, int mode,
     const int *__restrict__ nwide, const int *__restrict__ wide_n_list,
@@ -981,41 +983,48 @@ __global__ void k_auto_tiles(const int *__restrict__ excl_dense, int64_t Q, int6
 // packed minimum holds distances below 2^32 - 1 exactly; where it is at that limit (top1_flag: some
 // pair's distance reached it) the top-1 is the exact (distance, index) minimum over the scene instead.
 // Each such needle takes a pass over its haystack by one block, so the needles are dealt out to all
-// blocks of the grid one by one, all eight blocks of an SM at once (kFinalizeBlocks): 300 such needles x
-// 3,000 images of 32 x 32 take 6.7 ms, and 96.7 ms with 256 consecutive needles to a block.
-constexpr int kFinalizeBlocks = 152 * 8;
+// blocks of the grid one by one: 300 such needles x 3,000 images of 32 x 32 took 96.7 ms with 256
+// consecutive needles to a block.  Four blocks of 16 warps per SM: 1.29 ms for 1,000 needles x 2,000, 1.71
+// ms for 300 x 3,000 of 64 x 64, 4.6 us where there is no such needle (eight of 8 warps 1.16, 2.58 ms,
+// 4.7 us; two of 32 1.10, 1.66 ms, 5.4 us).
+constexpr int kFinalizeBlocks = 152 * 4, kFinalizeWarps = 16;
 template <bool kRows>
-__global__ void __launch_bounds__(256, 8) k_finalize(const SearchScene *__restrict__ tab,
-                                                  const int *__restrict__ qscene, int64_t Qtot,
-                                                  int N, const int *__restrict__ rank,
-                                                  const int64_t *__restrict__ dtrue,
-                                                  const unsigned long long *__restrict__ best,
-                                                  const int *__restrict__ nflags,
-                                                  const int *__restrict__ top1_flag) {
-  __shared__ int64_t exact_s[256];
+__global__ void __launch_bounds__(kFinalizeWarps * 32, 4)
+    k_finalize(const SearchScene *__restrict__ tab, const int *__restrict__ qscene, int64_t Qtot,
+               int N, const int *__restrict__ rank, const int64_t *__restrict__ dtrue,
+               const unsigned long long *__restrict__ best, const int *__restrict__ nflags,
+               const int *__restrict__ top1_flag) {
+  __shared__ int64_t exact_s[kFinalizeWarps * 32];
   __shared__ int nexact;
-  __shared__ long long bd[8];
-  __shared__ long long bj[8];
+  __shared__ long long bd[kFinalizeWarps];
+  __shared__ long long bj[kFinalizeWarps];
   const int64_t K = (int64_t)N * N;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  auto is_exact = [&](int64_t i) {
-    return top1_flag[i] && !nflags[i] && (best[i] >> 32) == 0xffffffffull && best[i] != kNoBest &&
-           tab[scene_at(qscene, i)].top1;
+  // (loads side by side: a chain of them is this kernel's time)
+  auto is_exact = [&](int64_t i, int flags, unsigned long long bv) -> bool {
+    const int t1 = top1_flag[i];
+    return (t1 != 0) & (flags == 0) & ((bv >> 32) == 0xffffffffull) & (bv != kNoBest);
   };
+  // needles blockIdx.x + k gridDim.x, one per thread at a time (the first look at them before the
+  // outputs below, whose latency covers it)
+  auto mine = [&](int64_t k0) { return blockIdx.x + (k0 + threadIdx.x) * gridDim.x; };
+  bool ex = mine(0) < Qtot && is_exact(mine(0), nflags[mine(0)], best[mine(0)]);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Qtot;
        i += (int64_t)gridDim.x * blockDim.x) {
+    const int flags = nflags[i], r = rank[i];
+    const unsigned long long bv = best[i];
+    const int64_t dt = dtrue[i];
+    const bool e = is_exact(i, flags, bv);
     const SearchScene &sc = tab[scene_at(qscene, i)];
     const int64_t il = i - sc.qoff;
-    sc.rank[il] = rank[i];
-    if (sc.dtrue) sc.dtrue[il] = dtrue[i];
-    if (sc.top1 && !is_exact(i))
-      sc.top1[il] = (nflags[i] != 0 || best[i] == kNoBest)
-                        ? -1 : (int32_t)(uint32_t)(best[i] & 0xffffffffull);
+    sc.rank[il] = r;
+    if (sc.dtrue) sc.dtrue[il] = dt;
+    if (sc.top1 && !e)
+      sc.top1[il] = (flags != 0 || bv == kNoBest) ? -1 : (int32_t)(uint32_t)(bv & 0xffffffffull);
   }
-  // needles blockIdx.x + k gridDim.x, 256 at a time
-  for (int64_t k0 = 0; blockIdx.x + k0 * gridDim.x < Qtot; k0 += 256) {
-    const int64_t i = blockIdx.x + (k0 + threadIdx.x) * gridDim.x;
-    const bool ex = i < Qtot && is_exact(i);
+  for (int64_t k0 = 0; blockIdx.x + k0 * gridDim.x < Qtot; k0 += kFinalizeWarps * 32) {
+    const int64_t i = mine(k0);
+    if (k0) ex = i < Qtot && is_exact(i, nflags[i], best[i]);
     if (threadIdx.x == 0) nexact = 0;
     if (!__syncthreads_or(ex)) continue;  // (uniform over the block)
     if (ex) exact_s[atomicAdd(&nexact, 1)] = i;
@@ -1023,9 +1032,10 @@ __global__ void __launch_bounds__(256, 8) k_finalize(const SearchScene *__restri
     for (int x = 0; x < nexact; ++x) {
       const int64_t ie = exact_s[x];
       const SearchScene &sc = tab[scene_at(qscene, ie)];
+      if (!sc.top1) continue;  // (uniform over the block)
       const int64_t il = ie - sc.qoff;
       long long md = 0x7fffffffffffffffll, mj = -1;
-      for (int64_t j = warp; j < sc.H; j += 8) {
+      for (int64_t j = warp; j < sc.H; j += kFinalizeWarps) {
         long long d = warp_crss<kRows>(sc.needles + il * K, sc.haystack + j * K, N);
         if (d < md) {
           md = d;
@@ -1039,7 +1049,7 @@ __global__ void __launch_bounds__(256, 8) k_finalize(const SearchScene *__restri
       __syncthreads();
       if (threadIdx.x == 0) {
         long long d0 = bd[0], j0 = bj[0];
-        for (int w = 1; w < 8; ++w)
+        for (int w = 1; w < kFinalizeWarps; ++w)
           if (bd[w] < d0 || (bd[w] == d0 && bj[w] < j0)) {
             d0 = bd[w];
             j0 = bj[w];
@@ -1443,6 +1453,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   unsigned long long *cnt = reinterpret_cast<unsigned long long *>(b.counters);
   const size_t wide_smem = sizeof(int2) * (size_t)K;
   const auto wide_kernel = rows_of_8(N) ? k_wide<true> : k_wide<false>;
+  const int wide_blocks = 152 * (rows_of_8(N) ? 12 : 8);
   if ((e = cudaFuncSetAttribute(wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)wide_smem)) != cudaSuccess)
     return e;
@@ -1450,7 +1461,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   // outside it (mode 0), or every pair (mode 2)
   auto wide = [&](int mode, const int *sub_list = nullptr, const int *sub_count = nullptr,
                   const int *list = nullptr, const int *list_count = nullptr) {
-    wide_kernel<<<152 * 8, kWideThreads, wide_smem, st>>>(
+    wide_kernel<<<wide_blocks, kWideThreads, wide_smem, st>>>(
         tab, qscene, hscene, Q, b.Hmax, N, mode, nwide, wn_list, counts + 0, list ? list : wh_list,
         list_count ? list_count : counts + 1, dt, nflags, rank, best, t1flag, cnt, sub_list,
         sub_count);
@@ -1563,8 +1574,8 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
     wide(2);
   }
   const auto finalize_kernel = pairs ? k_finalize<true> : k_finalize<false>;
-  finalize_kernel<<<(unsigned)(Q < kFinalizeBlocks ? Q : kFinalizeBlocks), 256, 0, st>>>(
-      tab, qscene, Q, N, rank, dt, best, nflags, t1flag);
+  finalize_kernel<<<(unsigned)(Q < kFinalizeBlocks ? Q : kFinalizeBlocks), kFinalizeWarps * 32, 0,
+                    st>>>(tab, qscene, Q, N, rank, dt, best, nflags, t1flag);
   count_launches(1);
   if (out_distances && b.num_scenes == 1) {
     const auto distances_kernel = pairs ? k_distances<true> : k_distances<false>;
