@@ -194,12 +194,14 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
 
 // Tensor-core search (tc_search.cu): operand encoding + persistent tcgen05 GEMM with the rank /
 // top-1 epilogue for narrow x narrow pairs of every scene.  Fills nwide/hwide and the wide
-// lists/counts (launch-wide indices).  With haystack (single scene) few needles take a kernel that reads its pixels
-// itself, and with split the haystack images outside
-// the fp16 class that only exceed its limit on one delta are ranked too, by a second GEMM with a
-// split square, and left_list / *left_count (zeroed before) receive the other ones.
+// lists/counts (launch-wide indices).  With haystack (single scene) few needles take a kernel that
+// reads its pixels itself.  With split, haystack images outside the fp16 class whose deltas are all
+// within 127 and whose partial sums stay below 2^24 are ranked too, by a second GEMM with a split
+// square (rows at split_rows, tc_split_bytes of them, free again after the launch), and left_list /
+// *left_count (zeroed before) receive the other ones.
 bool tc_supported(int N);
 int64_t tc_workspace_bytes(int64_t Q, int64_t H, int N, bool single_scene);
+int64_t tc_split_bytes(int64_t H, int N);
 cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, const int *qscene,
                                       const int *hscene, int64_t Qtot, int64_t Htot,
                                       int64_t tiles_total, int N, void *ws, int *nwide, int *hwide,
@@ -210,7 +212,8 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
                                       const int *skip_tile = nullptr,
                                       const int *any_tile = nullptr,
                                       const uint16_t *haystack = nullptr, bool split = false,
-                                      int *left_list = nullptr, int *left_count = nullptr);
+                                      int *left_list = nullptr, int *left_count = nullptr,
+                                      void *split_rows = nullptr);
 
 // Integer tensor-core search (i8_search.cu): int8 operand encoding + mma.sync s8 GEMM with the
 // rank / top-1 epilogue for int8-narrow x int8-narrow pairs of every scene (the tiles of the

@@ -1301,6 +1301,15 @@ void search_tiles(int64_t Q, int64_t H, int32_t *tiles_m, int32_t *tiles_n) {
   *tiles_n = (int32_t)((H + 255) / 256);
 }
 
+// Bytes of the haystack's int8 deltas (groups of 32 images).  In a tensor-core search the rows of its
+// split-square images lie there before: their GEMM is done when the images of neither class are
+// encoded, and from 6,144 images on they take no more room.
+static int64_t haystack_delta_bytes(int64_t H, int N, bool split_rows) {
+  const int64_t deltas = (H + 127) / 128 * 128 * N * N;
+  const int64_t rows = split_rows ? tc_split_bytes(H, N) : 0;
+  return deltas > rows ? deltas : rows;
+}
+
 int64_t search_batch_workspace_bytes(int num_scenes, int64_t Q, int64_t H, int N, int mode) {
   const int64_t K = (int64_t)N * N;
   mode &= 0xff;
@@ -1319,7 +1328,7 @@ int64_t search_batch_workspace_bytes(int num_scenes, int64_t Q, int64_t H, int N
   c.take<int8_t>(packed || mid ? Q * K : 0);  // needle deltas (CUDA-core forms)
   c.take<int8_t>(packed || mid ? Q * K : 0);  // needle masks
   c.take<int>((packed && !sparse) || mid ? Q * N : 0);  // needle row sums of squared deltas
-  c.take<int8_t>(packed || mid ? (H + 127) / 128 * 128 * K : 0);  // haystack deltas (groups of 32)
+  c.take<int8_t>(packed || mid ? haystack_delta_bytes(H, N, mid) : 0);  // haystack deltas
   c.take<int>(Q);                        // needle wide flags
   c.take<int>(H + 4);                    // haystack wide flags (or, sparse form, a bit per image)
   c.take<int>(Q);                        // wide needle list
@@ -1393,7 +1402,7 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
   int8_t *nd = c.take<int8_t>(packed || mid ? Q * K : 0);
   int8_t *nm = c.take<int8_t>(packed || mid ? Q * K : 0);
   int *nrs = c.take<int>(dense || mid ? Q * N : 0);
-  int8_t *hd = c.take<int8_t>(packed || mid ? (H + 127) / 128 * 128 * K : 0);
+  int8_t *hd = c.take<int8_t>(packed || mid ? haystack_delta_bytes(H, N, mid) : 0);
   int *nwide = c.take<int>(Q);
   int *hwide = c.take<int>(H + 4);
   int *wn_list = c.take<int>(Q);
@@ -1517,8 +1526,8 @@ cudaError_t launch_search_batch(const SearchScene *scenes, const SearchBatch &b,
                                        tc_ws, nwide, hwide, wn_list, wh_list, counts, nflags, dt,
                                        rank, best, b.status, withhold, st, sparse_of,
                                        autom ? skip_tile : nullptr, counts + 5,
-                                       mid ? s0.haystack : nullptr, split, left_list, left_count)) !=
-        cudaSuccess)
+                                       mid ? s0.haystack : nullptr, split, left_list, left_count,
+                                       hd)) != cudaSuccess)
       return e;
     if (mid) {
       // the haystack images of neither tensor-core class, compacted in list order (list and

@@ -428,13 +428,6 @@ __global__ void k_tc_encode_split(const uint16_t *__restrict__ imgs, int N,
   }
 }
 
-// Rows kept for split-square images: an eighth of the haystack, in whole tiles (3 KB of workspace per
-// image at N = 64; images beyond that go to the CUDA cores).
-int split_capacity(int64_t H) {
-  const int64_t want = (H / 8 + kBN) / kBN * kBN;
-  return (int)(want < H ? want : H);
-}
-
 // ---------------------------------------------------------------- GEMM + rank epilogue (S3, S5)
 
 struct TcArgs {
@@ -994,6 +987,17 @@ cudaError_t encode_map(CUtensorMap *map, const void *base, int64_t rows, int KT,
 
 }  // namespace
 
+// Rows kept for split-square images: an eighth of the haystack, in whole tiles (images beyond that go to
+// the CUDA cores).
+static int split_capacity(int64_t H) {
+  const int64_t want = (H / 8 + kBN) / kBN * kBN;
+  return (int)(want < H ? want : H);
+}
+
+int64_t tc_split_bytes(int64_t H, int N) {
+  return split_capacity(H) * (3ll * N * N) * (int64_t)sizeof(__half);
+}
+
 // Most needles of a call that k_tc_query takes (measured above).
 constexpr int64_t kQueryNeedles = 512;
 
@@ -1007,8 +1011,7 @@ int64_t tc_workspace_bytes(int64_t Q, int64_t H, int N, bool single_scene) {
   c.take<__half>(H * KT);
   c.take<int>(Q);                 // A_i
   c.take<uint32_t>(single_scene ? H : (H + 31) / 32 + 2);  // image of each row, or class bits
-  c.take<__half>(cap * (KT / 2 * 3));  // split-square rows
-  c.take<int>(cap);                    // their images
+  c.take<int>(cap);               // images of the split-square rows
   return c.off + 256;
 }
 
@@ -1021,7 +1024,7 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
                                       cudaStream_t st, const int *skip_needle,
                                       const int *skip_tile, const int *any_tile,
                                       const uint16_t *haystack, bool split, int *left_list,
-                                      int *left_count) {
+                                      int *left_count, void *split_rows) {
   const int64_t KT = 2ll * N * N;
   const int cap = num_scenes == 1 ? split_capacity(H) : 0;
   Carver c(ws);
@@ -1031,7 +1034,7 @@ cudaError_t launch_tc_encode_and_rank(const SearchScene *tab, int num_scenes, co
   const bool single = num_scenes == 1;
   uint32_t *hvalid = c.take<uint32_t>(single ? H : (H + 31) / 32 + 2);
   int *const row_map = single ? reinterpret_cast<int *>(hvalid) : nullptr;
-  __half *ops = c.take<__half>(cap * (KT / 2 * 3));
+  __half *const ops = static_cast<__half *>(split_rows);
   int *smap = c.take<int>(cap);
   int *const scount = counts + 7;  // their number (zeroed by the caller with the other counts)
   int *const rcount = counts + 8;  // rows of the fp16 class (zeroed likewise)
