@@ -593,27 +593,29 @@ static double sector_piece_area(double ax, double ay, double bx, double by, doub
     const double A = dx * dx + dy * dy;
     double ts[4];
     int nt = 0;
+    double in0 = 0.0, in1 = 0.0; /* the line is inside the circle for in0 < t < in1 */
+    if (!(A > 0.0)) return 0.0;
     ts[nt++] = 0.0;
-    if (A > 0.0) {
-        const double B = ax * dx + ay * dy;
-        const double C = ax * ax + ay * ay - R * R;
-        const double disc = B * B - A * C;
-        if (disc > 0.0) {
-            const double s = sqrt(disc);
-            const double t1 = (-B - s) / A, t2 = (-B + s) / A;
-            if (t1 > 0.0 && t1 < 1.0) ts[nt++] = t1;
-            if (t2 > 0.0 && t2 < 1.0) ts[nt++] = t2;
-        }
+    const double B = ax * dx + ay * dy;
+    const double C = ax * ax + ay * ay - R * R;
+    const double disc = B * B - A * C;
+    if (disc > 0.0) {
+        const double s = sqrt(disc);
+        in0 = (-B - s) / A;
+        in1 = (-B + s) / A;
+        if (in0 > 0.0 && in0 < 1.0) ts[nt++] = in0;
+        if (in1 > 0.0 && in1 < 1.0) ts[nt++] = in1;
     }
     ts[nt++] = 1.0;
     double sum = 0.0;
     for (int i = 0; i + 1 < nt; i++) {
         const double px = ax + ts[i] * dx, py = ay + ts[i] * dy;
         const double qx = ax + ts[i + 1] * dx, qy = ay + ts[i + 1] * dy;
+        /* by the roots, not by the middle's distance: a line that only touches the circle is outside
+         * also where it touches at the middle of the piece */
         const double tm = 0.5 * (ts[i] + ts[i + 1]);
-        const double mx = ax + tm * dx, my = ay + tm * dy;
         const double cross = px * qy - py * qx;
-        if (mx * mx + my * my <= R * R)
+        if (in0 < tm && tm < in1)
             sum += 0.5 * cross;
         else
             sum += 0.5 * R * R * atan2(cross, px * qx + py * qy);
