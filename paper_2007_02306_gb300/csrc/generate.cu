@@ -1624,12 +1624,17 @@ __device__ double disk_wedge(double px, double py, double qx, double qy, double 
   }
   const double ax = px + ta * dx, ay = py + ta * dy, bx = px + tb * dx, by = py + tb * dy;
   // an outer piece never spans opposite directions (the segment between them would cross the
-  // disk), so a zero cross product means an empty sector; this also keeps a zero-length piece
-  // at the origin, whose dot product may be -0, from reading as an angle of pi
+  // disk), so a zero cross product means an empty sector; a piece that the clipping leaves empty has
+  // none either: its ends differ by rounding alone, which near the axis is any angle
   const double c0 = px * ay - py * ax, c1 = bx * qy - by * qx;
-  const double s0 = c0 == 0.0 ? 0.0 : atan2(c0, px * ax + py * ay);  // sector p .. P(ta)
-  const double s1 = c1 == 0.0 ? 0.0 : atan2(c1, bx * qx + by * qy);  // sector P(tb) .. q
-  return 0.5 * R2 * (s0 + s1) + 0.5 * (ax * by - ay * bx);
+  double sectors = 0.0;
+#pragma unroll 1  // (one atan2 in the code: k_clutter does not spill then)
+  for (int k = 0; k < 2; ++k) {  // p .. P(ta), P(tb) .. q
+    const double c = k ? c1 : c0;
+    if (c != 0.0 && (k ? tb < 1.0 : ta > 0.0))
+      sectors += atan2(c, k ? bx * qx + by * qy : px * ax + py * ay);
+  }
+  return 0.5 * R2 * sectors + 0.5 * (ax * by - ay * bx);
 }
 
 // Area of the part of one projected triangle inside the support volume: clip it to the slab
