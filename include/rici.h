@@ -88,9 +88,9 @@ extern "C" {
                                    sparse form when at most a quarter of its 32-bit delta words
                                    hold a non-zero delta (N in 8..128, powers of two, single-scene
                                    calls; multi-scene calls take RICI_SEARCH_TENSOR) */
-/* Test hook, OR-ed into RICI_SEARCH_TENSOR: one CTA of the tensor-core kernel withholds its
- * first tile load, so its bounded waits run out (about 2 s), RICI_ERR_TIMEOUT is raised in the
- * status word and the kernel returns; outputs of that call are unspecified. */
+/* Test hook, OR-ed into RICI_SEARCH_TENSOR: one CTA of the tensor-core kernel that the call takes
+ * withholds its first tile load, so its bounded waits run out (about 2 s), RICI_ERR_TIMEOUT is raised
+ * in the status word and the kernel returns; outputs of that call are unspecified. */
 #define RICI_SEARCH_TEST_WITHHOLD_LOAD 0x100
 
 /*

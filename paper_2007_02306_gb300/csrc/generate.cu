@@ -44,8 +44,7 @@ constexpr float kCellClamp = 1048576.0f;  // |cell coordinate| limit (2^20)
 constexpr int kSlot = 20;  // words per staged triangle (a multiple of 4 whose first 8 multiples
                            // lie in 8 different groups of 4 banks: conflict-free 16-byte loads)
 constexpr int kScanItems = kGenScanItems;
-constexpr int kGenMaxCellsPerReach = 4;      // generation: up to (2 x 4 + 1)^3 cells per point
-constexpr int kSpinMaxCellsPerReach = 3;     // spin images: up to 7^3
+constexpr int kSpinMaxCellsPerReach = 3;  // spin images: up to (2 x 3 + 1)^3 cells per point
 constexpr int kBandQ = 128;  // band queue of a warp: 31 left over + 3 layers of each of 32 triangles
 // shared words per warp: candidate queue, band queue (triangle records, then their layers as
 // bytes), place in the walk over groups, staged triangles; a multiple of 4
@@ -1091,13 +1090,14 @@ __device__ __forceinline__ void neighbour_ranges(const KArgs &a, int64_t bucket_
 //    item is one base vertex, two slopes and one margin (three 16-byte loads, 4 fused
 //    multiply-adds), a column count is one rounding, and its margin test one comparison;
 //  - what is read once per batch or chunk (frame, spin vertex, walk over the groups) stays in shared
-//    memory: 72 registers, 7 blocks of 4 warps per SM at N = 64 (5 blocks 306 ms, 6 281 ms, 7 265 ms
-//    for 32,768 points at R = 0.6; 64 registers for 8 blocks spill: 284 ms);
+//    memory: 72 registers, 7 blocks of 4 warps per SM at N = 64 (5, 6, 7 blocks 306, 281, 265 ms for
+//    one set of 32,768 points at R = 0.6; 64 registers for 8 blocks spill: 284 ms);
 //  - undecided items go to pairs of floats, not to FP64: 0.6 % of the items, at FP64's 1/64 rate
 //    1/6 of the time before.
-// 32,768 points of the 5M-triangle scene at R = 0.6: 457 -> 222 ms; 131,072 at R = 0.15: 167 ->
-// 77 ms; every point of a 189k-triangle scene at R = 0.3: 33.3 -> 15.9 ms (edge selection, table
-// lookups and a dozen margin tests per item before, band items in FP64).
+// One set of inputs (another differs by a quarter), against edge selection, table lookups and a dozen
+// margin tests per item and band items in FP64: 32,768 points of a 5M-triangle scene at R = 0.6 553 ->
+// 256 ms; 131,072 at R = 0.15 170 -> 73.8 ms; every point of a 189k-triangle scene at R = 0.3 33.5 ->
+// 15.0 ms.
 template <int NW, bool kCount>
 __global__ void __launch_bounds__(NW * 32, NW == 4 ? 7 : 3) k_generate(KArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1902,9 +1902,9 @@ constexpr int kSpinMaxCells = 7 * 7 * 7 + 1;  // spin images: neighbourhoods of 
 // The last three queue apart, so that a warp's lanes run one of the FP64 paths together; what is
 // left at the end is shared out over the block's warps.  A triangle belongs to the object when
 // its first vertex index is below object_vertices.
-// FP64 (1/64 of the FP32 rate) bounds it: before, every candidate was projected in FP64 and every
-// triangle not wholly inside was clipped with up to six atan2.
-// 10,242 points, 189k triangles, R = 0.3: 18.3 -> 5.9 ms.
+// FP64 (1/64 of the FP32 rate) bounds it, 64 % of the pipe's cycles, behind it the block's last barrier
+// and instruction fetches: before, every candidate was projected in FP64 and every triangle not wholly
+// inside was clipped with up to six atan2.  10,242 points, 189k triangles, R = 0.3: 18.3 -> 5.8 ms.
 __global__ void __launch_bounds__(kClutterWarps * 32, 5)
     k_clutter(KArgs a, const uint32_t *__restrict__ area_hi, const int *__restrict__ area_lo,
               int64_t object_vertices, double *__restrict__ out_all, double *__restrict__ out_obj,
@@ -2297,13 +2297,14 @@ cudaError_t launch_project_fp32(const float *pts, int64_t n, const float *sv, co
   return cudaGetLastError();
 }
 
-// Bins every triangle of the scenes into the hashed grid for support volumes of radius amax and
-// half-height bmax around each oriented point, and fills the grid fields of k (table, records,
-// bucket starts, cell size, reach, pretest limits, neighbourhood width).
+// Sorts the triangles of the scenes into records: along a Morton curve with the bounding spheres of
+// chunks and groups (morton: generation, clutter measure), or by the cells of a hashed grid (spin
+// images), whose cells suit support volumes of radius amax and half-height bmax around each
+// oriented point.  Fills the fields of k that the kernels read (table, records, starts, spheres, pretest
+// limits, grid).
 static cudaError_t bin_triangles(const GenScene *scenes, int num_scenes, int64_t nt, int64_t TB,
                                  double R, double amax, double bmax, void *ws, int *status,
-                                 cudaStream_t st, KArgs &k, int max_cells_per_reach,
-                                 bool morton) {
+                                 cudaStream_t st, KArgs &k, bool morton) {
   Carver c(ws);
   GenScene *tab = c.take<GenScene>(num_scenes);
   int *counts = c.take<int>(TB);
@@ -2334,8 +2335,8 @@ static cudaError_t bin_triangles(const GenScene *scenes, int num_scenes, int64_t
   // a triangle (centre c, radius <= r_big) reaching the support volume has |c - S| <= reach;
   // with cell > reach / nhalf its cell lies within +-nhalf cells of the spin vertex's cell
   const double reach = (rho + gp.r_big) * 1.001;
-  const int cpr = tu.gen_cells_per_reach < max_cells_per_reach ? tu.gen_cells_per_reach
-                                                               : max_cells_per_reach;
+  const int cpr = tu.gen_cells_per_reach < kSpinMaxCellsPerReach ? tu.gen_cells_per_reach
+                                                                 : kSpinMaxCellsPerReach;
   const double cell = reach / cpr * 1.01;
   gp.inv_cell = (float)(1.0 / cell);
   gp.mask = 0;
@@ -2405,7 +2406,7 @@ cudaError_t launch_generate_batch(const GenScene *scenes, const GenerateBatch &g
   const double bmax = R * (N - 1.0) / (2.0 * N);
   KArgs k;
   cudaError_t e = bin_triangles(scenes, g.num_scenes, g.total_tris, g.total_buckets, R, amax,
-                                bmax, ws, g.status, st, k, kGenMaxCellsPerReach, true);
+                                bmax, ws, g.status, st, k, true);
   if (e != cudaSuccess) return e;
   k.nhalf = 0;  // no neighbour-cell list: candidates come from the sphere hierarchy
   k.R = g.R;
@@ -2433,7 +2434,7 @@ cudaError_t launch_clutter(const ClutterArgs &a, void *ws, cudaStream_t st) {
   const double R = a.support_radius;
   KArgs k;
   cudaError_t e = bin_triangles(&sc, 1, a.num_triangles, (int64_t)sc.nbuckets + 1, R, R, 0.5 * R,
-                                ws, a.status, st, k, kSpinMaxCellsPerReach, true);
+                                ws, a.status, st, k, true);
   if (e != cudaSuccess) return e;
   k.N = 0;
   k.mode = 0;
@@ -2480,7 +2481,7 @@ cudaError_t launch_spin(const SpinArgs &a, void *ws, cudaStream_t st) {
   const double R = a.support_radius;
   KArgs k;
   cudaError_t e = bin_triangles(&sc, 1, a.num_triangles, (int64_t)sc.nbuckets + 1, R, R, 0.5 * R,
-                                ws, a.status, st, k, kSpinMaxCellsPerReach, false);
+                                ws, a.status, st, k, false);
   if (e != cudaSuccess) return e;
   k.N = a.resolution;
   k.mode = 0;

@@ -342,7 +342,8 @@ __global__ void __launch_bounds__(kDenseThreads, (N * kImg <= 64 ? 4 : 2) * 256 
     const int *__restrict__ hmap, const int *__restrict__ gate) {
   // kCounted: the haystack holds *hcount images (H is an upper bound), usually far fewer, so the grid
   // is bounded and its blocks step through the `blocks` work items (a grid for H took 0.1-0.2 ms to
-  // find nothing to do in 131,072 blocks); otherwise one block per item.  hmap (optional): haystack image j is image hmap[j] of the caller's haystack (a compacted subset);
+  // find nothing to do in 131,072 blocks); otherwise one block per item.
+  // hmap (optional): haystack image j is image hmap[j] of the caller's haystack (a compacted subset)
   // gate (optional): *gate == 0 means no needle is ranked here, and every block returns at once
   constexpr int WPR = N / 4;  // 32-bit words per row
   constexpr int K = N * N;
@@ -363,203 +364,203 @@ __global__ void __launch_bounds__(kDenseThreads, (N * kImg <= 64 ? 4 : 2) * 256 
   if (kCounted) H = *hcount < H ? *hcount : H;
   int64_t L = tile0 + blockIdx.x;
   do {
-  const int64_t band = L / tiles_q, qt = L - band * tiles_q;
-  const int64_t h0 = band * band_h;
-  const int64_t h1 = tiles_h - h0 < band_h ? tiles_h : h0 + band_h;
-  const int64_t q0 = qt * kTQ;
-  if (kCounted) {
-    // bands ascend: nothing is left for this block (uniform over the block)
-    if (h0 * (int64_t)(kDenseThreads * kImg) >= H) return;
-    __syncthreads();  // the item before is done with the shared arrays
-  }
+    const int64_t band = L / tiles_q, qt = L - band * tiles_q;
+    const int64_t h0 = band * band_h;
+    const int64_t h1 = tiles_h - h0 < band_h ? tiles_h : h0 + band_h;
+    const int64_t q0 = qt * kTQ;
+    if (kCounted) {
+      // bands ascend: nothing is left for this block (uniform over the block)
+      if (h0 * (int64_t)(kDenseThreads * kImg) >= H) return;
+      __syncthreads();  // the item before is done with the shared arrays
+    }
 
-  bool act = false;
-  if (tid < kTQ) {
-    const int64_t q = q0 + tid;
-    act = q < Q && nflags[q] == 0 && !nwide[q];
-    int64_t t = act ? dtrue[q] : -1;
-    thr_s[tid] = t > 0x7fffffffll ? 0x7fffffff : (int)t;
-    act_s[tid] = act;
-  }
-  if (!__syncthreads_or(act)) continue;  // no needle of this tile is ranked here
-  for (int x = tid; x < kTQ * (K / 4); x += kDenseThreads) {
-    int q = x / (K / 4), wd = x - q * (K / 4);
-    int a = 0, m = 0;
-    if (q0 + q < Q) {
-      a = reinterpret_cast<const int *>(ndelta + (q0 + q) * K)[wd];
-      m = reinterpret_cast<const int *>(nmask + (q0 + q) * K)[wd];
+    bool act = false;
+    if (tid < kTQ) {
+      const int64_t q = q0 + tid;
+      act = q < Q && nflags[q] == 0 && !nwide[q];
+      int64_t t = act ? dtrue[q] : -1;
+      thr_s[tid] = t > 0x7fffffffll ? 0x7fffffff : (int)t;
+      act_s[tid] = act;
     }
-    am[q][wd] = make_int2(a, m);
-  }
-  __syncthreads();
-  // Rows are visited heaviest first so that distances pass the early-exit threshold sooner;
-  // the sum is order independent, so the result is unchanged.  Rows where no needle of the
-  // tile has a non-zero delta contribute nothing and are skipped.
-  for (int x = tid; x < kTQ * N; x += kDenseThreads) {
-    int q = x / N, r = x - q * N;
-    wrow[q][r] = act_s[q] ? nrowsq[(q0 + q) * N + r] : 0;
-  }
-  __syncthreads();
-  __shared__ int tile_w[N];
-  if (tid < N) {
-    int W = 0;
-    unsigned msk = 0;
-#pragma unroll
-    for (int q = 0; q < kTQ; ++q) {
-      W += wrow[q][tid];
-      if (wrow[q][tid] > 0) msk |= 1u << q;
+    if (!__syncthreads_or(act)) continue;  // no needle of this tile is ranked here
+    for (int x = tid; x < kTQ * (K / 4); x += kDenseThreads) {
+      int q = x / (K / 4), wd = x - q * (K / 4);
+      int a = 0, m = 0;
+      if (q0 + q < Q) {
+        a = reinterpret_cast<const int *>(ndelta + (q0 + q) * K)[wd];
+        m = reinterpret_cast<const int *>(nmask + (q0 + q) * K)[wd];
+      }
+      am[q][wd] = make_int2(a, m);
     }
-    rmask[tid] = msk;
-    tile_w[tid] = W;
-  }
-  __syncthreads();
-  if (tid < N) {
-    const int W = tile_w[tid];
-    int rk = 0, nz = 0;
-    for (int r2 = 0; r2 < N; ++r2) {
-      const int W2 = tile_w[r2];
-      rk += (W2 > W) || (W2 == W && r2 < tid);
-      nz += W2 > 0;
+    __syncthreads();
+    // Rows are visited heaviest first so that distances pass the early-exit threshold sooner;
+    // the sum is order independent, so the result is unchanged.  Rows where no needle of the
+    // tile has a non-zero delta contribute nothing and are skipped.
+    for (int x = tid; x < kTQ * N; x += kDenseThreads) {
+      int q = x / N, r = x - q * N;
+      wrow[q][r] = act_s[q] ? nrowsq[(q0 + q) * N + r] : 0;
     }
-    ord[rk] = tid;
-    if (tid == 0) nrows_s = nz;
-  }
-  __syncthreads();
-  const int nrows = nrows_s;
-
-  constexpr int kTile = kDenseThreads * kImg;  // haystack images per tile
-  constexpr int CW = WPR < 4 ? WPR : 4;
-  constexpr int64_t kGroupWords = (int64_t)N * WPR * 32;  // one group of 32 interleaved images
-  const int warp = tid >> 5;
-  for (int64_t ht = h0; ht < h1; ++ht) {
-    // this thread's images: j0 + 32 k, k < kImg (a warp owns kImg consecutive groups of 32)
-    const int64_t j0 = ht * kTile + (int64_t)warp * (32 * kImg) + lane;
-    int acc[kImg][kTQ];  // partial distance minus the needle's true distance (exit once > 0)
-    unsigned alive[kImg];
-    unsigned inrange = 0;  // images of this thread inside the haystack (their rows are loaded)
-#pragma unroll
-    for (int k = 0; k < kImg; ++k) {
-      const int64_t j = j0 + 32 * k;
-      const bool valid = j < H && !hwide[j];
-      if (j < H) inrange |= 1u << k;
-      alive[k] = 0;
+    __syncthreads();
+    __shared__ int tile_w[N];
+    if (tid < N) {
+      int W = 0;
+      unsigned msk = 0;
 #pragma unroll
       for (int q = 0; q < kTQ; ++q) {
-        acc[k][q] = -thr_s[q];
-        if (valid && act_s[q]) alive[k] |= 1u << q;
+        W += wrow[q][tid];
+        if (wrow[q][tid] > 0) msk |= 1u << q;
       }
+      rmask[tid] = msk;
+      tile_w[tid] = W;
     }
-    const int *hgrp = reinterpret_cast<const int *>(hdelta) + (j0 >> 5) * kGroupWords + lane * CW;
-    unsigned long long pair_rows = 0, lane_slots = 0;
-    int hw[kImg][WPR];
-#pragma unroll
-    for (int k = 0; k < kImg; ++k)
-#pragma unroll
-      for (int v = 0; v < WPR; ++v) hw[k][v] = 0;
-    for (int i = 0; i < nrows; ++i) {
-      unsigned any = 0;
-#pragma unroll
-      for (int k = 0; k < kImg; ++k) any |= alive[k];
-      if (__ballot_sync(0xffffffffu, any != 0) == 0) break;
-      const int r = ord[i];
-      const unsigned rm = rmask[r];
-      unsigned use[kImg], uor = 0;
-#pragma unroll
-      for (int k = 0; k < kImg; ++k) {
-        use[k] = alive[k] & rm;
-        uor |= use[k];
-        if (kCount) pair_rows += __popc(use[k]);
+    __syncthreads();
+    if (tid < N) {
+      const int W = tile_w[tid];
+      int rk = 0, nz = 0;
+      for (int r2 = 0; r2 < N; ++r2) {
+        const int W2 = tile_w[r2];
+        rk += (W2 > W) || (W2 == W && r2 < tid);
+        nz += W2 > 0;
       }
-      const unsigned wuse = __reduce_or_sync(0xffffffffu, uor);  // needles any lane still needs
+      ord[rk] = tid;
+      if (tid == 0) nrows_s = nz;
+    }
+    __syncthreads();
+    const int nrows = nrows_s;
+
+    constexpr int kTile = kDenseThreads * kImg;  // haystack images per tile
+    constexpr int CW = WPR < 4 ? WPR : 4;
+    constexpr int64_t kGroupWords = (int64_t)N * WPR * 32;  // one group of 32 interleaved images
+    const int warp = tid >> 5;
+    for (int64_t ht = h0; ht < h1; ++ht) {
+      // this thread's images: j0 + 32 k, k < kImg (a warp owns kImg consecutive groups of 32)
+      const int64_t j0 = ht * kTile + (int64_t)warp * (32 * kImg) + lane;
+      int acc[kImg][kTQ];  // partial distance minus the needle's true distance (exit once > 0)
+      unsigned alive[kImg];
+      unsigned inrange = 0;  // images of this thread inside the haystack (their rows are loaded)
 #pragma unroll
       for (int k = 0; k < kImg; ++k) {
-        // every row of an image inside the haystack is loaded, even once its pairs have all
-        // exited: a uniform load is cheaper than the divergent branch that would skip it
-        if ((inrange >> k) & 1u) {
-          const int *src = hgrp + k * kGroupWords + r * (WPR * 32);
+        const int64_t j = j0 + 32 * k;
+        const bool valid = j < H && !hwide[j];
+        if (j < H) inrange |= 1u << k;
+        alive[k] = 0;
 #pragma unroll
-          for (int v = 0; v < WPR / CW; ++v) {
-            if constexpr (CW == 4) {
-              const int4 x = *reinterpret_cast<const int4 *>(src + v * 32 * CW);
-              hw[k][4 * v] = x.x;
-              hw[k][4 * v + 1] = x.y;
-              hw[k][4 * v + 2] = x.z;
-              hw[k][4 * v + 3] = x.w;
-            } else {
-              const int2 x = *reinterpret_cast<const int2 *>(src + v * 32 * CW);
-              hw[k][2 * v] = x.x;
-              hw[k][2 * v + 1] = x.y;
+        for (int q = 0; q < kTQ; ++q) {
+          acc[k][q] = -thr_s[q];
+          if (valid && act_s[q]) alive[k] |= 1u << q;
+        }
+      }
+      const int *hgrp = reinterpret_cast<const int *>(hdelta) + (j0 >> 5) * kGroupWords + lane * CW;
+      unsigned long long pair_rows = 0, lane_slots = 0;
+      int hw[kImg][WPR];
+#pragma unroll
+      for (int k = 0; k < kImg; ++k)
+#pragma unroll
+        for (int v = 0; v < WPR; ++v) hw[k][v] = 0;
+      for (int i = 0; i < nrows; ++i) {
+        unsigned any = 0;
+#pragma unroll
+        for (int k = 0; k < kImg; ++k) any |= alive[k];
+        if (__ballot_sync(0xffffffffu, any != 0) == 0) break;
+        const int r = ord[i];
+        const unsigned rm = rmask[r];
+        unsigned use[kImg], uor = 0;
+#pragma unroll
+        for (int k = 0; k < kImg; ++k) {
+          use[k] = alive[k] & rm;
+          uor |= use[k];
+          if (kCount) pair_rows += __popc(use[k]);
+        }
+        const unsigned wuse = __reduce_or_sync(0xffffffffu, uor);  // needles any lane still needs
+#pragma unroll
+        for (int k = 0; k < kImg; ++k) {
+          // every row of an image inside the haystack is loaded, even once its pairs have all
+          // exited: a uniform load is cheaper than the divergent branch that would skip it
+          if ((inrange >> k) & 1u) {
+            const int *src = hgrp + k * kGroupWords + r * (WPR * 32);
+#pragma unroll
+            for (int v = 0; v < WPR / CW; ++v) {
+              if constexpr (CW == 4) {
+                const int4 x = *reinterpret_cast<const int4 *>(src + v * 32 * CW);
+                hw[k][4 * v] = x.x;
+                hw[k][4 * v + 1] = x.y;
+                hw[k][4 * v + 2] = x.z;
+                hw[k][4 * v + 3] = x.w;
+              } else {
+                const int2 x = *reinterpret_cast<const int2 *>(src + v * 32 * CW);
+                hw[k][2 * v] = x.x;
+                hw[k][2 * v + 1] = x.y;
+              }
             }
           }
         }
-      }
 #pragma unroll
-      for (int q = 0; q < kTQ; ++q) {
-        if (((wuse >> q) & 1u) == 0) continue;
-        if (kCount) lane_slots += kImg;  // kImg warp-wide needle-row iterations (32 lane slots each)
-        // row sum of m (a - b)^2 = sum a^2 + sum (m b)^2 - 2 sum a b, with sum a^2 precomputed;
-        // the (m b)^2 chain starts from the running value, and one chain per term and image
-        // suffices because the warps of the block hide the dp4a latency
-        const int w = wrow[q][r];
-        int sb[kImg], sa[kImg];
-#pragma unroll
-        for (int k = 0; k < kImg; ++k) {
-          sb[k] = acc[k][q] + w;
-          sa[k] = 0;
-        }
-        const int4 *amq = reinterpret_cast<const int4 *>(&am[q][r * WPR]);
-#pragma unroll
-        for (int v = 0; v < WPR; v += 2) {
-          const int4 x = amq[v >> 1];  // (a_v, m_v, a_v+1, m_v+1)
+        for (int q = 0; q < kTQ; ++q) {
+          if (((wuse >> q) & 1u) == 0) continue;
+          if (kCount) lane_slots += kImg;  // kImg warp-wide needle-row iterations (32 lane slots each)
+          // row sum of m (a - b)^2 = sum a^2 + sum (m b)^2 - 2 sum a b, with sum a^2 precomputed;
+          // the (m b)^2 chain starts from the running value, and one chain per term and image
+          // suffices because the warps of the block hide the dp4a latency
+          const int w = wrow[q][r];
+          int sb[kImg], sa[kImg];
 #pragma unroll
           for (int k = 0; k < kImg; ++k) {
-            const int b0 = hw[k][v], b1 = hw[k][v + 1];
-            const int bm0 = b0 & x.y, bm1 = b1 & x.w;
-            sb[k] = __dp4a(bm0, bm0, sb[k]);
-            sa[k] = __dp4a(x.x, b0, sa[k]);
-            sb[k] = __dp4a(bm1, bm1, sb[k]);
-            sa[k] = __dp4a(x.z, b1, sa[k]);
+            sb[k] = acc[k][q] + w;
+            sa[k] = 0;
+          }
+          const int4 *amq = reinterpret_cast<const int4 *>(&am[q][r * WPR]);
+#pragma unroll
+          for (int v = 0; v < WPR; v += 2) {
+            const int4 x = amq[v >> 1];  // (a_v, m_v, a_v+1, m_v+1)
+#pragma unroll
+            for (int k = 0; k < kImg; ++k) {
+              const int b0 = hw[k][v], b1 = hw[k][v + 1];
+              const int bm0 = b0 & x.y, bm1 = b1 & x.w;
+              sb[k] = __dp4a(bm0, bm0, sb[k]);
+              sa[k] = __dp4a(x.x, b0, sa[k]);
+              sb[k] = __dp4a(bm1, bm1, sb[k]);
+              sa[k] = __dp4a(x.z, b1, sa[k]);
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < kImg; ++k) {
+            // an image whose pair has exited keeps computing with stale deltas; its value is
+            // never read again, since only pairs still alive are counted
+            acc[k][q] = sb[k] - 2 * sa[k];
+            if (acc[k][q] > 0) alive[k] &= ~(1u << q);
           }
         }
+      }
+      // count and top-1 candidates (pairs that never exceeded the threshold hold exact values)
+#pragma unroll
+      for (int q = 0; q < kTQ; ++q) {
+        if (!act_s[q]) continue;
+        int c = 0;
+        unsigned long long b = kNoBest;
 #pragma unroll
         for (int k = 0; k < kImg; ++k) {
-          // an image whose pair has exited keeps computing with stale deltas; its value is
-          // never read again, since only pairs still alive are counted
-          acc[k][q] = sb[k] - 2 * sa[k];
-          if (acc[k][q] > 0) alive[k] &= ~(1u << q);
+          const bool fin = (alive[k] >> q) & 1u;
+          c += fin && acc[k][q] < 0;
+          const int64_t jj = j0 + 32 * k;
+          const unsigned long long bk =
+              fin ? pack_best(acc[k][q] + thr_s[q], hmap ? (int64_t)hmap[jj] : jj) : kNoBest;
+          b = bk < b ? bk : b;
+        }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) c += __shfl_down_sync(0xffffffffu, c, d);
+        b = warp_min_u64(b);
+        if (lane == 0) {
+          if (c) atomicAdd(&rank[q0 + q], c);
+          if (b != kNoBest) atomicMin(&best[q0 + q], b);
         }
       }
-    }
-    // count and top-1 candidates (pairs that never exceeded the threshold hold exact values)
+      if (kCount) {
 #pragma unroll
-    for (int q = 0; q < kTQ; ++q) {
-      if (!act_s[q]) continue;
-      int c = 0;
-      unsigned long long b = kNoBest;
-#pragma unroll
-      for (int k = 0; k < kImg; ++k) {
-        const bool fin = (alive[k] >> q) & 1u;
-        c += fin && acc[k][q] < 0;
-        const int64_t jj = j0 + 32 * k;
-        const unsigned long long bk =
-            fin ? pack_best(acc[k][q] + thr_s[q], hmap ? (int64_t)hmap[jj] : jj) : kNoBest;
-        b = bk < b ? bk : b;
-      }
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) c += __shfl_down_sync(0xffffffffu, c, d);
-      b = warp_min_u64(b);
-      if (lane == 0) {
-        if (c) atomicAdd(&rank[q0 + q], c);
-        if (b != kNoBest) atomicMin(&best[q0 + q], b);
+        for (int d = 16; d > 0; d >>= 1) pair_rows += __shfl_down_sync(0xffffffffu, pair_rows, d);
+        if (lane == 0 && pair_rows) atomicAdd(counters, pair_rows);
+        if (lane == 0 && lane_slots) atomicAdd(counters + 3, 32ull * lane_slots);
       }
     }
-    if (kCount) {
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) pair_rows += __shfl_down_sync(0xffffffffu, pair_rows, d);
-      if (lane == 0 && pair_rows) atomicAdd(counters, pair_rows);
-      if (lane == 0 && lane_slots) atomicAdd(counters + 3, 32ull * lane_slots);
-    }
-  }
   } while (kCounted && (L += gridDim.x) < blocks);
 }
 
@@ -639,9 +640,10 @@ __global__ void __launch_bounds__(256) k_sparse_needles(const int8_t *__restrict
 // is decided by the needle's first two words where it can be: both stay in registers for the band,
 // their words of the next tile are loaded (one coalesced 128-byte access per entry and 32 images, at
 // constant distances from one running address) before the current tile is summed, and where every
-// image is narrow and none is left the tile ends at one vote.  Bound by instruction issue (as fast on
-// 32 x 32 images with a quarter of the words).  16,384 sparse needles x 262,144 images of 64 x 64, whole
-// calls: 7.8 ms with early loads alone, 4.4 ms with the constant distances and the single vote (64
+// image is narrow and none is left the tile ends at one vote.  104 instructions per needle and tile; half of
+// the issue slots are used, the gathers' latency is the first stall (2,048 needles x 65,536 images), and
+// with a quarter of the words (32 x 32 images) it is as fast.  16,384 sparse needles x 262,144 images of 64 x
+// 64, whole calls: 7.8 ms with early loads alone, 4.4 ms with the constant distances and the single vote (64
 // registers, four blocks per SM; three 5.2 ms).  Groups held in shared memory instead of gathers
 // were slower (+0.8 ms), as was deciding by one word (+0.65 ms).
 // The images of a tile that the needle's first two words leave: the further entries, 32 at a time

@@ -653,11 +653,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 //               operand tiles (K-major, same swizzle), and the image's class
 //   warp 22     TMA of the needles' operand blocks [m | a] of the chunk, 2 stages
 // Shared-memory bandwidth bounds it: per chunk 48 KB arrive, 48 KB pass through the converters and the
-// MMAs read 64 KB, 1,250 cycles at 128 bytes each against 1,376 measured (0.2 ms for 90,001 images of
+// MMAs read 64 KB, 1,280 cycles at 128 bytes each against 1,376 measured (0.2 ms for 90,001 images of
 // 64 x 64 and a needle tile; their pixels alone take 0.11 ms of HBM).  Whole calls, operand rows
 // written by an encode and read by k_tc_rank against this kernel: 100 needles 715 -> 355 us, 256
 // 754 -> 554 us, 512 959 -> 916 us, 1,024 1,357 -> 1,712 us; 90,001 images of 32 x 32: 128 needles
-// 262 -> 147 us, 512 352 -> 305 us; so up to 512 needles take it.  (100 needles since then: 319 us.)
+// 262 -> 147 us, 512 352 -> 305 us; so up to 512 needles take it.  (100 needles since then: 319 us.)  Over
+// N = 8 to 128, 1 to 512 needles and 300 to 100,000 images no call is slower than with the rows in memory
+// (512 needles of 8 x 8: 48 against 51 us with 300 images, 87 against 150 us with 100,000).
 constexpr int kQN = 128;          // haystack images per tile
 constexpr int kQRaw = 3;          // pixel stages (16 KB)
 constexpr int kQOps = 2;          // operand stages (needles 32 KB, haystack 32 KB)
